@@ -582,6 +582,17 @@ iscsi_status iscsi_stats(char* json, int len) {
                     pl.issued_products, pl.grid, (int)pl.items.size(), pl.counters, J.tiles, pl.model_balance);
       out += v;
     }
+    // the residue products of the last FP64 sigma step (zeros: none): bf16 MMA flops issued, work
+    // items, CTAs, moduli
+    {
+      double flops = 0.0;
+      int items = 0, grid = 0, moduli = 0;
+      crt_stats(*ctx, flops, items, grid, moduli);
+      std::snprintf(v, sizeof(v),
+                    ", \"residues\": {\"bf16_flops\": %.17g, \"items\": %d, \"grid\": %d, \"moduli\": %d}", flops, items,
+                    grid, moduli);
+      out += v;
+    }
     // GAS restriction: subspaces (0: none) and kept determinants
     std::snprintf(v, sizeof(v), ", \"gas_subspaces\": %d, \"gas_ndet\": %lld, \"level_split\": [%d, %d]",
                   ctx->gas_nspace, ctx->gas_ndet, ctx->sp[0].nocc, ctx->sp[1].nocc);

@@ -142,8 +142,8 @@ int StreamPool::join(cudaStream_t main) {
 namespace {
 
 // both contractions of the context on the tensor cores (one combined list)
-bool both_tc(const Context& c, int prec) {
-  return c.have_ab && ab_on_tc(c, prec) && (prec == 64 ? samespin_tc_active(c) : samespin_tc32_active(c));
+bool both_tc(Context& c, int prec, int nvec) {
+  return !(prec == 64 && crt_parts(c, nvec)) && c.have_ab && ab_on_tc(c, prec) && (prec == 64 ? samespin_tc_active(c) : samespin_tc32_active(c));
 }
 
 // one phase of every context, each on a pool stream (concurrent chains);
@@ -189,9 +189,10 @@ int sigma_batch_sequence(SigmaBatch& B) {
       for (int i = 0; i < n; ++i) {
         Context& c = *B.ctxs[i];
         if (!c.have_ab || !ab_on_tc(c, B.prec)) continue;
+        if (B.prec == 64 && (crt_parts(c, B.nvec) & 1)) continue;  // through residues, below
         const OzJob* J = B.prec == 64 ? &c.oz_ab : &c.t3_ab;
         void* base = nullptr;  // the opposite-spin outputs are absolute (the context's T workspace)
-        if (both_tc(c, B.prec)) {
+        if (both_tc(c, B.prec, B.nvec)) {
           // the context's combined list: its same-spin outputs are relative to its sigma
           J = both_tc_job(c, B.prec);
           if (!J) return kErrCuda;
@@ -202,6 +203,10 @@ int sigma_batch_sequence(SigmaBatch& B) {
       }
       ISCSI_TRY(merge_jobs(B.ab, jobs, tb, B.prec, st));
       ISCSI_TRY(launch_merged(B.ab, B.prec, B.err.as<int>(), st));
+      std::vector<Context*> cr;
+      for (Context* c : B.ctxs)
+        if (B.prec == 64 && crt_parts(*c, B.nvec)) cr.push_back(c);
+      ISCSI_TRY(crt_batch_launch(B.crt, cr, B.err.as<int>(), st));
     }
     ISCSI_TRY(phase_all(B, kPhAbGemm, /*skip_tc=*/true));
   }
@@ -212,7 +217,8 @@ int sigma_batch_sequence(SigmaBatch& B) {
     for (int i = 0; i < n; ++i) {
       Context& c = *B.ctxs[i];
       const bool on = B.prec == 64 ? samespin_tc_active(c) : samespin_tc32_active(c);
-      if (!on || both_tc(c, B.prec)) continue;  // combined contexts ran above
+      if (B.prec == 64 && (crt_parts(c, B.nvec) & 2)) continue;
+      if (!on || both_tc(c, B.prec, B.nvec)) continue;  // combined contexts ran above
       jobs.push_back(B.prec == 64 ? &c.oz_ss : &c.t3_ss);
       tb.push_back(B.prec == 64 ? static_cast<void*>(B.ss[i]) : static_cast<void*>(c.s32.as<float>()));
     }

@@ -185,6 +185,8 @@ struct OzJob {
 };
 
 struct DensityPlan;     // density.cu
+struct CrtState;        // crt.cu
+struct CrtBatch;        // crt.cu: the residue products of several contexts as one launch
 
 struct ColClass {       // column level class c = level(X) + level(Y)
   int level = 0;
@@ -256,6 +258,8 @@ struct Context {
   } route[2];
   long long pl_route_key = -1, pl_route_key32 = -1;  // routing the grouped-GEMM lists were built for
   int pl_ss_tc = -1;  // same-spin routing the FP64 grouped-GEMM list was built for
+  // FP64 contractions through residue numbers (crt.cu), built at first use
+  CrtState* crt = nullptr;
   // FP32 form of the tensor-core contractions (three bf16 terms per element)
   OzJob t3_ab, t3_ss, t3_both;
   DevBuf t3_gs, t3_bs, t3_mas, t3_mbs, t3_cs;
@@ -378,6 +382,21 @@ int oz_job_add_seg(OzJob& job, const SliceArray& A, int a_row0, const int* a_exp
 int oz_job_upload(OzJob& job, cudaStream_t st);
 int oz_job_launch(Context& ctx, const OzJob& job, cudaStream_t st);
 
+// crt.cu: the FP64 contractions through residue numbers.  parts: 1 opposite
+// spin, 2 same spin (all levels); crt_parts: what the current routing sends there
+bool crt_ab_active(Context& ctx, int nvec);
+bool crt_ss_active(Context& ctx);
+int crt_parts(Context& ctx, int nvec);
+int crt_operands(Context& ctx, const double* c, int nvec, int parts);
+int crt_gemm(Context& ctx);
+int crt_fold(Context& ctx, double* sigma);  // sigma (overwritten): the parts that went through residues
+int crt_matrices_changed(Context& ctx);
+void crt_release(Context& ctx);
+// bf16 MMA flops, work items and CTAs of the last built launch (0 without one)
+void crt_stats(const Context& ctx, double& flops, int& items, int& grid, int& moduli);
+int crt_batch_launch(CrtBatch*& b, const std::vector<Context*>& ctxs, int* err, cudaStream_t st);
+void crt_batch_release(CrtBatch*& b);
+
 // density.cu: one- and two-body density matrices (Eqs. d1, d2)
 int density_run(Context& ctx, const double* bra, const double* ket, double* d1, double* d2);
 void density_release(Context& ctx);
@@ -442,6 +461,11 @@ struct SigmaBatch {
   std::vector<double*> ss;
   int nvec = 0, prec = 0;
   MergedJob ab, sst;  // the opposite-spin (or combined) jobs; the same-spin-only jobs
+  CrtBatch* crt = nullptr;  // the residue products of the contexts that use them
+  SigmaBatch() = default;
+  SigmaBatch(const SigmaBatch&) = delete;
+  SigmaBatch& operator=(const SigmaBatch&) = delete;
+  ~SigmaBatch() { crt_batch_release(crt); }
   DevBuf err;
   StreamPool pool;
 };

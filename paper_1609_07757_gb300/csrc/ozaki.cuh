@@ -183,26 +183,6 @@ constexpr uint32_t OZ_INFO_END = 1u << 9;          // no step: the CTA's work is
 // that stage as a data step and then waited for a step that never came.
 __device__ __forceinline__ uint32_t oz_info_seq(int g) { return ((uint32_t)g & 0xFFFFu) << 16; }
 
-// W x W transpose (W a power of two up to 32) within each group of W lanes:
-// lane i of a group holds row i of the group's block on entry and column i on
-// return (butterfly exchanges over lane distances W/2, ..., 1).  The epilogue
-// holds one output row per thread; after this, each store instruction writes
-// runs of W consecutive doubles instead of 32 scattered 8-byte words.
-template <int W>
-__device__ __forceinline__ void oz_lane_transpose(double (&a)[W], int lane) {
-#pragma unroll
-  for (int s = W / 2; s >= 1; s >>= 1) {
-    const bool hi = (lane & s) != 0;
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-      if (j & s) continue;
-      const double recv = __shfl_xor_sync(0xffffffffu, hi ? a[j] : a[j ^ s], s);
-      if (hi) a[j] = recv;
-      else a[j ^ s] = recv;
-    }
-  }
-}
-
 // Accumulators restart without a separate clearing pass: the MMA thread keeps
 // a mask of the levels written since their last drain, and the first MMA that
 // writes a level uses accumulate = 0 (a run of levels whose written state

@@ -84,6 +84,26 @@ __device__ __forceinline__ double oz_i64_scaled(long long q, int e) {
   return __longlong_as_double((long long)bits);
 }
 
+// W x W transpose (W a power of two up to 32) within each group of W lanes:
+// lane i of a group holds row i of the group's block on entry and column i on
+// return (butterfly exchanges over lane distances W/2, ..., 1).  The epilogue
+// holds one output row per thread; after this, each store instruction writes
+// runs of W consecutive doubles instead of 32 scattered 8-byte words.
+template <int W>
+__device__ __forceinline__ void oz_lane_transpose(double (&a)[W], int lane) {
+#pragma unroll
+  for (int s = W / 2; s >= 1; s >>= 1) {
+    const bool hi = (lane & s) != 0;
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      if (j & s) continue;
+      const double recv = __shfl_xor_sync(0xffffffffu, hi ? a[j] : a[j ^ s], s);
+      if (hi) a[j] = recv;
+      else a[j ^ s] = recv;
+    }
+  }
+}
+
 // exponent field of |x|: frexp exponent = field - 1022 for normal x (0 for zero)
 __device__ __forceinline__ int oz_exp_field(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
 

@@ -66,6 +66,7 @@ void DevBuf::release() {
 }
 
 Context::~Context() {
+  crt_release(*this);
   density_release(*this);
   if (ev0) cudaEventDestroy(ev0);
   if (ev1) cudaEventDestroy(ev1);

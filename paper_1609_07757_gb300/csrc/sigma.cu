@@ -544,6 +544,7 @@ static int build_problems(Context& ctx, int nvec, const T* G, const T* Ma, const
       int nba = (int)ctx.nb_allowed_lvl[a];
       if (rows == 0 || nba == 0) continue;
       const int routed = std::is_same<T, double>::value ? ctx.pl_ss_tc : ctx.pl_ss_tc32;
+      if (routed == 2) continue;  // every block through residues
       if (routed == 1 && samespin_block_on_tc(ctx, a, std::is_same<T, double>::value ? 64 : 32)) continue;
       long long obase = ctx.off_h[SA.level_start[a]];
       Problem<T> p;
@@ -736,12 +737,15 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
   T* ctw = ctx.ct.as<T>();
   T* ttw = ctx.tt.as<T>();
   constexpr bool f64 = std::is_same<T, double>::value;
-  const int ss_tc = (f64 ? samespin_tc_active(ctx) : samespin_tc32_active(ctx)) ? 1 : 0;
+  // FP64: the products that go through residue numbers (crt.cu)
+  const int crt = f64 ? crt_parts(ctx, nvec) : 0;
+  const bool crt_ss = (crt & 2) != 0;
+  const int ss_tc = crt_ss ? 2 : (f64 ? samespin_tc_active(ctx) : samespin_tc32_active(ctx)) ? 1 : 0;
   const bool tc_path = ab_on_tc(ctx, f64 ? 64 : 32);
   // both contractions on the tensor cores: one launch for both problem lists
   // (fewer partly filled waves); sigma starts at zero, the same-spin products
   // add into it, the fold adds last
-  const bool comb = ctx.have_ab && tc_path && ss_tc;
+  const bool comb = ctx.have_ab && tc_path && ss_tc && !crt;
   // per-phase events only when the whole step runs in this call
   const bool timed = phases == kPhAll;
   const int call = ctx.ntimed;
@@ -752,7 +756,7 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
     int& routed = f64 ? ctx.pl_ss_tc : ctx.pl_ss_tc32;
     long long& rkey = f64 ? ctx.pl_route_key : ctx.pl_route_key32;
     const Context::Route& R = ctx.route[f64 ? 0 : 1];
-    const long long key = ((long long)R.ss_min << 2) | (R.ab_tc << 1) | ss_tc;
+    const long long key = ((long long)R.ss_min << 3) | (R.ab_tc << 2) | ss_tc;
     if (routed != ss_tc || rkey != key) {
       routed = ss_tc;
       rkey = key;
@@ -764,7 +768,16 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
       pl_nvec = nvec;
     }
     ISCSI_TRY(ev(0));
-    if (ctx.have_ab && tc_path) {
+    if (crt) {
+      const int rc = crt_operands(ctx, reinterpret_cast<const double*>(c), nvec, crt);
+      // no room for the residues: the context takes the slices from here on
+      if (rc == kErrNoMem && !ctx.capturing)
+        return sigma_impl<T, TC>(ctx, c_in, s_out, c, sigma, nvec, ab, ss, pl_nvec, G, Ma, Mb, phases);
+      ISCSI_TRY(rc);
+    }
+    if (ctx.have_ab && tc_path && (crt & 1)) {
+      // operands above
+    } else if (ctx.have_ab && tc_path) {
       // opposite-spin operands for the tensor cores (lift + slice)
       if (f64)
         ISCSI_TRY(opposite_tc_operands(ctx, reinterpret_cast<const double*>(c_in), reinterpret_cast<double*>(ttw),
@@ -791,13 +804,16 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
             ctx.off.as<long long>(), c_in, ctx.ndet, ctw); ISCSI_COUNT_LAUNCH();
         ISCSI_CUDA(cudaGetLastError());
       }
-    } else {
+    } else if (!crt_ss) {
       ISCSI_CUDA(cudaMemsetAsync(sigma, 0, sizeof(T) * ctx.ndet * nvec, st));
     }
     ISCSI_TRY(ev(1));
   }
   if (phases & kPhAbGemm) {
-    if (comb)
+    // (a batch launches its contexts' residue products together)
+    if (crt && phases == kPhAll) ISCSI_TRY(crt_gemm(ctx));
+    if (crt & 1) {
+    } else if (comb)
       ISCSI_TRY(f64 ? both_tc_gemm(ctx, reinterpret_cast<double*>(sigma))
                     : both_tc32_gemm(ctx, reinterpret_cast<float*>(sigma)));
     else if (ctx.have_ab && tc_path)
@@ -807,26 +823,27 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
     ISCSI_TRY(ev(2));
   }
   if (phases & kPhMid) {
-    if (ctx.have_ab) {
+    if (crt) ISCSI_TRY(crt_fold(ctx, reinterpret_cast<double*>(sigma)));
+    if (ctx.have_ab && !(crt & 1)) {
       ClassTable ct = class_table(ctx, nvec);
       k_fold<T><<<ctx.sp[0].count, 256, 0, st>>>(ct, nvec, ctx.n, ctx.na, ctx.nb, ctx.sp[1].nhole,
                                                  ctx.sp[0].dec.as<int>(), ctx.sp[1].dec.as<int>(),
                                                  ctx.hp_class.as<int8_t>(), ctx.hp_local.as<int>(),
                                                  ctx.pair_index.as<int>(), ctx.off.as<long long>(), ttw, ctx.ndet,
-                                                 sigma, comb ? 1 : 0); ISCSI_COUNT_LAUNCH();
+                                                 sigma, comb || crt_ss ? 1 : 0); ISCSI_COUNT_LAUNCH();
       ISCSI_CUDA(cudaGetLastError());
     }
     ISCSI_TRY(ev(3));
     ISCSI_TRY(launch_grouped<T>(ss, c, sigma, st));
-    if (ss_tc && !comb && f64)
+    if (ss_tc == 1 && !comb && f64)
       ISCSI_TRY(samespin_tc_operands(ctx, reinterpret_cast<const double*>(c), reinterpret_cast<double*>(sigma), nvec));
-    else if (ss_tc && !comb)
+    else if (ss_tc == 1 && !comb)
       ISCSI_TRY(samespin_tc32_operands(ctx, reinterpret_cast<const float*>(c), reinterpret_cast<float*>(sigma), nvec));
   }
   if (phases & kPhSsGemm) {
-    if (ss_tc && !comb && f64)
+    if (ss_tc == 1 && !comb && f64)
       ISCSI_TRY(samespin_tc_gemm(ctx, reinterpret_cast<double*>(sigma)));
-    else if (ss_tc && !comb)
+    else if (ss_tc == 1 && !comb)
       ISCSI_TRY(samespin_tc32_gemm(ctx, reinterpret_cast<float*>(sigma)));
   }
   if (phases & kPhPost) {
@@ -835,6 +852,13 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
   }
   (void)s_out;
   return kOk;
+}
+
+int crt_parts(Context& ctx, int nvec) {
+  int parts = 0;
+  if (ctx.have_ab && ab_on_tc(ctx, 64) && crt_ab_active(ctx, nvec)) parts |= 1;
+  if (ctx.route[0].ss_min <= kThinN && samespin_tc_active(ctx) && crt_ss_active(ctx)) parts |= 2;
+  return parts;
 }
 
 int sigma_run(Context& ctx, const double* c, double* sigma, int nvec, int precision, int phases) {
@@ -940,6 +964,8 @@ int sigma_autotune(Context& ctx, const double* c, double* sigma, int nvec, int p
           double rows = block_rows(ctx, a), nba = (double)ctx.nb_allowed_lvl[a];
           same = (rows > q.ss && nba > q.ss) == (rows > ss && nba > ss);
         }
+        // the lowest threshold is the residue products (all blocks at once), the others slices
+        if (prec == 64 && crt_ss_active(ctx) && (q.ss == kThinN) != (ss == kThinN)) same = false;
         if (same) dup = true;
       }
       if (!dup) cands.push_back({ab, ss, route_model_ms(ctx, prec, ab, ss, nvec), -1.0});

@@ -1042,6 +1042,7 @@ int launch_tc_problems(const OzProblem* probs, int nprobs, const OzSeg* segs, co
 int samespin_matrices_changed(Context& ctx) {
   if (ctx.oz_m_ready) ISCSI_TRY(tc_prepare_m(ctx, true));
   if (ctx.t3_m_ready) ISCSI_TRY(t3_prepare_m(ctx, true));
+  ISCSI_TRY(crt_matrices_changed(ctx));
   return kOk;
 }
 

@@ -1,0 +1,100 @@
+"""GPU: the contractions through residue numbers at the edges of their tiles and runs.
+
+Reference: the FP64 FMA kernels of the same library (option fp64_tc = 0), which
+share only the tables with the residue products.  Bars as in test_gpu_sigma
+(1e-12 of the 2-norm and of the largest element): both routes round at about
+1e-15 of the unit-weighted sums, whatever the sums' cancellation leaves of the
+bar's three digits.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1609_07757_gb300 import _lib as L
+from paper_1609_07757_gb300.synthetic import make_integrals, unit_vector
+
+pytestmark = pytest.mark.gpu
+
+REL64 = 1e-12
+
+
+@pytest.fixture(autouse=True)
+def _fresh_library():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    L.load()
+    L.iscsi_set_option("autotune", 0)
+    L.iscsi_set_stream(torch.cuda.current_stream())
+    yield
+    torch.cuda.synchronize()
+    L.iscsi_finalize()
+    L.iscsi_set_option("fp64_tc", 1)
+    L.iscsi_set_option("autotune", 1)
+
+
+def sigma(C, nvec):
+    c = torch.as_tensor(np.ascontiguousarray(C), dtype=torch.float64, device="cuda")
+    s = torch.full_like(c, float("nan"))
+    L.iscsi_sigma(c, s, nvec)
+    torch.cuda.synchronize()
+    return s.cpu().numpy()
+
+
+def both(C, nvec):
+    """sigma through residues (twice, bit for bit the same) and on the FMA kernels."""
+    s = sigma(C, nvec)
+    assert L.iscsi_stats()["residues"]["items"] > 0
+    assert np.array_equal(s, sigma(C, nvec))
+    L.iscsi_set_option("fp64_tc", 0)
+    ref = sigma(C, nvec)
+    L.iscsi_set_option("fp64_tc", 1)
+    return s, ref
+
+
+def check(s, ref):
+    d = s - ref
+    assert np.linalg.norm(d) <= REL64 * np.linalg.norm(ref)
+    assert np.abs(d).max() <= REL64 * np.abs(ref).max()
+
+
+# strings around 16, 64, 128 and 256 (tiles of C and M), pairs around 64 and 256 (K blocks and row
+# tiles), one to five beta electrons (unrolled and general folds), unequal spins, runs of levels
+SHAPES = [
+    (7, 2, 2, 4), (11, 2, 2, 4), (12, 2, 2, 4), (16, 2, 2, 4), (17, 2, 2, 4), (23, 2, 2, 4), (24, 2, 2, 4),
+    (20, 1, 1, 2), (12, 3, 3, 6), (9, 4, 4, 8), (11, 2, 5, 7), (11, 5, 2, 7), (13, 3, 1, 4),
+    (17, 2, 2, 3), (24, 2, 2, 3), (12, 3, 3, 3), (12, 3, 3, 4), (10, 3, 4, 5),
+]
+
+
+@pytest.mark.parametrize("n,na,nb,kmax", SHAPES)
+@pytest.mark.parametrize("nvec", [1, 3])
+def test_residues_match_fma(n, na, nb, kmax, nvec):
+    h1, eri = make_integrals(n, 7000 + n, ell=4.0, nchol=12)
+    L.iscsi_init(n, na, nb, kmax, h1, eri, 1e-14)
+    nd = L.iscsi_ndet()
+    # vectors of different sizes: each has its own scale
+    C = np.stack([unit_vector(nd, 10 + v) * 10.0 ** (3 * v) for v in range(nvec)])
+    s, ref = both(C, nvec)
+    for v in range(nvec):
+        check(s[v], ref[v])
+
+
+@pytest.mark.parametrize("what", ["constant", "graded", "single", "zero"])
+def test_residues_extreme_vectors(what):
+    # constant integrals and vector: every product of a chunk has the same sign and residues (the
+    # largest sums); eight decades of magnitudes; one determinant; nothing
+    n = 18
+    h1, eri = make_integrals(n, 7100, ell=4.0, nchol=12)
+    if what == "constant":
+        h1, eri = np.ones_like(h1), np.ones_like(eri)
+    L.iscsi_init(n, 2, 2, 4, h1, eri, 0.0)
+    nd = L.iscsi_ndet()
+    rng = np.random.default_rng(5)
+    c = {"constant": np.full(nd, 1.0 / 3.0), "graded": rng.normal(size=nd) * 10.0 ** (-8 * rng.random(nd)),
+         "single": np.eye(1, nd, nd // 3)[0], "zero": np.zeros(nd)}[what]
+    s, ref = both(c[None], 1)
+    if what == "zero":
+        assert not s.any()
+    else:
+        check(s, ref)
