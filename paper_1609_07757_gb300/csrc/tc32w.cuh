@@ -11,8 +11,11 @@
 // accumulators: order 0 (A_0 B_0) has its own 128 columns, orders 1 and 2
 // (five pairs, each at most 2^-8 of order 0) sum into a second 128; a buffer
 // is 256 columns, buffer b at 256 b, and the MMAs of chunk c + 1 run while
-// the epilogue drains chunk c.  Per K step: one MMA of N = 128 into the
-// order-0 columns and five into the others.
+// the epilogue drains chunk c.  Per K step five MMAs: A_0 (B_0, B_1) as one of
+// N = 256 over the order-0 columns and the others', then the four remaining
+// pairs (N = 128).  The MMA warp runs its loop whole and one elected lane
+// issues: full CI n = 60, one sigma 1058 -> 1004 us against a single-lane branch
+// with six MMAs, the same results bit for bit.
 //
 // Warp 0 loads (TMA; A and B in 128-row boxes), warp 1 issues the MMAs, warps 2-9 drain
 // (two per TMEM lane quarter, 64 columns each).  Problems, segments and
@@ -145,34 +148,44 @@ __global__ void __launch_bounds__(T3W_THREADS, 1)
         tc::mbar_wait_bounded(tc::smem_u32(&full_b[g % T3W_STAGES]), (g / T3W_STAGES) & 1, OZ_SPIN);
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t N128 = tc::idesc_bf16_f32(T3_BM, T3W_BN);
-      for (int g = 0; g < total; ++g) {
-        const int st = g % T3W_STAGES;
-        const int ch = g / SPC, kin = g % SPC, b = ch & 1;
-        if (kin == 0 && ch >= 2 && !wait(&free_b[b], ((ch >> 1) - 1) & 1, OZ_SITE_FREE, ch)) break;
-        if (!wait(&full_b[st], (g / T3W_STAGES) & 1, OZ_SITE_FULL, g)) break;
-        tc::fence_after_sync();
-        const uint32_t sa = s_stage0 + st * T3W_STAGE_BYTES;
-        const uint32_t sb = sa + T3_S * T3_A_SLICE_BYTES;
-        auto A = [&](int t) { return tc::smem_desc_sw32(sa + t * T3_A_SLICE_BYTES); };
-        auto B = [&](int u) { return tc::smem_desc_sw32(sb + u * T3W_B_SLICE_BYTES); };
+    // ---------------- MMA issuer: the whole warp runs the loop, one elected lane issues
+    // (in a branch of a single lane the compiler moves the MMAs' operands through per-thread
+    // registers, and the tensor core runs dry between them)
+    constexpr uint32_t N128 = tc::idesc_bf16_f32(T3_BM, T3W_BN), N256 = tc::idesc_bf16_f32(T3_BM, 2 * T3W_BN);
+    const uint64_t dA0 = tc::smem_desc_sw32(s_stage0), dB0 = tc::smem_desc_sw32(s_stage0 + T3_S * T3_A_SLICE_BYTES);
+    constexpr uint64_t kSt = T3W_STAGE_BYTES >> 4, kA = T3_A_SLICE_BYTES >> 4, kB = T3W_B_SLICE_BYTES >> 4;
+    bool ok = true;
+    int st = 0;
+    uint32_t ph = 0;
+    for (int g = 0; g < total; ++g) {
+      const int ch = g / SPC, kin = g % SPC, b = ch & 1;
+      if (kin == 0 && ch >= 2) ok = wait(&free_b[b], ((ch >> 1) - 1) & 1, OZ_SITE_FREE, ch);
+      ok = ok && wait(&full_b[st], ph, OZ_SITE_FULL, g);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+        const uint64_t A = dA0 + kSt * st, B = dB0 + kSt * st;
         const uint32_t D0 = tmem + (uint32_t)(b * T3W_BUF_COLS), D1 = D0 + T3W_BN;
         const uint32_t first = kin == 0 ? 0u : 1u;  // the first step of a chunk restarts the buffer
-        tc::mma_bf16(D0, A(0), B(0), N128, first);
-        tc::mma_bf16(D1, A(0), B(1), N128, first);
-        tc::mma_bf16(D1, A(1), B(0), N128, 1u);
-        tc::mma_bf16(D1, A(0), B(2), N128, 1u);
-        tc::mma_bf16(D1, A(1), B(1), N128, 1u);
-        tc::mma_bf16(D1, A(2), B(0), N128, 1u);
+        // A_0 (B_0, B_1): order 0 and the first of orders 1-2 lie side by side, as B's slices do
+        tc::mma_bf16(D0, A, B, N256, first);
+        tc::mma_bf16(D1, A + kA, B, N128, 1u);           // A_1 B_0
+        tc::mma_bf16(D1, A, B + 2 * kB, N128, 1u);       // A_0 B_2
+        tc::mma_bf16(D1, A + kA, B + kB, N128, 1u);      // A_1 B_1
+        tc::mma_bf16(D1, A + 2 * kA, B, N128, 1u);       // A_2 B_0
         tc::mma_commit(tc::smem_u32(&empty_b[st]));
         if (kin == SPC - 1 || g == total - 1) tc::mma_commit(tc::smem_u32(&chunk_b[b]));
       }
-      if (abort_s) {
-        tc::mma_commit(tc::smem_u32(&drain_b));
-        tc::mbar_wait_bounded(tc::smem_u32(&drain_b), 0, OZ_SPIN);
+      __syncwarp();
+      if (++st == T3W_STAGES) {
+        st = 0;
+        ph ^= 1u;
       }
+    }
+    if (abort_s) {
+      if (tc::elect_one()) tc::mma_commit(tc::smem_u32(&drain_b));
+      __syncwarp();
+      tc::mbar_wait_bounded(tc::smem_u32(&drain_b), 0, OZ_SPIN);
     }
   } else {
     // ---------------- epilogue: warps 2-9; lane quarter = warp % 4, column half = (warp - 2) / 4
