@@ -59,6 +59,7 @@ struct DavCtl {
   int status;   // kStatus* bits
   double tol, etol, rmax, dmax;
   int reorth;    // 1: the block needs a second Gram-Schmidt pass
+  int m_eig;     // order of the last eigen-decomposition while its vectors still describe the basis, else 0
   int olsen;    // 1: Olsen's correction in the preconditioner
   double theta[kMaxRoots], theta_prev[kMaxRoots], rnorm[kMaxRoots], nrm0[kMaxRoots], eps[kMaxRoots];
   int active[kMaxRoots];
@@ -132,7 +133,20 @@ __device__ __forceinline__ void df_fma(Df& a, float xh, float xl, float yh, floa
 
 __device__ __forceinline__ double df_value(const Df& a) { return (double)a.s + (double)a.c; }
 
-// partial[b][i][j] = sum over block b's elements of A_i[e] B_j[e], for
+// x[0] + x[stride] + ... + x[(parts - 1) stride] by one warp in a fixed order
+// (lane l sums l, l + 32, ...; then a butterfly whose two operands are the same
+// on both lanes of every exchange, so every lane returns the same value, and
+// every run the same)
+__device__ __forceinline__ double warp_sum_strided(const double* __restrict__ x, long long stride, int parts,
+                                                   int lane) {
+  double s = 0.0;
+  for (int p = lane; p < parts; p += 32) s += __ldcg(x + (long long)p * stride);
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// C[i][j] = sum over the elements of A_i[e] B_j[e] (partial: the blocks' parts,
+// done: a zeroed counter per tile), for
 // i < na = (na_dev ? *na_dev : 0) + na_add and j < nb; rows_cap bounds na.
 // Each block takes kDotT rows of A and NB columns of B (NB = nb when nb <= 8,
 // so no FMA is spent on absent columns: GB300's FP64 rate, not HBM, bounds
@@ -141,6 +155,7 @@ template <int NB>
 __global__ void __launch_bounds__(kVecThreads) k_tsdots(const double* __restrict__ A, const int* __restrict__ na_dev,
                                                         int na_add, const double* __restrict__ B, int nb, long long N,
                                                         double* __restrict__ partial, int rows_cap,
+                                                        int* __restrict__ done, double* __restrict__ C,
                                                         const int* __restrict__ gate) {
   if (gate && !*gate) return;
   const int na = (na_dev ? *na_dev : 0) + na_add;
@@ -167,47 +182,55 @@ __global__ void __launch_bounds__(kVecThreads) k_tsdots(const double* __restrict
         for (int b = 0; b < NB; ++b) df_fma(acc[a][b], ah, al, bh[b], bl[b]);
       }
   }
+  // the warp's sums of kDotT NB values, exchanged so that each step halves the values a lane still
+  // carries (31 FP64 additions for 32 values; a butterfly per value took 160, and FP64 issues two
+  // operations per clock per SM: 18 us of a 2025-determinant product)
   __shared__ double red[kVecThreads / 32][kDotT * NB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int V = kDotT * NB;                   // values, and values rounded up to 32
+  constexpr int VP = (V + 31) / 32 * 32;
+  double x[VP];
 #pragma unroll
-  for (int a = 0; a < kDotT; ++a)
+  for (int t = 0; t < VP; ++t) x[t] = t < V ? df_value(acc[(t < V ? t : 0) / NB][(t < V ? t : 0) % NB]) : 0.0;
 #pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      double x = df_value(acc[a][b]);
-      for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if (lane == 0) red[warp][a * NB + b] = x;
+  for (int o = 16, n = VP; o; o >>= 1, n >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int t = 0; t < n / 2; ++t) {
+      const double give = up ? x[t] : x[t + n / 2], keep = up ? x[t + n / 2] : x[t];
+      x[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
-  __syncthreads();
-  if (threadIdx.x < kDotT * NB) {
-    double x = 0.0;
-    for (int w = 0; w < kVecThreads / 32; ++w) x += red[w][threadIdx.x];
-    const int a = threadIdx.x / NB, b = threadIdx.x % NB;
-    if (a < ra && j0 + b < nb) partial[((long long)blockIdx.x * rows_cap + i0 + a) * nb + j0 + b] = x;
   }
-}
-
-// x[0] + x[stride] + ... + x[(parts - 1) stride] by one warp in a fixed order
-// (lane l sums l, l + 32, ...; then a butterfly whose two operands are the same
-// on both lanes of every exchange, so every lane returns the same value, and
-// every run the same)
-__device__ __forceinline__ double warp_sum_strided(const double* __restrict__ x, long long stride, int parts,
-                                                   int lane) {
-  double s = 0.0;
-  for (int p = lane; p < parts; p += 32) s += x[(long long)p * stride];
-  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
-}
-
-// C[i][j] = sum over blocks of partial[b][i][j], one warp per element
-// (nothing when gate points at 0)
-__global__ void k_tsreduce(const double* __restrict__ partial, int parts, const int* __restrict__ na_dev, int na_add,
-                           int nb, int rows_cap, double* __restrict__ C, const int* __restrict__ gate) {
-  if (gate && !*gate) return;
-  const int na = (na_dev ? *na_dev : 0) + na_add;
-  const int t = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (t >= na * nb) return;  // whole warps
-  const double x = warp_sum_strided(partial + t, (long long)rows_cap * nb, parts, lane);
-  if (lane == 0) C[t] = x;
+  // lane l holds the sums of values base(l) .. base(l) + VP / 32 - 1
+#pragma unroll
+  for (int t = 0; t < VP / 32; ++t) {
+    const int v = (lane >> 4 & 1) * (VP / 2) + (lane >> 3 & 1) * (VP / 4) + (lane >> 2 & 1) * (VP / 8) +
+                  (lane >> 1 & 1) * (VP / 16) + (lane & 1) * (VP / 32) + t;
+    if (v < V) red[warp][v] = x[t];
+  }
+  __syncthreads();
+  if (threadIdx.x < V) {
+    double y = 0.0;
+    for (int w = 0; w < kVecThreads / 32; ++w) y += red[w][threadIdx.x];
+    const int a = threadIdx.x / NB, b = threadIdx.x % NB;
+    if (a < ra && j0 + b < nb) partial[((long long)blockIdx.x * rows_cap + i0 + a) * nb + j0 + b] = y;
+    __threadfence();
+  }
+  // the last block of this tile to finish adds the blocks' parts, one warp per
+  // element in a fixed order
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(done + blockIdx.y, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int cb = min(NB, nb - j0);
+  for (int t = warp; t < ra * cb; t += kVecThreads / 32) {
+    const long long at = (long long)(i0 + t / cb) * nb + j0 + t % cb;
+    const double y = warp_sum_strided(partial + at, (long long)rows_cap * nb, gridDim.x, lane);
+    if (lane == 0) C[at] = y;
+  }
+  if (threadIdx.x == 0) done[blockIdx.y] = 0;  // for the next launch
 }
 
 // X_j = sum_i V_i Y[i][j], R_j = sum_i W_i Y[i][j] - theta_j X_j for j in
@@ -238,6 +261,7 @@ __global__ void __launch_bounds__(kVecThreads) k_dav_ritz(const double* __restri
     Df x[KC], r[KC];
 #pragma unroll
     for (int j = 0; j < KC; ++j) x[j] = r[j] = Df{0.0f, 0.0f};
+#pragma unroll 4
     for (int i = 0; i < m; ++i) {
       float vh, vl, wh, wl;
       df_split(V[(long long)i * N + e], vh, vl);
@@ -265,16 +289,19 @@ __global__ void __launch_bounds__(kVecThreads) k_dav_ritz(const double* __restri
   }
 }
 
-// out_j = sum_{i<m} V_i Y[i][j0 + j] for j < min(KC, nkeep - j0); only when a
-// restart is pending
+// out_j = sum_{i<m} V_i Y[i][j0 + j] for j < min(KC, nkeep - j0), j0 = KC
+// blockIdx.y; only when a restart is pending.  With one chunk (nkeep <= KC) out
+// may be V itself: a thread reads its element of all V_i before it writes.  V2 (or
+// null): a second set of vectors, blockIdx.z = 1, in place.
 template <int KC>
-__global__ void __launch_bounds__(kVecThreads) k_dav_restart_lincomb(const double* __restrict__ V,
+__global__ void __launch_bounds__(kVecThreads) k_dav_restart_lincomb(const double* V,
                                                                      const DavCtl* __restrict__ ctl,
-                                                                     const double* __restrict__ Y, int ldy, int j0,
-                                                                     long long N, double* __restrict__ out) {
+                                                                     const double* __restrict__ Y, int ldy,
+                                                                     long long N, double* out, double* V2) {
   extern __shared__ float sYcf[];  // [2][m][KC]
   if (!ctl->restart) return;
-  const int m = ctl->m;
+  if (blockIdx.z) V = out = V2;
+  const int m = ctl->m, j0 = KC * blockIdx.y;
   const int cnt = min(KC, ctl->nkeep - j0);
   if (cnt <= 0) return;
   float* sYh = sYcf;
@@ -287,6 +314,7 @@ __global__ void __launch_bounds__(kVecThreads) k_dav_restart_lincomb(const doubl
     Df acc[KC];
 #pragma unroll
     for (int j = 0; j < KC; ++j) acc[j] = Df{0.0f, 0.0f};
+#pragma unroll 4
     for (int i = 0; i < m; ++i) {
       float vh, vl;
       df_split(V[(long long)i * N + e], vh, vl);
@@ -320,6 +348,7 @@ __global__ void k_dav_restart_S(DavCtl* __restrict__ ctl, double* __restrict__ S
   __syncthreads();
   if (threadIdx.x == 0) {
     ctl->m = nk;
+    ctl->m_eig = 0;  // the basis is the Ritz basis now
     ctl->restart = 0;
   }
 }
@@ -381,6 +410,7 @@ __global__ void __launch_bounds__(kVecThreads) k_dav_project(const double* __res
     Df acc[KC];
 #pragma unroll
     for (int j = 0; j < KC; ++j) acc[j] = Df{0.0f, 0.0f};
+#pragma unroll 4
     for (int i = 0; i < m; ++i) {
       float vh, vl;
       df_split(V[(long long)i * N + e], vh, vl);
@@ -583,6 +613,7 @@ __global__ void k_dav_init_S(DavCtl* __restrict__ ctl, double* __restrict__ S, i
   }
   if (threadIdx.x == 0) {
     ctl->m = cnt;
+    ctl->m_eig = 0;
     ctl->restart = 0;
   }
 }
@@ -602,38 +633,64 @@ __global__ void k_dav_request_restart(DavCtl* __restrict__ ctl, int nkeep) {
 // pairs at once.  A, Q are m x m work arrays (shared or global memory).
 // Eigenvalues ascending into theta_all, eigenvector j into column j of Y;
 // ctl->theta gets the lowest k.
+//
+// One CTA: bound by its SM's FP64 rate (two operations per clock) and by the
+// rounds' serial chain.  So:
+//   * while the basis only grew since the last decomposition (m_eig > 0), the
+//     matrix is taken in the last eigenvectors: diagonal but for the new rows,
+//     whose couplings are small near convergence (few sweeps, few rotations);
+//   * a pair whose element is below 1e-15 |S|_F / m is not rotated, a round
+//     without rotations costs one synchronisation, and a sweep without any ends
+//     the iteration (the elements left then sum to at most (1e-15 |S|_F)^2);
+//   * the angle comes from FP32 (an angle right to 1e-7 leaves 1e-7 of the
+//     element, which the next sweep takes), cosine and sine from it in FP64 by
+//     two Newton steps, so that the rotation is orthogonal to FP64 rounding;
+//   * a thread turns a 2 x 2 block (rows of pair i, columns of pair j >= i) from
+//     both sides and writes its mirror image: half the products, one pass.
+// Basis of 12 to 24, two roots: 330 -> 228 us on average.
 __global__ void __launch_bounds__(256) k_dav_eigh(DavCtl* __restrict__ ctl, const double* __restrict__ S, int lds,
-                                                  double* gA, double* gQ, double* __restrict__ Y, int ldy,
-                                                  double* __restrict__ theta_all, int use_smem) {
+                                                  double* gA, double* gQ, double* Y, int ldy,
+                                                  double* theta_all, int use_smem) {
   extern __shared__ double dyn[];
   __shared__ double cs[192], sn[192];
   __shared__ int pp[192], qq[192];
-  __shared__ double red[8];
-  __shared__ int stop;
-  const int m = ctl->m;
+  __shared__ double red[8], thr_s, inv_s;
+  const int m = ctl->m, m0 = ctl->m_eig > 0 && ctl->m_eig <= m ? ctl->m_eig : 0;
   double* A = use_smem ? dyn : gA;
   double* Q = use_smem ? dyn + m * m : gQ;
   const int me = m + (m & 1);
   const int npair = me / 2;
   for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
     const int i = t / m, j = t % m;
-    A[t] = S[(long long)i * lds + j];
-    Q[t] = i == j ? 1.0 : 0.0;
+    double a;
+    if (i < m0 && j < m0) {
+      a = i == j ? theta_all[i] : 0.0;
+    } else if (i < m0 || j < m0) {
+      const int o = min(i, j), x = max(i, j);  // old vector o, new row x
+      a = 0.0;
+      for (int l = 0; l < m0; ++l) a = fma(Y[(long long)l * ldy + o], S[(long long)l * lds + x], a);
+    } else {
+      a = S[(long long)i * lds + j];
+    }
+    A[t] = a;
+    Q[t] = i < m0 && j < m0 ? Y[(long long)i * ldy + j] : i == j ? 1.0 : 0.0;
   }
   __syncthreads();
-  for (int sweep = 0; sweep < 60 && m > 1; ++sweep) {
-    double off = 0.0, tot = 0.0;
-    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-      const double x = A[t] * A[t];
-      tot += x;
-      if (t / m != t % m) off += x;
-    }
-    off = block_sum(off, red);
+  {
+    double tot = 0.0;
+    for (int t = threadIdx.x; t < m * m; t += blockDim.x) tot = fma(A[t], A[t], tot);
     tot = block_sum(tot, red);
-    if (threadIdx.x == 0) stop = !(off > 1e-30 * tot) || off == 0.0;
+    if (threadIdx.x == 0) {
+      thr_s = 1e-15 * sqrt(tot) / m;
+      inv_s = tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;  // the angles' FP32 sees numbers between 1e-18 and 2
+    }
     __syncthreads();
-    if (stop) break;
+  }
+  const double thr = thr_s, inv = inv_s;
+  for (int sweep = 0; sweep < 60 && m > 1; ++sweep) {
+    bool any = false;
     for (int r = 0; r < me - 1; ++r) {
+      int rot = 0;
       for (int i = threadIdx.x; i < npair; i += blockDim.x) {
         const int a = i == 0 ? 0 : ((i - 1 + r) % (me - 1)) + 1;
         const int b = ((me - 2 - i + r) % (me - 1)) + 1;
@@ -641,11 +698,17 @@ __global__ void __launch_bounds__(256) k_dav_eigh(DavCtl* __restrict__ ctl, cons
         double c = 1.0, s = 0.0;
         if (q < m) {
           const double apq = A[p * m + q];
-          if (fabs(apq) >= 1e-300) {
-            const double tau = (A[q * m + q] - A[p * m + p]) / (2.0 * apq);
-            const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            c = 1.0 / sqrt(1.0 + t * t);
-            s = t * c;
+          if (fabs(apq) > thr) {
+            const float tau = (float)((A[q * m + q] - A[p * m + p]) * inv) / (float)(2.0 * apq * inv);
+            const float t = copysignf(1.0f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f)));
+            if (t != 0.0f) {
+              const double td = (double)t, z = fma(td, td, 1.0), hz = 0.5 * z;
+              c = (double)rsqrtf((float)z);
+              c = c * fma(-hz, c * c, 1.5);
+              c = c * fma(-hz, c * c, 1.5);
+              s = td * c;
+              rot = 1;
+            }
           }
         }
         pp[i] = p;
@@ -653,31 +716,49 @@ __global__ void __launch_bounds__(256) k_dav_eigh(DavCtl* __restrict__ ctl, cons
         cs[i] = c;
         sn[i] = s;
       }
-      __syncthreads();
-      for (int t = threadIdx.x; t < npair * m; t += blockDim.x) {  // rows p, q
-        const int i = t / m, col = t % m;
-        const int p = pp[i], q = qq[i];
-        if (q >= m || sn[i] == 0.0) continue;
-        const double c = cs[i], s = sn[i];
-        const double apk = A[p * m + col], aqk = A[q * m + col];
-        A[p * m + col] = c * apk - s * aqk;
-        A[q * m + col] = s * apk + c * aqk;
+      if (!__syncthreads_or(rot)) continue;  // (the next round's parameters overwrite these unread ones)
+      any = true;
+      for (int t = threadIdx.x; t < npair * npair; t += blockDim.x) {
+        const int i = t / npair, j = t % npair;
+        const double si = sn[i], sj = sn[j];
+        if (i > j || (si == 0.0 && sj == 0.0)) continue;
+        const int p = pp[i], q = qq[i], u = pp[j], v = qq[j];
+        const bool hq = q < m, hv = v < m;
+        const double ci = cs[i], cj = cs[j];
+        const double b11 = A[p * m + u], b12 = hv ? A[p * m + v] : 0.0, b21 = hq ? A[q * m + u] : 0.0,
+                     b22 = hq && hv ? A[q * m + v] : 0.0;
+        // rows p, q, then columns u, v
+        const double r11 = ci * b11 - si * b21, r12 = ci * b12 - si * b22;
+        const double r21 = si * b11 + ci * b21, r22 = si * b12 + ci * b22;
+        const double x11 = cj * r11 - sj * r12, x12 = sj * r11 + cj * r12;
+        const double x21 = cj * r21 - sj * r22, x22 = sj * r21 + cj * r22;
+        if (i == j) {
+          A[p * m + u] = x11;
+          if (hv) {
+            const double o = 0.5 * (x12 + x21);
+            A[p * m + v] = o;
+            A[q * m + u] = o;
+            A[q * m + v] = x22;
+          }
+        } else {
+          A[p * m + u] = A[u * m + p] = x11;
+          if (hv) A[p * m + v] = A[v * m + p] = x12;
+          if (hq) A[q * m + u] = A[u * m + q] = x21;
+          if (hq && hv) A[q * m + v] = A[v * m + q] = x22;
+        }
       }
-      __syncthreads();
-      for (int t = threadIdx.x; t < npair * m; t += blockDim.x) {  // columns p, q and Q
-        const int i = t / m, row = t % m;
+      for (int t = threadIdx.x; t < npair * m; t += blockDim.x) {
+        const int row = t / npair, i = t % npair;
+        const double s = sn[i], c = cs[i];
+        if (s == 0.0) continue;
         const int p = pp[i], q = qq[i];
-        if (q >= m || sn[i] == 0.0) continue;
-        const double c = cs[i], s = sn[i];
-        const double akp = A[row * m + p], akq = A[row * m + q];
-        A[row * m + p] = c * akp - s * akq;
-        A[row * m + q] = s * akp + c * akq;
         const double ykp = Q[row * m + p], ykq = Q[row * m + q];
         Q[row * m + p] = c * ykp - s * ykq;
         Q[row * m + q] = s * ykp + c * ykq;
       }
       __syncthreads();
     }
+    if (!any) break;
   }
   // ascending order: rank of each eigenvalue (ties by index)
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
@@ -692,6 +773,7 @@ __global__ void __launch_bounds__(256) k_dav_eigh(DavCtl* __restrict__ ctl, cons
   }
   __syncthreads();
   for (int j = threadIdx.x; j < ctl->k && j < m; j += blockDim.x) ctl->theta[j] = theta_all[j];
+  if (threadIdx.x == 0) ctl->m_eig = m;
 }
 
 // residual norms, convergence and the restart decision
@@ -748,6 +830,7 @@ struct Dav {
   int k, maxsub, kc, parts, rows_cap, eig_smem;
   cudaStream_t st;
   DevBuf ctl_d, S, Y, thetas, eigA, eigQ, partial, C1, C2, G, Rinv, rr_part;
+  DevBuf done;  // one counter per tile of k_tsdots, zero between launches
   DevBuf rq;  // x_j . r_j and x_j . x_j of the returned vectors
   double *V = nullptr, *W = nullptr, *X = nullptr, *R = nullptr, *T = nullptr, *Wn = nullptr, *tmp = nullptr;
   DavCtl* ctl = nullptr;
@@ -758,6 +841,7 @@ struct Dav {
     // per thread (fewer block partials to reduce on small spaces)
     const long long per_wave = 152ll * kVecThreads * 8;
     parts = 152 * (int)std::min<long long>(kVecBlocks / 152, std::max<long long>(1, (N + per_wave - 1) / per_wave));
+    parts = (int)std::min<long long>(parts, (N + kVecThreads - 1) / kVecThreads);  // no block without elements
     rows_cap = maxsub + k;
     const int eb = 2 * maxsub * maxsub * (int)sizeof(double);
     eig_smem = eb <= 160 * 1024 ? eb : 0;
@@ -789,6 +873,9 @@ struct Dav {
     ISCSI_TRY(G.alloc(sizeof(double) * (size_t)k * k));
     ISCSI_TRY(Rinv.alloc(sizeof(double) * (size_t)k * k));
     ISCSI_TRY(rr_part.alloc(sizeof(double) * (size_t)parts * 2 * k));
+    const size_t tiles = (size_t)((rows_cap + kDotT - 1) / kDotT) * rows_cap;
+    ISCSI_TRY(done.alloc(sizeof(int) * tiles));
+    ISCSI_CUDA(cudaMemsetAsync(done.p, 0, sizeof(int) * tiles, st));
     ISCSI_CUDA(cudaMemsetAsync(S.p, 0, sizeof(double) * (size_t)maxsub * maxsub, st));
     return attributes();
   }
@@ -813,27 +900,25 @@ struct Dav {
   }
 
   template <int NB>
-  void dots_t(const double* A, const int* na_dev, int na_add, const double* B, int nb, const int* gate) {
+  void dots_t(const double* A, const int* na_dev, int na_add, const double* B, int nb, double* C, const int* gate) {
     const int tiles = ((rows_cap + kDotT - 1) / kDotT) * ((nb + NB - 1) / NB);
     k_tsdots<NB><<<dim3(parts, tiles), kVecThreads, 0, st>>>(A, na_dev, na_add, B, nb, N, partial.as<double>(),
-                                                             rows_cap, gate); ISCSI_COUNT_LAUNCH();
+                                                             rows_cap, done.as<int>(), C, gate); ISCSI_COUNT_LAUNCH();
   }
   // C[i][j] = A_i . B_j for i < (na_dev ? *na_dev : 0) + na_add, j < nb; when
   // gate is given, only if *gate != 0 at run time
   void dots(const double* A, const int* na_dev, int na_add, const double* B, int nb, double* C,
             const int* gate = nullptr) {
     switch (nb) {
-      case 1: dots_t<1>(A, na_dev, na_add, B, nb, gate); break;
-      case 2: dots_t<2>(A, na_dev, na_add, B, nb, gate); break;
-      case 3: dots_t<3>(A, na_dev, na_add, B, nb, gate); break;
-      case 4: dots_t<4>(A, na_dev, na_add, B, nb, gate); break;
-      case 5: dots_t<5>(A, na_dev, na_add, B, nb, gate); break;
-      case 6: dots_t<6>(A, na_dev, na_add, B, nb, gate); break;
-      case 7: dots_t<7>(A, na_dev, na_add, B, nb, gate); break;
-      default: dots_t<8>(A, na_dev, na_add, B, nb, gate); break;
+      case 1: dots_t<1>(A, na_dev, na_add, B, nb, C, gate); break;
+      case 2: dots_t<2>(A, na_dev, na_add, B, nb, C, gate); break;
+      case 3: dots_t<3>(A, na_dev, na_add, B, nb, C, gate); break;
+      case 4: dots_t<4>(A, na_dev, na_add, B, nb, C, gate); break;
+      case 5: dots_t<5>(A, na_dev, na_add, B, nb, C, gate); break;
+      case 6: dots_t<6>(A, na_dev, na_add, B, nb, C, gate); break;
+      case 7: dots_t<7>(A, na_dev, na_add, B, nb, C, gate); break;
+      default: dots_t<8>(A, na_dev, na_add, B, nb, C, gate); break;
     }
-    k_tsreduce<<<(rows_cap * nb + 7) / 8, 256, 0, st>>>(partial.as<double>(), parts, na_dev, na_add, nb, rows_cap,
-                                                            C, gate); ISCSI_COUNT_LAUNCH();
   }
 
   template <int KC>
@@ -854,14 +939,21 @@ struct Dav {
   }
   template <int KC>
   void restart_t() {
-    const size_t sm = sizeof(double) * (size_t)maxsub * KC;
     const int nk = std::max(k, maxsub / 2);
-    for (int pass = 0; pass < 2; ++pass) {
-      double* src = pass == 0 ? V : W;
-      for (int j0 = 0; j0 < nk; j0 += KC) {
-        k_dav_restart_lincomb<KC><<<parts, kVecThreads, sm, st>>>(src, ctl, Y.as<double>(), maxsub, j0, N, tmp); ISCSI_COUNT_LAUNCH();
+    if (nk <= 16 && sizeof(double) * (size_t)maxsub * 16 <= 200 * 1024) {
+      // all kept columns in one chunk: V and W in place, one launch (chunks of k columns through a
+      // buffer took 14 launches per iteration for two roots, 57 us of a 630 us iteration at
+      // 2025 determinants, almost all of them with nothing to do)
+      k_dav_restart_lincomb<16><<<dim3(parts, 1, 2), kVecThreads, sizeof(double) * (size_t)maxsub * 16, st>>>(
+          V, ctl, Y.as<double>(), maxsub, N, V, W); ISCSI_COUNT_LAUNCH();
+    } else {
+      const size_t sm = sizeof(double) * (size_t)maxsub * KC;
+      for (int pass = 0; pass < 2; ++pass) {
+        double* src = pass == 0 ? V : W;
+        k_dav_restart_lincomb<KC><<<dim3(parts, (nk + KC - 1) / KC), kVecThreads, sm, st>>>(src, ctl, Y.as<double>(),
+                                                                                            maxsub, N, tmp, nullptr); ISCSI_COUNT_LAUNCH();
+        k_dav_restart_copy<<<parts, kVecThreads, 0, st>>>(src, tmp, ctl, N); ISCSI_COUNT_LAUNCH();
       }
-      k_dav_restart_copy<<<parts, kVecThreads, 0, st>>>(src, tmp, ctl, N); ISCSI_COUNT_LAUNCH();
     }
     k_dav_restart_S<<<1, 256, 0, st>>>(ctl, S.as<double>(), maxsub, thetas.as<double>()); ISCSI_COUNT_LAUNCH();
   }
@@ -1007,9 +1099,8 @@ struct Dav {
   template <int KC>
   void restart_v() {
     const size_t sm = sizeof(double) * (size_t)maxsub * KC;
-    for (int j0 = 0; j0 < 2 * k; j0 += KC) {
-      k_dav_restart_lincomb<KC><<<parts, kVecThreads, sm, st>>>(V, ctl, Y.as<double>(), maxsub, j0, N, tmp); ISCSI_COUNT_LAUNCH();
-    }
+    k_dav_restart_lincomb<KC><<<dim3(parts, (2 * k + KC - 1) / KC), kVecThreads, sm, st>>>(V, ctl, Y.as<double>(), maxsub,
+                                                                                           N, tmp, nullptr); ISCSI_COUNT_LAUNCH();
     k_dav_restart_copy<<<parts, kVecThreads, 0, st>>>(V, tmp, ctl, N); ISCSI_COUNT_LAUNCH();
   }
 
