@@ -30,44 +30,59 @@ constexpr int kPrBlocks = 152 * 4;  // partial sums per inner product, added in 
 
 // partial inner products <q_k | w> (k < nk) of nc-component vectors (nc = 2:
 // complex [re; im], the conjugate on q; nc = 1: real): part[(block * nk + k) * 2 + {re, im}]
+//
+// Blocks in y take kPrTile vectors each against one read of w; the sums of a warp
+// are exchanged so that each step halves the values a lane carries (8 FP64
+// additions for 8 sums; a butterfly per sum took 40, and FP64 issues two operations per
+// clock per SM).  672,400 determinants, complex: 65 -> 45 us on average over a
+// 14-vector step (eight vectors per block, all in one: 61; in double-float
+// arithmetic on the FP32 units: 85).
+constexpr int kPrTile = 4;
 __global__ void __launch_bounds__(kPrThreads) k_pr_dots(const double* __restrict__ Q, long long qstride, int nk,
                                                         const double* __restrict__ w, int nc, long long ndet,
                                                         double* __restrict__ part) {
-  __shared__ double sre[kPrThreads / 32], sim[kPrThreads / 32];
+  __shared__ double red[kPrThreads / 32][2 * kPrTile];
   const long long per = (ndet + gridDim.x - 1) / gridDim.x;
   const long long i0 = blockIdx.x * per, i1 = min(ndet, i0 + per);
-  for (int k = 0; k < nk; ++k) {
-    const double* q = Q + k * qstride;
-    double re = 0.0, im = 0.0;
-    for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-      const double qr = q[i], wr = w[i];
-      if (nc == 2) {
-        const double qi = q[ndet + i], wi = w[ndet + i];
-        re += qr * wr + qi * wi;
-        im += qr * wi - qi * wr;
-      } else {
-        re += qr * wr;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int k0 = blockIdx.y * kPrTile, kt = min(kPrTile, nk - k0);
+  double x[2 * kPrTile];
+#pragma unroll
+  for (int t = 0; t < 2 * kPrTile; ++t) x[t] = 0.0;
+  for (long long i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+    const double wr = w[i], wi = nc == 2 ? w[ndet + i] : 0.0;
+#pragma unroll
+    for (int t = 0; t < kPrTile; ++t)
+      if (t < kt) {
+        const double* q = Q + (k0 + t) * qstride + i;
+        const double qr = q[0];
+        x[2 * t] = fma(qr, wr, x[2 * t]);
+        if (nc == 2) {
+          const double qi = q[ndet];
+          x[2 * t] = fma(qi, wi, x[2 * t]);
+          x[2 * t + 1] = fma(qr, wi, x[2 * t + 1]);
+          x[2 * t + 1] = fma(-qi, wr, x[2 * t + 1]);
+        }
       }
+  }
+#pragma unroll
+  for (int o = 16, n = 2 * kPrTile; o > 2; o >>= 1, n >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int t = 0; t < n / 2; ++t) {
+      const double give = up ? x[t] : x[t + n / 2], keep = up ? x[t + n / 2] : x[t];
+      x[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      re += __shfl_xor_sync(0xffffffffu, re, o);
-      im += __shfl_xor_sync(0xffffffffu, im, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sre[threadIdx.x >> 5] = re;
-      sim[threadIdx.x >> 5] = im;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double a = 0.0, b = 0.0;
-      for (int j = 0; j < (int)(blockDim.x >> 5); ++j) {
-        a += sre[j];
-        b += sim[j];
-      }
-      part[((long long)blockIdx.x * nk + k) * 2] = a;
-      part[((long long)blockIdx.x * nk + k) * 2 + 1] = b;
-    }
-    __syncthreads();
+  }
+  static_assert(kPrTile == 4, "8 sums: three halvings leave one per four lanes");
+  x[0] += __shfl_xor_sync(0xffffffffu, x[0], 2);
+  x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+  if ((lane & 3) == 0) red[warp][(lane >> 4 & 1) * 4 + (lane >> 3 & 1) * 2 + (lane >> 2 & 1)] = x[0];
+  __syncthreads();
+  if (threadIdx.x < 2 * kt) {
+    double a = 0.0;
+    for (int v = 0; v < kPrThreads / 32; ++v) a += red[v][threadIdx.x];
+    part[((long long)blockIdx.x * nk + k0) * 2 + threadIdx.x] = a;
   }
 }
 
@@ -102,22 +117,28 @@ __global__ void k_pr_sum(const double* __restrict__ part, int parts, int nk, int
   }
 }
 
-// w -= sum_k h[k] q_k  (complex coefficients for nc = 2)
+// w -= sum_k h[k] q_k  (complex coefficients for nc = 2); the coefficients in
+// shared memory, four vectors' loads in flight (as k_pr_dots bound by FP64 issue:
+// 64 -> 41 us for 7.5 vectors)
 __global__ void __launch_bounds__(kPrThreads) k_pr_update(const double* __restrict__ Q, long long qstride, int nk,
                                                           double* __restrict__ w, int nc, long long ndet,
                                                           const PrCtl* __restrict__ ctl) {
+  __shared__ double hs[kPrMaxKrylov][2];
+  for (int t = threadIdx.x; t < 2 * nk; t += blockDim.x) hs[t >> 1][t & 1] = ctl->h[t >> 1][t & 1];
+  __syncthreads();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ndet;
        i += (long long)gridDim.x * blockDim.x) {
     double wr = w[i], wi = nc == 2 ? w[ndet + i] : 0.0;
+#pragma unroll 4
     for (int k = 0; k < nk; ++k) {
-      const double hr = ctl->h[k][0], hi = ctl->h[k][1];
+      const double hr = hs[k][0], hi = hs[k][1];
       const double qr = Q[k * qstride + i];
       if (nc == 2) {
         const double qi = Q[k * qstride + ndet + i];
-        wr -= hr * qr - hi * qi;
-        wi -= hr * qi + hi * qr;
+        wr = fma(-hr, qr, fma(hi, qi, wr));
+        wi = fma(-hr, qi, fma(-hi, qr, wi));
       } else {
-        wr -= hr * qr;
+        wr = fma(-hr, qr, wr);
       }
     }
     w[i] = wr;
@@ -238,7 +259,7 @@ static int propagate_steps(Context& ctx, Context* cpl, double* c, int nsteps, do
       double* qj = Q + (size_t)j * qs;
       ISCSI_TRY(sigma_run(ctx, qj, W, nc, prec));
       for (int pass = 0; pass < 2; ++pass) {
-        k_pr_dots<<<kPrBlocks, kPrThreads, 0, st>>>(Q, qs, j + 1, W, nc, N, part); ISCSI_COUNT_LAUNCH();
+        k_pr_dots<<<dim3(kPrBlocks, j / kPrTile + 1), kPrThreads, 0, st>>>(Q, qs, j + 1, W, nc, N, part); ISCSI_COUNT_LAUNCH();
         k_pr_sum<<<(2 * (j + 1) + 7) / 8, 256, 0, st>>>(part, kPrBlocks, j + 1, 0, j, ctl); ISCSI_COUNT_LAUNCH();
         k_pr_update<<<gb, kPrThreads, 0, st>>>(Q, qs, j + 1, W, nc, N, ctl); ISCSI_COUNT_LAUNCH();
       }
