@@ -34,6 +34,8 @@
 
 #include "internal.cuh"
 #include "crt.cuh"
+#include "crt_gemm.cuh"
+#include "crt_host.cuh"
 #include "ozaki_digits.cuh"
 #include "tma_map.h"
 
@@ -41,15 +43,12 @@ namespace iscsi {
 
 constexpr int kCrtUnitBits = 49;  // bits of the largest unit (the error-free slices' width)
 constexpr int kCrtCBits = 50;     // bits of the largest coefficient
-constexpr int kCrtResMax = 257;   // |residue| as k_crt_gemm stores it
 
 // ---------------------------------------------------------------------------
 // constants
 
-namespace {
-
 // modular inverse of a mod m (coprime)
-int mod_inverse(int a, int m) {
+static int mod_inverse(int a, int m) {
   long long t = 0, nt = 1, r = m, nr = a % m;
   while (nr) {
     const long long q = r / nr;
@@ -59,7 +58,7 @@ int mod_inverse(int a, int m) {
   return (int)(t < 0 ? t + m : t);
 }
 
-CrtMods make_mods(int nm) {
+CrtMods crt_make_mods(int nm) {
   CrtMods c;
   std::memset(&c, 0, sizeof(c));
   c.nm = nm;
@@ -86,7 +85,7 @@ CrtMods make_mods(int nm) {
 
 // reconstruction weights: M's top 64 bits and the fractions (M/m)^-1 / m to 78
 // bits by long division; terms: residues of the first pass of k_crt_fold, of each later pass, later passes
-CrtWeights make_weights(int nm, int terms, int terms_next, int passes_next) {
+CrtWeights crt_make_weights(int nm, int terms, int terms_next, int passes_next) {
   CrtWeights W;
   std::memset(&W, 0, sizeof(W));
   std::vector<uint32_t> M(1, 1);
@@ -132,21 +131,19 @@ CrtWeights make_weights(int nm, int terms, int terms_next, int passes_next) {
   return W;
 }
 
-double log2_product(int nm) {
+double crt_log2_product(int nm) {
   double s = 0.0;
   for (int i = 0; i < nm; ++i) s += std::log2((double)kCrtModuli[i]);
   return s;
 }
 
-inline int up(int x, int m) { return (x + m - 1) / m * m; }
+static inline int up(int x, int m) { return (x + m - 1) / m * m; }
 
 // columns per tile: as few tiles as 256 columns allow, equally wide
-int tile_cols(int N) {
+static int tile_cols(int N) {
   const int nt = (N + CRT_MAXN - 1) / CRT_MAXN;
   return std::max(16, up((N + nt - 1) / nt, 16));
 }
-
-}  // namespace
 
 // ---------------------------------------------------------------------------
 // operand kernels
@@ -579,7 +576,8 @@ __global__ void __launch_bounds__(kFoldThreads) k_crt_fold(const __grid_constant
     }
   }
   const int f = F.cexp[v];
-  const int e = (f > 0 ? f - 1022 : 0) + F.ebias;
+  // a vector with an infinity or NaN: every nonzero sum overflows
+  const int e = (f > 0 ? f - 1022 : 0) + (f == 0x7FF ? 4096 : 0) + F.ebias;
   double* out = sigma + v * F.ndet + F.off[A];
 #pragma unroll
   for (int u = 0; u < kFoldPer; ++u) {
@@ -590,15 +588,6 @@ __global__ void __launch_bounds__(kFoldThreads) k_crt_fold(const __grid_constant
 
 // ---------------------------------------------------------------------------
 // work list and schedule
-// host description of a product: which tiles it has and their k blocks
-struct CrtHostProblem {
-  CrtProblem p;
-  int mt;                          // pairs of row blocks
-  std::function<bool(int, int, int&, int&)> range;  // tile (mt, nt) -> its k blocks; false: no tile
-  int second = -1;                 // product added into the same tiles (relative index), its k blocks by its own range
-  bool own = true;                 // false: only as another's second product
-};
-
 // items in the order that keeps the pairs on neighbouring tiles of one modulus
 // (their operands shared in L2), dealt out in that order to the pair with the
 // least work so far; the products with the largest tiles first
@@ -663,46 +652,40 @@ static int crt_sm_count() {
   return n;
 }
 
-// a list of products on the device with its schedule (one context's, or several merged)
-struct CrtJob {
-  std::vector<CrtHostProblem> probs;
-  DevBuf d_probs, d_items, d_start;
-  int grid = 0, nitems = 0;
-  double flops = 0.0;
-  int upload(cudaStream_t st) {
-    std::vector<CrtItem> items;
-    std::vector<int> start;
-    crt_schedule(probs, crt_sm_count() / 2, items, start, flops);
-    grid = 2 * ((int)start.size() - 1);
-    nitems = (int)items.size();
-    std::vector<CrtProblem> pr;
-    for (const CrtHostProblem& h : probs) pr.push_back(h.p);
-    ISCSI_TRY(d_probs.grow(sizeof(CrtProblem) * std::max<size_t>(1, pr.size())));
-    ISCSI_TRY(d_items.grow(sizeof(CrtItem) * std::max<size_t>(1, items.size())));
-    ISCSI_TRY(d_start.grow(sizeof(int) * start.size()));
-    if (!pr.empty())
-      ISCSI_CUDA(cudaMemcpyAsync(d_probs.p, pr.data(), sizeof(CrtProblem) * pr.size(), cudaMemcpyHostToDevice, st));
-    if (!items.empty())
-      ISCSI_CUDA(
-          cudaMemcpyAsync(d_items.p, items.data(), sizeof(CrtItem) * items.size(), cudaMemcpyHostToDevice, st));
-    ISCSI_CUDA(cudaMemcpyAsync(d_start.p, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, st));
-    ISCSI_CUDA(cudaStreamSynchronize(st));  // the host vectors end here
-    return kOk;
+int CrtJob::upload(cudaStream_t st) {
+  std::vector<CrtItem> items;
+  std::vector<int> start;
+  crt_schedule(probs, crt_sm_count() / 2, items, start, flops);
+  grid = 2 * ((int)start.size() - 1);
+  nitems = (int)items.size();
+  std::vector<CrtProblem> pr;
+  for (const CrtHostProblem& h : probs) pr.push_back(h.p);
+  ISCSI_TRY(d_probs.grow(sizeof(CrtProblem) * std::max<size_t>(1, pr.size())));
+  ISCSI_TRY(d_items.grow(sizeof(CrtItem) * std::max<size_t>(1, items.size())));
+  ISCSI_TRY(d_start.grow(sizeof(int) * start.size()));
+  if (!pr.empty())
+    ISCSI_CUDA(cudaMemcpyAsync(d_probs.p, pr.data(), sizeof(CrtProblem) * pr.size(), cudaMemcpyHostToDevice, st));
+  if (!items.empty())
+    ISCSI_CUDA(
+        cudaMemcpyAsync(d_items.p, items.data(), sizeof(CrtItem) * items.size(), cudaMemcpyHostToDevice, st));
+  ISCSI_CUDA(cudaMemcpyAsync(d_start.p, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, st));
+  ISCSI_CUDA(cudaStreamSynchronize(st));  // the host vectors end here
+  return kOk;
+}
+
+int CrtJob::launch(int* err, cudaStream_t st) const {
+  if (grid == 0) return kOk;
+  static bool attr = false;
+  if (!attr) {
+    ISCSI_CUDA(cudaFuncSetAttribute(k_crt_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, CRT_SMEM_BYTES));
+    attr = true;
   }
-  int launch(int* err, cudaStream_t st) const {
-    if (grid == 0) return kOk;
-    static bool attr = false;
-    if (!attr) {
-      ISCSI_CUDA(cudaFuncSetAttribute(k_crt_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, CRT_SMEM_BYTES));
-      attr = true;
-    }
-    static const CrtMods all = make_mods(kCrtMaxMods);  // the kernel reads the moduli themselves
-    k_crt_gemm<<<grid, CRT_THREADS, CRT_SMEM_BYTES, st>>>(d_probs.as<CrtProblem>(), d_items.as<CrtItem>(),
-                                                          d_start.as<int>(), all, err); ISCSI_COUNT_LAUNCH();
-    ISCSI_CUDA(cudaGetLastError());
-    return kOk;
-  }
-};
+  static const CrtMods all = crt_make_mods(kCrtMaxMods);  // the kernel reads the moduli themselves
+  k_crt_gemm<<<grid, CRT_THREADS, CRT_SMEM_BYTES, st>>>(d_probs.as<CrtProblem>(), d_items.as<CrtItem>(),
+                                                        d_start.as<int>(), all, err); ISCSI_COUNT_LAUNCH();
+  ISCSI_CUDA(cudaGetLastError());
+  return kOk;
+}
 
 // ---------------------------------------------------------------------------
 // a context's state
@@ -720,6 +703,7 @@ struct CrtFoldLaunch {
 
 struct CrtState {
   bool off = false;  // its buffers did not fit (or its units are not finite): the context stays on the slices
+  size_t held = 0;   // bytes of residue buffers (crt_alloc)
   bool flat = false;  // every class reaches every row: no levels in the orders
   std::vector<CrtGroup> groups;
   std::vector<int> ystart;
@@ -860,7 +844,7 @@ bool crt_ss_active(Context& ctx) {
   return !S.off && ctx.sp[0].count >= kCrtMinRows && ctx.sp[1].count >= kCrtMinRows;
 }
 
-static int encode(CrtProblem& P, const void* a, const void* b, int nm) {
+int crt_encode(CrtProblem& P, const void* a, const void* b, int nm) {
   if (crt_encode_map(&P.a, a, (long long)nm * P.nblk_a * P.nkb_a * CRT_BM, CRT_BM) ||
       crt_encode_map(&P.b, b, (long long)nm * P.nblk_b * P.nkb_b * (P.ntile / 2), P.ntile / 2)) {
     set_error("residue contraction: TMA descriptor rejected");
@@ -932,7 +916,7 @@ static void choose_scale(double bound, double maxel, double ref, int& nm, int& s
   if (ref <= 0.0) ref = maxel;
   for (nm = 10; nm <= kCrtMaxMods; ++nm) {
     // 2^(sh + bc) bound < M / 2, a hundredth of a bit apart (the roundings of the integers)
-    sh = (int)std::floor(log2_product(nm) - 1.01 - kCrtCBits - std::log2(bound));
+    sh = (int)std::floor(crt_log2_product(nm) - 1.01 - kCrtCBits - std::log2(bound));
     const int cap = 51 - (int)std::floor(std::log2(maxel));  // integers below 2^52
     const bool full = sh >= cap;  // more moduli would add nothing
     sh = std::min(sh, cap);
@@ -950,7 +934,7 @@ static int crt_cut_m(Context& ctx) {
   if (ctx.na > 0 && ctx.M64[0].p) {
     const int rp = up(NA, 2 * CRT_BM);
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)S.mods.nm * rp * ka * CRT_BK;
-    if (S.ma_res.bytes < bytes) ISCSI_TRY(S.ma_res.alloc(bytes));
+    if (S.ma_res.bytes < bytes) ISCSI_TRY(crt_alloc(S.ma_res, bytes, S.held));
     ISCSI_TRY(cut_matrix(ctx.M64[0].as<double>(), NA, NA, NA, 0, nullptr, S.sh, CRT_BM, rp, ka, S.mods,
                          S.ma_res.as<__nv_bfloat16>(), st));
   }
@@ -959,7 +943,7 @@ static int crt_cut_m(Context& ctx) {
     const double* Mb = beta_matrix(ctx, trans);
     const int rp = tn * ntile;
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)S.mods.nm * rp * kb * CRT_BK;
-    if (S.mb_res.bytes < bytes) ISCSI_TRY(S.mb_res.alloc(bytes));
+    if (S.mb_res.bytes < bytes) ISCSI_TRY(crt_alloc(S.mb_res, bytes, S.held));
     ISCSI_TRY(cut_matrix(Mb, NB, NB, NB, trans, nullptr, S.sh, bt, rp, kb, S.mods, S.mb_res.as<__nv_bfloat16>(), st));
   }
   S.m_cut[0] = S.mods.nm;
@@ -1005,7 +989,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
     int nm = 0;
     choose_scale(b, maxel, (parts & 1) ? S.gmax : mmax, nm, S.sh);
     S.bound = b;
-    S.mods = make_mods(nm);
+    S.mods = crt_make_mods(nm);
   }
   const int nm = S.mods.nm;
   S.job.probs.clear();
@@ -1096,7 +1080,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
     }
     const size_t gbytes = sizeof(__nv_bfloat16) * (size_t)nm * rp * gk * CRT_BK;
     if (S.g_res.bytes < gbytes) {
-      ISCSI_TRY(S.g_res.alloc(gbytes));
+      ISCSI_TRY(crt_alloc(S.g_res, gbytes, S.held));
       S.g_cut[0] = -1;
     }
     if (S.g_cut[0] != nm || S.g_cut[1] != S.sh) {
@@ -1126,7 +1110,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
       O.blk_start[gi + 1] = O.blk_start[gi] + (N + 8 / L.wpc - 1) / (8 / L.wpc);
     }
     S.ops_smem = crt_lift_col_bytes(n) * cpb;
-    if (S.b_res.bytes < sizeof(__nv_bfloat16) * elems) ISCSI_TRY(S.b_res.alloc(sizeof(__nv_bfloat16) * elems));
+    if (S.b_res.bytes < sizeof(__nv_bfloat16) * elems) ISCSI_TRY(crt_alloc(S.b_res, sizeof(__nv_bfloat16) * elems, S.held));
     // the padding rows of every group stay zero from here on
     ISCSI_CUDA(cudaMemsetAsync(S.b_res.p, 0, S.b_res.bytes, st));
     O.lift = S.b_res.as<__nv_bfloat16>();
@@ -1153,7 +1137,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
         k1 = nkb;
         return true;
       };
-      ISCSI_TRY(encode(H.p, S.g_res.p, S.b_res.as<__nv_bfloat16>() + L.base, nm));
+      ISCSI_TRY(crt_encode(H.p, S.g_res.p, S.b_res.as<__nv_bfloat16>() + L.base, nm));
       F.g[gi].res = (long long)out_elems;
       F.g[gi].ncol = L.ncol;
       F.g[gi].ntile = H.p.ntile;
@@ -1191,8 +1175,8 @@ static int crt_build(Context& ctx, int nvec, int parts) {
     O.ctx_x = (NB + 63) / 64;
     O.ctx_y = (NA + 63) / 64;
     const size_t ctb = sizeof(__nv_bfloat16) * (size_t)O.ct_vec * nvec, cab = sizeof(__nv_bfloat16) * (size_t)O.ca_vec * nvec;
-    if (al && S.ct_res.bytes < ctb) ISCSI_TRY(S.ct_res.alloc(ctb));
-    if (be && S.ca_res.bytes < cab) ISCSI_TRY(S.ca_res.alloc(cab));
+    if (al && S.ct_res.bytes < ctb) ISCSI_TRY(crt_alloc(S.ct_res, ctb, S.held));
+    if (be && S.ca_res.bytes < cab) ISCSI_TRY(crt_alloc(S.ca_res, cab, S.held));
     // elements outside the space (and padding) stay zero from here on
     if (al) ISCSI_CUDA(cudaMemsetAsync(S.ct_res.p, 0, S.ct_res.bytes, st));
     if (be) ISCSI_CUDA(cudaMemsetAsync(S.ca_res.p, 0, S.ca_res.bytes, st));
@@ -1240,7 +1224,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
             k1 = (ls[std::min(l1, maxl + 1)] + CRT_BK - 1) / CRT_BK;
             return true;
           };
-          ISCSI_TRY(encode(H.p, S.ma_res.p, S.ct_res.as<__nv_bfloat16>() + O.ct_vec * v, nm));
+          ISCSI_TRY(crt_encode(H.p, S.ma_res.p, S.ct_res.as<__nv_bfloat16>() + O.ct_vec * v, nm));
           if (be) H.second = 1;
         } else {
           // the allowed beta prefix of the tile's first (lowest) level
@@ -1251,7 +1235,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
             k1 = (int)((nba[lo] + CRT_BK - 1) / CRT_BK);
             return true;
           };
-          ISCSI_TRY(encode(H.p, S.ca_res.as<__nv_bfloat16>() + O.ca_vec * v, S.mb_res.p, nm));
+          ISCSI_TRY(crt_encode(H.p, S.ca_res.as<__nv_bfloat16>() + O.ca_vec * v, S.mb_res.p, nm));
         }
         if (first) {
           if (v == 1) F.ss_vec = (long long)out_elems - F.ss_res;
@@ -1265,7 +1249,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
       }
     }
   }
-  if (S.out.bytes < sizeof(int16_t) * out_elems) ISCSI_TRY(S.out.alloc(sizeof(int16_t) * out_elems));
+  if (S.out.bytes < sizeof(int16_t) * out_elems) ISCSI_TRY(crt_alloc(S.out, sizeof(int16_t) * out_elems, S.held));
   for (size_t i = 0; i < S.job.probs.size(); ++i) S.job.probs[i].p.res = S.out.as<int16_t>() + out_off[i];
   F.res = S.out.as<int16_t>();
   // the fold's launches: levels of alpha strings with their own staged shape (fewer than 64 strings
@@ -1295,7 +1279,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
       L.smem = fs.smem;
       passes = (ctx.na + ni - 1) / ni;
     }
-    L.w = make_weights(nm, ((parts & 1) ? ni * ctx.nb : 0) + 1, ni * ctx.nb, passes - 1);
+    L.w = crt_make_weights(nm, ((parts & 1) ? ni * ctx.nb : 0) + 1, ni * ctx.nb, passes - 1);
     int lim = (int)ctx.nb_allowed_lvl[l0], most = (int)ctx.nb_allowed_lvl[l - 1];
     L.threads = std::min(kFoldThreads, std::max(64, up((std::max(most, (lim + 3) / 4) + kFoldPer - 1) / kFoldPer, 32)));
     L.blocks = (lim + L.threads * kFoldPer - 1) / (L.threads * kFoldPer);
@@ -1306,6 +1290,20 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   S.nvec = nvec;
   S.parts = parts;
   ++S.version;
+  return kOk;
+}
+
+int crt_alloc(DevBuf& d, size_t bytes, size_t& held) {
+  held -= std::min(held, d.bytes);
+  d.release();
+  size_t free_b = 0, total = 0;
+  ISCSI_CUDA(cudaMemGetInfo(&free_b, &total));
+  if (held + bytes > (free_b + held) / 2) {
+    set_error("residues: less than half of the free memory would be left");
+    return kErrNoMem;
+  }
+  ISCSI_TRY(d.alloc(bytes));
+  held += bytes;
   return kOk;
 }
 

@@ -6,7 +6,7 @@
 // The paper builds them with the sigma step's class loops, a product of two CI
 // coefficients in place of the integral.  Here each two-body block is one
 // Gram-type contraction of "lifted" vectors, on the tensor cores with FP64
-// accuracy (the exact bf16 slices of ozaki.cuh):
+// accuracy:
 //   ab: L[(q,t)][(X,Y)] = <X,Y| a_tu a_qs |ket> (X, Y: strings with one alpha
 //       and one beta electron removed -- the sigma step's hole strings and its
 //       lift tables), so d2_ab[p,q,r,t] = sum_XY L_bra[(p,r)] L_ket[(q,t)];
@@ -20,6 +20,10 @@
 // (the block's "staircase"), one tensor-core problem per region pair.  With
 // ket = bra the result is symmetric and only the upper regions (and, in a
 // diagonal region, the tiles right of each 128-row block's start) are computed.
+// The products go through residue numbers (crt.cuh): one integer scale per vector,
+// |d2| <= |bra| |ket| by Cauchy-Schwarz (a row of L holds each coefficient at most
+// once), 13 moduli.  Contexts whose residues do not fit take the exact bf16
+// slices of ozaki.cuh instead.
 // An expansion kernel writes the n^4 tensors from the pair-indexed results.
 // d1 comes from d2's partial trace when d2 is computed for that spin (sum_r
 // d2_ss[p,q,r,r] = (N_s - 1) d1_s[p,q], summed by the expansion kernel), else
@@ -29,6 +33,8 @@
 #include <cstring>
 #include <vector>
 
+#include "crt.cuh"
+#include "crt_host.cuh"
 #include "internal.cuh"
 #include "ozaki_digits.cuh"
 
@@ -39,7 +45,8 @@ constexpr int kDmMaxBnd = 2 * kMaxElec + 2;
 // ---------------------------------------------------------------------------
 // host plan
 
-struct DmPart {            // one column level class of a block
+struct DmPart {            // one column level class of a block (kb0, nkb: its 64-wide K blocks in the residues)
+  int kb0 = 0, nkb = 0;
   int col_start = 0;       // first column in the block's column list
   int ncol = 0;            // columns (K)
   int rows = 0;            // rows reached (pairs with level <= k - c)
@@ -56,10 +63,26 @@ struct DmBlock {
   size_t q_off = 0;        // double offset of the R x R result in the result workspace
   size_t exp_off = 0;      // int offset of its row exponents (parts x R128) in an exponent workspace
   int R128 = 0;
+  // residue operands: R256 rows of nkb K blocks per modulus, at res_off
+  int R256 = 0, nkb = 0;
+  size_t res_off = 0;
 };
+
+constexpr int kDmMods = 13;     // products of two vectors of 57 bits' 2-norm stay below half the moduli's product
+constexpr int kDmNormBits = 57;
+constexpr int kDmScaleBlocks = 304;
+constexpr int kDmNotFinite = -(1 << 20);  // scale of a vector with an infinity or NaN: every element of the result is NaN
 
 struct DensityPlan {
   bool built = false;
+  // residues (res_fail: they do not fit): operands of bra and ket, output residues, scales
+  bool res_fail = false;
+  size_t res_held = 0;
+  DevBuf res_bra, res_ket, res_out, scale, scale_part;
+  CrtJob res_job[2];             // ket = bra / general
+  bool res_ready[2] = {false, false};
+  std::vector<size_t> res_out_off;
+  bool slices = false;           // the slice workspaces below are allocated
   DmBlock blk[3];
   // same-spin tables per spin: pair row of {u<v}, two-hole lift, column list (Z, other string)
   DevBuf pp_row[2], lift2[2], cols[2];
@@ -261,18 +284,32 @@ static int plan_build(Context& ctx) {
     q = (q + 31) / 32 * 32;
     B.exp_off = ex;
     ex += (size_t)B.parts.size() * B.R128;
+    B.R256 = rup(std::max(B.R, 1), 2 * CRT_BM);
+    B.nkb = 0;
+    for (DmPart& pt : B.parts) {
+      pt.kb0 = B.nkb;
+      pt.nkb = rup(pt.ncol, CRT_BK) / CRT_BK;
+      B.nkb += pt.nkb;
+    }
   }
   for (cudaEvent_t& e : P.ev) ISCSI_CUDA(cudaEventCreate(&e));
   P.sl_elems = sl;
   P.q_elems = q;
   P.ex_elems = ex;
-  if (sl) ISCSI_TRY(P.sl_bra.alloc(sizeof(__nv_bfloat16) * sl));
   if (q) ISCSI_TRY(P.q.alloc(sizeof(double) * q));
-  if (ex) {
-    ISCSI_TRY(P.ex_bra.alloc(sizeof(int) * ex));
-    ISCSI_CUDA(cudaMemset(P.ex_bra.p, 0, sizeof(int) * ex));
-  }
   P.built = true;
+  return kOk;
+}
+
+// workspaces of the slices (contexts without residues)
+static int slices_alloc(DensityPlan& P) {
+  if (P.slices) return kOk;
+  if (P.sl_elems) ISCSI_TRY(P.sl_bra.alloc(sizeof(__nv_bfloat16) * P.sl_elems));
+  if (P.ex_elems) {
+    ISCSI_TRY(P.ex_bra.alloc(sizeof(int) * P.ex_elems));
+    ISCSI_CUDA(cudaMemset(P.ex_bra.p, 0, sizeof(int) * P.ex_elems));
+  }
+  P.slices = true;
   return kOk;
 }
 
@@ -410,6 +447,180 @@ __global__ void __launch_bounds__(256) k_dm_lift_slice(DmGather g, int col_start
   }
 }
 
+// Scale of a vector: the integer unit 2^-scale with |c| 2^scale <= 2^57 (2-norm) and
+// max |c_i| 2^scale <= 2^52.  Block b leaves the largest exponent field of its elements
+// and the sum of their squares relative to it, the last block to finish combines
+// them and clears the counter.  Squares are FP32 sums of values built by integer
+// operations, rounded up (an FP64 product costs 64 cycles a warp: 3.1 M determinants took 26 us
+// with FP64 products, 16 with these): only the norm's binary order is wanted.  A vector
+// that is not finite gets kDmNotFinite.
+__global__ void __launch_bounds__(256) k_dm_norm(const double* __restrict__ c, long long ndet, int* __restrict__ pmax,
+                                                 float* __restrict__ psum, int* __restrict__ done,
+                                                 int* __restrict__ scale) {
+  const long long per = (ndet + gridDim.x - 1) / gridDim.x;
+  const long long i0 = blockIdx.x * per, i1 = min(ndet, i0 + per);
+  __shared__ int sm[8];
+  __shared__ float ss[8];
+  __shared__ bool last;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int m = 0;
+#pragma unroll 8
+  for (long long i = i0 + threadIdx.x; i < i1; i += 256) m = max(m, oz_exp_field(c[i]));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) sm[warp] = m;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) m = max(m, sm[w]);
+  float s = 0.0f;
+#pragma unroll 8
+  for (long long i = i0 + threadIdx.x; i < i1; i += 256) {
+    // |x| 2^(1022 - m) < 1 as FP32, its mantissa cut to 23 bits and raised by one; 0 below 2^-60
+    const unsigned long long b = (unsigned long long)__double_as_longlong(c[i]);
+    const int E = (int)((b >> 52) & 0x7FF) - m + 126;
+    const float x = E > 66 ? __uint_as_float(((uint32_t)E << 23 | (uint32_t)((b >> 29) & 0x7FFFFFu)) + 1u) : 0.0f;
+    s = fmaf(x, x, s);
+  }
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) ss[warp] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float t = 0.0f;
+    for (int w = 0; w < 8; ++w) t += ss[w];
+    pmax[blockIdx.x] = m;
+    psum[blockIdx.x] = t;
+    __threadfence();
+    last = atomicAdd(done, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last || warp != 0) return;
+  __threadfence();
+  int M = 0;
+  for (int b = lane; b < (int)gridDim.x; b += 32) M = max(M, __ldcg(pmax + b));
+  M = __reduce_max_sync(0xffffffffu, M);
+  float t = 0.0f;
+  for (int b = lane; b < (int)gridDim.x; b += 32) t += ldexpf(__ldcg(psum + b), 2 * max(__ldcg(pmax + b) - M, -60));
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane != 0) return;
+  *done = 0;
+  int k = 0;  // |c| < 2^(e + k), max |c_i| < 2^e
+  // a thread's FP32 sum of up to 2^18 terms (2^34 determinants) is within 2^-6 of the truth
+  for (float u = t * 1.02f; u >= 1.0f && k < 64; u *= 0.25f) ++k;
+  const int e = M - 1022;
+  *scale = M == 0x7FF ? kDmNotFinite : M > 0 ? min(kDmNormBits - e - k, 52 - e) : 0;
+}
+
+// Residues of one part's columns, one block per row of L: 8 consecutive columns
+// per thread (row entries staged as in k_dm_lift_slice).  Rows the part does not
+// reach and padding are zero from the buffer's first clearing on.  26 bytes written per
+// element: full CI in 60 orbitals 495 MB in 206 us (the slices: 187 us), latency of the
+// gathers and the row staging.
+template <bool STAGED>
+__global__ void __launch_bounds__(256) k_dm_cut(DmGather g, int col_start, int ncol, int kb0, int nkb, int nkb_all,
+                                                long long mod_stride, const int* __restrict__ scale,
+                                                const __grid_constant__ CrtMods M, const double* __restrict__ c,
+                                                __nv_bfloat16* __restrict__ out) {
+  const int r = blockIdx.x;
+  __shared__ DmStageRow S;
+  if (STAGED) {
+    const int qt = g.pair_of[r];
+    const int q = qt / g.n, t = qt - (qt / g.n) * g.n;
+    for (int X = threadIdx.x; X < g.nholeA; X += blockDim.x) {
+      const int ea = g.liftA[q * g.nholeA + X];
+      S.a[X] = ea;
+      if (ea >= 0) {
+        const int A = ea >> 1;
+        S.off[X] = g.off[A];
+        S.lim[X] = g.nballow[g.alevel[A]];
+      }
+    }
+    for (int Y = threadIdx.x; Y < g.nholeB; Y += blockDim.x) S.b[Y] = g.liftB[t * g.nholeB + Y];
+    __syncthreads();
+  }
+  const int sc = *scale;
+  __nv_bfloat16* row = out + ((long long)(r >> 7) * nkb_all + kb0) * (CRT_BM * CRT_BK) + (r & 127) * CRT_BK;
+  for (int kc = blockIdx.y * 256 + threadIdx.x; kc < 8 * nkb; kc += 256 * gridDim.y) {
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = kc * 8 + j;
+      v[j] = k < ncol ? dm_row_value<STAGED>(g, S, col_start + k, r, c) : 0.0;
+    }
+    CrtLimbs2 x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] = crt_limbs2(crt_fixed(v[2 * j], 0, sc), crt_fixed(v[2 * j + 1], 0, sc));
+    crt_store8(x, M, row + (long long)(kc >> 3) * (CRT_BM * CRT_BK) + (kc & 7) * 8, mod_stride);
+  }
+}
+
+// Q (R x R) from the residues of L_bra L_ket^T: a warp 32 rows x 8 columns, its rows' runs turned
+// across lane octets; ket = bra: only the tiles on and above the diagonal exist, their mirror
+// images are written with them (32 rows of a column at once).  All moduli's loads in flight, one
+// launch for the three blocks (four in flight and a launch per block: 160 us at n = 60, now 88;
+// the slices' kernel rebuilt in its epilogue and mirrored in 46).
+struct DmRebuild {
+  const int16_t* res[3];
+  double* q[3];
+  int R[3], tn[3], tile0[4];  // of the blocks ab, aa, bb; tile0: first tile of each in the grid
+};
+__global__ void __launch_bounds__(256) k_dm_rebuild(const __grid_constant__ DmRebuild D, int sym,
+                                                    const int* __restrict__ scale_bra, const int* __restrict__ scale_ket,
+                                                    const __grid_constant__ CrtWeights W) {
+  const int blk = ((int)blockIdx.x >= D.tile0[1] ? 1 : 0) + ((int)blockIdx.x >= D.tile0[2] ? 1 : 0);
+  const int tl = blockIdx.x - D.tile0[blk], R = D.R[blk], tn = D.tn[blk];
+  double* __restrict__ q = D.q[blk];
+  const int rt = tl / tn, nt = tl - rt * tn;
+  if (sym && (rt >> 1) > nt) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int e = -(*scale_bra + *scale_ket);
+  const bool bad = min(*scale_bra, *scale_ket) == kDmNotFinite;
+  const int lift = e < -900 ? 600 : 0;  // crt_value gives 0 below the normal range: rounded there by a product
+  constexpr int tile = CRT_BM * CRT_MAXN;
+  const int16_t* base = D.res[blk] + ((long long)rt * tn + nt) * kDmMods * tile;
+  for (int w = warp; w < 32; w += 8) {
+    const int cg = blockIdx.y * 8 + (w >> 2), quarter = w & 3;
+    const int r0 = rt * CRT_BM + quarter * 32, col = nt * CRT_MAXN + cg * 8;
+    if (r0 >= R || col >= R) continue;
+    unsigned long long lo[8];
+    uint32_t hi[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      lo[j] = W.start_lo;
+      hi[j] = W.start_hi;
+    }
+    const int16_t* src = base + (cg * CRT_BM + quarter * 32 + lane) * 8;
+#pragma unroll
+    for (int i = 0; i < kDmMods; ++i) {
+      const uint4 x = __ldg(reinterpret_cast<const uint4*>(src + (long long)i * tile));
+      const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
+      const uint32_t w0 = W.lo0[i], w1 = W.lo1[i], w2 = W.hi[i];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint32_t t = (uint32_t)((int)(int16_t)(xw[j >> 1] >> (16 * (j & 1))) + W.off[i]);
+        lo[j] += (unsigned long long)t * w0;
+        lo[j] += (unsigned long long)(t * w1) << 32;
+        hi[j] += t * w2;
+      }
+    }
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = crt_value(lo[j], hi[j], W.mman, W.mexp, e + lift);
+    if (lift)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] *= 0x1p-600;
+    if (bad)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = __longlong_as_double(0x7FF8000000000000ll);
+    if (sym && (rt >> 1) < nt && r0 + lane < R)
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (col + j < R) q[(long long)(col + j) * R + r0 + lane] = v[j];
+    oz_lane_transpose<8>(v, lane);
+    const int rr = r0 + (lane & ~7), cc = col + (lane & 7);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (cc < R && rr + k < R) q[(long long)(rr + k) * R + cc] = v[k];
+  }
+}
+
 // ---------------------------------------------------------------------------
 // device: expansion to the n^4 tensors, one-body matrices
 
@@ -447,12 +658,6 @@ __global__ void __launch_bounds__(256) k_dm_mirror(DmResult Q, double* __restric
   }
 }
 
-// Q[x][y] (0 outside the rows any class reaches)
-__device__ __forceinline__ double dm_read(const DmResult& Q, int x, int y) {
-  if (x >= Q.R || y >= Q.R) return 0.0;
-  return Q.q[(long long)x * Q.R + y];
-}
-
 struct DmExpand {
   int n, na, nb;
   DmResult blk[3];        // in d2's block order: aa, ab, bb
@@ -460,43 +665,65 @@ struct DmExpand {
   const int* pp_row[2];   // aa / bb: {u < v} -> row
 };
 
-// d2 block b = 0 (aa) or 2 (bb): s(p,r) s(q,t) Q[{p,r}][{q,t}]
-__device__ __forceinline__ double dm_samespin(const DmExpand& E, int b, int p, int q, int r, int t) {
-  if (p == r || q == t) return 0.0;
-  const int* pr = E.pp_row[b == 0 ? 0 : 1];
-  int x = pr[min(p, r) * E.n + max(p, r)], y = pr[min(q, t) * E.n + max(q, t)];
-  double v = dm_read(E.blk[b], x, y);
-  return ((p < r) == (q < t)) ? v : -v;
-}
-
-// one block per (p, q) and d2 block b: writes d2[b][p][q][r][t] for all (r, t),
-// consecutive threads on consecutive t (coalesced stores; the pair-indexed
-// reads are mostly consecutive within a level group)
+// One block per (p, q) and d2 block b writes d2[b][p][q][r][t] for all (r, t): b = 1 (ab)
+// Q[(p,r)][(q,t)], b = 0 (aa) or 2 (bb) s(p,r) s(q,t) Q[{p,r}][{q,t}].  A row's index, a
+// column's index and their signs are taken once per block into shared memory
+// (twice the row, 1 for the sign; -1: no row), so an element costs one read of
+// Q (mostly consecutive in t within a level group) and one store; lanes run over
+// t, a warp over the rows r, eight reads in flight.  3 n^4 stores; n = 60: 157 us
+// (indices and a division per element: 173).
 // A same-spin block's (p, q) block also yields d1_s[p][q] = sum_r d2_ss[p,q,r,r]
 // / (N_s - 1) (written when d1 is given and N_s >= 2).
 __global__ void __launch_bounds__(256) k_dm_expand(DmExpand E, double* __restrict__ d2, double* __restrict__ d1) {
+  extern __shared__ int dm_idx[];
   const int n = E.n, p = blockIdx.x / n, q = blockIdx.x - (blockIdx.x / n) * n, b = blockIdx.y;
   const long long n2 = (long long)n * n;
   double* __restrict__ out = d2 + (long long)b * n2 * n2 + (long long)blockIdx.x * n2;
   const bool ab = b == 1 && E.na > 0 && E.nb > 0;
   const bool ss = b != 1 && (b == 0 ? E.na : E.nb) >= 2;
+  const DmResult& Q = E.blk[b];
+  for (int i = threadIdx.x; i < 2 * n; i += 256) {
+    const int u = i < n ? p : q, w = i < n ? i : i - n;
+    int x = -1, sg = 0;
+    if (ab) {
+      x = E.pair_index[u * n + w];
+    } else if (ss && u != w) {
+      x = E.pp_row[b == 0 ? 0 : 1][min(u, w) * n + max(u, w)];
+      sg = u < w ? 1 : 0;
+    }
+    dm_idx[i] = x >= 0 && x < Q.R ? 2 * x + sg : -1;
+  }
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double tr = 0.0;
-  for (int rt = threadIdx.x; rt < n * n; rt += blockDim.x) {
-    const int r = rt / n, t = rt - (rt / n) * n;
-    double v = 0.0;
-    if (ab) v = dm_read(E.blk[1], E.pair_index[p * n + r], E.pair_index[q * n + t]);
-    else if (ss) v = dm_samespin(E, b, p, q, r, t);
-    out[rt] = v;
-    if (r == t) tr += v;
+  for (int t = lane; t < n; t += 32) {
+    const int y = dm_idx[n + t];
+    const double* __restrict__ col = Q.q + (y >> 1);
+    for (int r0 = warp; r0 < n; r0 += 64) {
+      long long v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int r = r0 + 8 * j, x = r < n ? dm_idx[r] : -1;
+        v[j] = x >= 0 && y >= 0
+                   ? __double_as_longlong(__ldg(col + (long long)(x >> 1) * Q.R)) ^ ((long long)((x ^ y) & 1) << 63)
+                   : 0;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int r = r0 + 8 * j;
+        if (r < n) __stcs(out + r * n + t, __longlong_as_double(v[j]));
+        if (r == t) tr += __longlong_as_double(v[j]);
+      }
+    }
   }
   if (!ss || !d1) return;
   __shared__ double red[8];
   for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = tr;
+  if (lane == 0) red[warp] = tr;
   __syncthreads();
   if (threadIdx.x == 0) {
     double sum = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
+    for (int w = 0; w < 8; ++w) sum += red[w];
     const int spin = b == 0 ? 0 : 1;
     d1[(long long)spin * n2 + blockIdx.x] = sum / (double)((spin == 0 ? E.na : E.nb) - 1);
   }
@@ -653,6 +880,100 @@ static int build_job(Context& ctx, bool sym) {
   return kOk;
 }
 
+// residue operands, products and schedule (sym: ket = bra); kErrNoMem: they do not fit
+static int residues_build(Context& ctx, bool sym) {
+  DensityPlan& P = *ctx.dm;
+  const int idx = sym ? 0 : 1;
+  if (P.res_ready[idx]) return kOk;
+  cudaStream_t st = stream();
+  size_t elems = 0, out = 0;
+  P.res_out_off.assign(3, 0);
+  for (int b = 0; b < 3; ++b) {
+    DmBlock& B = P.blk[b];
+    if (B.parts.empty()) continue;
+    B.res_off = elems;
+    elems += (size_t)kDmMods * B.R256 * B.nkb * CRT_BK;
+    P.res_out_off[b] = out;
+    out += (size_t)kDmMods * B.R256 * B.R256;
+    // sums of chunk residues stay exact below 2^24 / 257 chunks; tensor map rows are 32-bit
+    if (B.nkb > CRT_CHUNK * 60000 || (long long)kDmMods * B.R256 * B.nkb >= (1ll << 31)) return kErrNoMem;
+  }
+  DevBuf* ops[2] = {&P.res_bra, sym ? nullptr : &P.res_ket};
+  for (DevBuf* d : ops)
+    if (d && d->bytes < sizeof(__nv_bfloat16) * elems) {
+      ISCSI_TRY(crt_alloc(*d, sizeof(__nv_bfloat16) * elems, P.res_held));
+      ISCSI_CUDA(cudaMemsetAsync(d->p, 0, d->bytes, st));
+    }
+  if (P.res_out.bytes < sizeof(int16_t) * out) ISCSI_TRY(crt_alloc(P.res_out, sizeof(int16_t) * out, P.res_held));
+  if (!P.scale.p) {
+    ISCSI_TRY(P.scale.alloc(2 * sizeof(int)));
+    ISCSI_TRY(P.scale_part.alloc(sizeof(int) * (2 * kDmScaleBlocks + 1)));
+    ISCSI_CUDA(cudaMemsetAsync(P.scale_part.p, 0, P.scale_part.bytes, st));
+  }
+  CrtJob& job = P.res_job[idx];
+  job.probs.clear();
+  double f64 = 0.0;
+  for (int b = 0; b < 3; ++b) {
+    const DmBlock& B = P.blk[b];
+    if (B.parts.empty()) continue;
+    CrtHostProblem H;
+    std::memset(&H.p, 0, sizeof(H.p));
+    H.p.ntile = CRT_MAXN;
+    H.p.tn = B.R256 / CRT_MAXN;
+    H.p.nm = kDmMods;
+    H.p.rt = rup(B.R, CRT_BM) / CRT_BM;
+    H.p.nblk_a = H.p.nblk_b = B.R256 / CRT_BM;
+    H.p.nkb_a = H.p.nkb_b = B.nkb;
+    H.p.res = P.res_out.as<int16_t>() + P.res_out_off[b];
+    H.mt = B.R256 / (2 * CRT_BM);
+    std::vector<DmPart> parts = B.parts;
+    H.range = [parts, sym](int mt, int nt, int& k0, int& k1) {
+      if (sym && mt > nt) return false;
+      // the classes that reach both row ranges: a prefix
+      k0 = k1 = 0;
+      for (const DmPart& pt : parts)
+        if (pt.rows > std::max(mt, nt) * 2 * CRT_BM) k1 = pt.kb0 + pt.nkb;
+      return true;
+    };
+    const __nv_bfloat16* a = P.res_bra.as<__nv_bfloat16>() + B.res_off;
+    ISCSI_TRY(crt_encode(H.p, a, sym ? a : P.res_ket.as<__nv_bfloat16>() + B.res_off, kDmMods));
+    job.probs.push_back(H);
+    for (const DmPart& pt : B.parts) f64 += 2.0 * pt.ncol * pt.rows * (sym ? 0.5 * (pt.rows + 1.0) : (double)pt.rows);
+  }
+  ISCSI_TRY(job.upload(st));
+  P.bf16_flops[idx] = job.flops;
+  P.fp64_flops[idx] = f64;
+  P.res_ready[idx] = true;
+  return kOk;
+}
+
+// a vector's residues (which: 0 bra, 1 ket)
+static int residues_cut(Context& ctx, const double* v, int which, cudaStream_t st) {
+  DensityPlan& P = *ctx.dm;
+  static const CrtMods mods = crt_make_mods(kDmMods);
+  int* part = P.scale_part.as<int>();
+  k_dm_norm<<<kDmScaleBlocks, 256, 0, st>>>(v, ctx.ndet, part, reinterpret_cast<float*>(part + kDmScaleBlocks),
+                                            part + 2 * kDmScaleBlocks, P.scale.as<int>() + which); ISCSI_COUNT_LAUNCH();
+  for (int b = 0; b < 3; ++b) {
+    const DmBlock& B = P.blk[b];
+    if (B.parts.empty()) continue;
+    const DmGather g = gather_of(ctx, P, b);
+    __nv_bfloat16* out = (which ? P.res_ket : P.res_bra).as<__nv_bfloat16>() + B.res_off;
+    const long long mod_stride = (long long)B.R256 * B.nkb * CRT_BK;
+    for (const DmPart& pt : B.parts) {
+      const dim3 grid(pt.rows, std::max(1, std::min(8, pt.nkb / 64)));
+      const int* sc = P.scale.as<int>() + which;
+      if (b == 0 && g.nholeA <= kDmStage && g.nholeB <= kDmStage)
+        k_dm_cut<true><<<grid, 256, 0, st>>>(g, pt.col_start, pt.ncol, pt.kb0, pt.nkb, B.nkb, mod_stride, sc, mods, v, out);
+      else
+        k_dm_cut<false><<<grid, 256, 0, st>>>(g, pt.col_start, pt.ncol, pt.kb0, pt.nkb, B.nkb, mod_stride, sc, mods, v, out);
+      ISCSI_COUNT_LAUNCH();
+    }
+  }
+  ISCSI_CUDA(cudaGetLastError());
+  return kOk;
+}
+
 int density_run(Context& ctx, const double* bra, const double* ket, double* d1, double* d2) {
   cudaStream_t st = stream();
   const bool sym = (ket == nullptr || ket == bra);
@@ -669,21 +990,64 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
     ISCSI_TRY(plan_build(ctx));
     Pp = ctx.dm;
     DensityPlan& P = *Pp;
-    if (!sym && !P.sl_ket.p && P.sl_elems) {
-      ISCSI_TRY(P.sl_ket.alloc(sizeof(__nv_bfloat16) * P.sl_elems));
-      ISCSI_TRY(P.ex_ket.alloc(sizeof(int) * P.ex_elems));
-      ISCSI_CUDA(cudaMemsetAsync(P.ex_ket.p, 0, sizeof(int) * P.ex_elems, st));
+    if (!P.res_fail) {
+      const int rc = residues_build(ctx, sym);
+      if (rc == kErrNoMem) {
+        P.res_fail = true;
+        for (DevBuf* d : {&P.res_bra, &P.res_ket, &P.res_out}) d->release();
+        cudaGetLastError();
+      } else {
+        ISCSI_TRY(rc);
+      }
     }
-    if (sym ? !P.sym_ready : !P.gen_ready) ISCSI_TRY(build_job(ctx, sym));
-    ISCSI_TRY(cut_operands(ctx, bra, P.sl_bra.as<__nv_bfloat16>(), P.ex_bra.as<int>(), st));
-    if (!sym) ISCSI_TRY(cut_operands(ctx, ket, P.sl_ket.as<__nv_bfloat16>(), P.ex_ket.as<int>(), st));
-    const OzJob& job = sym ? P.job_sym : P.job_gen;
-    if (job.tiles > 0) {
-      const bool ev = !ctx.capturing;
-      if (ev) ISCSI_CUDA(cudaEventRecord(P.ev[0], st));
-      ISCSI_TRY(oz_job_launch(ctx, job, st));
-      if (ev) ISCSI_CUDA(cudaEventRecord(P.ev[1], st));
-      P.timed = ev;
+    const bool res = !P.res_fail;
+    const bool ev = !ctx.capturing;
+    if (res) {
+      ISCSI_TRY(residues_cut(ctx, bra, 0, st));
+      if (!sym) ISCSI_TRY(residues_cut(ctx, ket, 1, st));
+      const CrtJob& job = P.res_job[sym ? 0 : 1];
+      if (job.grid > 0) {
+        ISCSI_TRY(tc_err_buf(ctx));
+        if (ev) ISCSI_CUDA(cudaEventRecord(P.ev[0], st));
+        ISCSI_TRY(job.launch(ctx.oz_err.as<int>(), st));
+        if (ev) ISCSI_CUDA(cudaEventRecord(P.ev[1], st));
+        P.timed = ev;
+      }
+      static const CrtWeights weights = crt_make_weights(kDmMods, 1);
+      DmRebuild D;
+      D.tile0[0] = 0;
+      for (int b = 0; b < 3; ++b) {
+        const DmBlock& B = P.blk[b];
+        const bool some = !B.parts.empty();
+        D.res[b] = P.res_out.as<int16_t>() + P.res_out_off[b];
+        D.q[b] = P.q.as<double>() + B.q_off;
+        D.R[b] = some ? B.R : 0;
+        D.tn[b] = some ? B.R256 / CRT_MAXN : 1;
+        D.tile0[b + 1] = D.tile0[b] + (some ? (rup(B.R, CRT_BM) / CRT_BM) * D.tn[b] : 0);
+      }
+      if (D.tile0[3] > 0) {
+        const int* sc = P.scale.as<int>();
+        k_dm_rebuild<<<dim3(D.tile0[3], CRT_MAXN / 64), 256, 0, st>>>(D, sym ? 1 : 0, sc, sc + (sym ? 0 : 1), weights);
+        ISCSI_COUNT_LAUNCH();
+      }
+      ISCSI_CUDA(cudaGetLastError());
+    } else {
+      ISCSI_TRY(slices_alloc(P));
+      if (!sym && !P.sl_ket.p && P.sl_elems) {
+        ISCSI_TRY(P.sl_ket.alloc(sizeof(__nv_bfloat16) * P.sl_elems));
+        ISCSI_TRY(P.ex_ket.alloc(sizeof(int) * P.ex_elems));
+        ISCSI_CUDA(cudaMemsetAsync(P.ex_ket.p, 0, sizeof(int) * P.ex_elems, st));
+      }
+      if (sym ? !P.sym_ready : !P.gen_ready) ISCSI_TRY(build_job(ctx, sym));
+      ISCSI_TRY(cut_operands(ctx, bra, P.sl_bra.as<__nv_bfloat16>(), P.ex_bra.as<int>(), st));
+      if (!sym) ISCSI_TRY(cut_operands(ctx, ket, P.sl_ket.as<__nv_bfloat16>(), P.ex_ket.as<int>(), st));
+      const OzJob& job = sym ? P.job_sym : P.job_gen;
+      if (job.tiles > 0) {
+        if (ev) ISCSI_CUDA(cudaEventRecord(P.ev[0], st));
+        ISCSI_TRY(oz_job_launch(ctx, job, st));
+        if (ev) ISCSI_CUDA(cudaEventRecord(P.ev[1], st));
+        P.timed = ev;
+      }
     }
     // expansion: slot 0 = aa, 1 = ab, 2 = bb (d2's block order)
     const int slot_of_plan[3] = {1, 0, 2};
@@ -697,14 +1061,14 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
     }
     E.pp_row[0] = P.pp_row[0].as<int>();
     E.pp_row[1] = P.pp_row[1].as<int>();
-    if (sym)
+    if (sym && !res)
       for (int b = 0; b < 3; ++b) {
         const DmResult& R = E.blk[b];
         if (R.R == 0) continue;
         dim3 grid((R.R + 31) / 32, (R.R + 31) / 32);
         k_dm_mirror<<<grid, 256, 0, st>>>(R, const_cast<double*>(R.q)); ISCSI_COUNT_LAUNCH();
       }
-    k_dm_expand<<<dim3(n * n, 3), 256, 0, st>>>(E, d2, d1); ISCSI_COUNT_LAUNCH();
+    k_dm_expand<<<dim3(n * n, 3), 256, 2 * n * sizeof(int), st>>>(E, d2, d1); ISCSI_COUNT_LAUNCH();
     ISCSI_CUDA(cudaGetLastError());
   }
   if (d1) {

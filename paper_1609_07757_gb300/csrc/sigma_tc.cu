@@ -268,7 +268,7 @@ static int tc_attr() {
   return kOk;
 }
 
-static int tc_err_buf(Context& ctx) {
+int tc_err_buf(Context& ctx) {
   if (ctx.oz_err.p) return kOk;
   ISCSI_TRY(ctx.oz_err.alloc(sizeof(int)));
   ISCSI_CUDA(cudaMemsetAsync(ctx.oz_err.p, 0, sizeof(int), stream()));

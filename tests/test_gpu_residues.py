@@ -98,3 +98,29 @@ def test_residues_extreme_vectors(what):
         assert not s.any()
     else:
         check(s, ref)
+
+
+# n, na, nb, kmax, transition: one tile, a tile and a remainder, classes that end inside a tile, one electron
+# of a spin, K of less than one block and of several chunks
+@pytest.mark.parametrize("n,na,nb,k,transition", [(16, 2, 2, 4, False), (17, 2, 2, 4, True), (19, 2, 2, 3, False),
+                                                  (20, 2, 2, 2, True), (24, 2, 1, 3, False), (9, 4, 3, 7, True),
+                                                  (8, 3, 3, 6, False)])
+def test_density_residues(n, na, nb, k, transition):
+    """Bar: 1e-12 of the block's largest element.  A coefficient's unit is 2^-57 of the vector's 2-norm and
+    an element sums K products, so its error is below 2^-57 sqrt(K) of |bra| |ket| over the mean element,
+    under 1e-14 of the largest one for these sizes."""
+    h1, eri = make_integrals(n, 40 + n, ell=3.0, nchol=6)
+    L.iscsi_init(n, na, nb, k, h1, eri, 0.0)
+    nd = L.iscsi_ndet()
+    bra = unit_vector(nd, 5) * 3e-150
+    ket = unit_vector(nd, 6) * 7e120 if transition else bra
+    bra[::7] *= 1e-9
+    b = torch.as_tensor(bra, device="cuda")
+    c = torch.as_tensor(ket, device="cuda") if transition else None
+    d1 = torch.full((2, n, n), float("nan"), dtype=torch.float64, device="cuda")
+    d2 = torch.full((3, n, n, n, n), float("nan"), dtype=torch.float64, device="cuda")
+    L.iscsi_density(b, c, d1, d2)
+    from oracle import Oracle
+    r1, r2 = Oracle(n, na, nb, k, 0.0, h1, eri).density(bra, ket)
+    for got, ref in [(d1.cpu().numpy(), np.asarray(r1))] + list(zip(d2.cpu().numpy(), np.asarray(r2))):
+        assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
