@@ -187,27 +187,32 @@ __global__ void __launch_bounds__(kVecThreads) k_tsdots(const double* __restrict
   // operations per clock per SM: 18 us of a 2025-determinant product)
   __shared__ double red[kVecThreads / 32][kDotT * NB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int V = kDotT * NB;                   // values, and values rounded up to 32
-  constexpr int VP = (V + 31) / 32 * 32;
+  constexpr int V = kDotT * NB;                                     // values, rounded up to a power of two
+  constexpr int VP = V <= 8 ? 8 : V <= 16 ? 16 : V <= 32 ? 32 : 64;
+  static_assert(V <= 64, "values per tile");
+  constexpr int VL = VP / 32 > 0 ? VP / 32 : 1;                     // values a lane ends with
   double x[VP];
 #pragma unroll
   for (int t = 0; t < VP; ++t) x[t] = t < V ? df_value(acc[(t < V ? t : 0) / NB][(t < V ? t : 0) % NB]) : 0.0;
+  int v0 = 0;                                                       // the first of them
 #pragma unroll
-  for (int o = 16, n = VP; o; o >>= 1, n >>= 1) {
+  for (int o = 16, n = VP; o; o >>= 1, n = n > 1 ? n >> 1 : 1) {
     const bool up = (lane & o) != 0;
+    if (n == 1) {  // (compile-time) all values handed out: the lanes left add the same one
+      x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+      continue;
+    }
+    if (up) v0 += n / 2;
 #pragma unroll
     for (int t = 0; t < n / 2; ++t) {
       const double give = up ? x[t] : x[t + n / 2], keep = up ? x[t + n / 2] : x[t];
       x[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
     }
   }
-  // lane l holds the sums of values base(l) .. base(l) + VP / 32 - 1
+  if (VP >= 32 || (lane & (32 / (VP < 32 ? VP : 32) - 1)) == 0)
 #pragma unroll
-  for (int t = 0; t < VP / 32; ++t) {
-    const int v = (lane >> 4 & 1) * (VP / 2) + (lane >> 3 & 1) * (VP / 4) + (lane >> 2 & 1) * (VP / 8) +
-                  (lane >> 1 & 1) * (VP / 16) + (lane & 1) * (VP / 32) + t;
-    if (v < V) red[warp][v] = x[t];
-  }
+    for (int t = 0; t < VL; ++t)
+      if (v0 + t < V) red[warp][v0 + t] = x[t];
   __syncthreads();
   if (threadIdx.x < V) {
     double y = 0.0;
@@ -627,6 +632,195 @@ __global__ void k_dav_request_restart(DavCtl* __restrict__ ctl, int nkeep) {
   }
 }
 
+constexpr int kEighRefine = 48;  // largest order whose refinement arrays are given shared memory
+
+// Eigenvectors X (m x m, shared memory) of the symmetric A by FP32 Jacobi sweeps and FP64
+// refinement; false when they did not get there (close or equal eigenvalues): the
+// caller rotates in FP64 then.
+//
+// The sweeps run on A - mu in FP32: at order 24, 20 to 35 us where FP64 rotations, at 64
+// cycles per warp operation, take 150; a refinement step takes 10.  Each refinement step is the one of Ogita and
+// Aishima ("Iterative refinement for symmetric eigenvalue decomposition", Japan J.
+// Indust. Appl. Math. 35, 2018, Algorithm 1): R = I - X^T X, T = X^T A X in FP64,
+// lambda_i = T_ii / (1 - R_ii), E_ij = (T_ij + lambda_j R_ij) / (lambda_j - lambda_i),
+// E_ii = R_ii / 2, X <- X + X E.  It squares the error, so the step whose
+// corrections are below 3e-9 is the last (1e-17 is left).  E enters to FP32's
+// seven digits of itself: the next step takes what that leaves, and the last one's is 2e-16.
+// A is the warm-started matrix: diagonal but for its rows from m0 on, so A X costs
+// 2 (m - m0) products per element, and the step m^3 (the upper triangles of X^T X and
+// X^T A X).
+// AX, RT: m x m work (RT: T above and on the diagonal, R below); Xf (one), Ff (two): FP32 work
+// of m rows of m | 1.
+__device__ __forceinline__ bool eigh_refined(const double* A, int m, int m0, double* X, double* AX, double* RT, float* Xf, float* Ff,
+                             double* lam) {
+  __shared__ double rdiag[kEighRefine];
+  __shared__ float fred[8];
+  __shared__ unsigned emax_s;
+  const int tid = threadIdx.x, nt = blockDim.x, mm = m * m, warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
+  // FP32 matrix, shifted by the middle of the diagonal's ends and scaled by its norm, odd row stride
+  const int ld = m | 1;
+  float inv;
+  {
+    const double mu = 0.5 * (A[0] + A[mm - 1]);
+    float tot = 0.0f;
+    for (int t = tid; t < mm; t += nt) {
+      const int i = t / m, j = t - i * m;
+      const float a = (float)(i == j ? A[t] - mu : A[t]);
+      tot = fmaf(a, a, tot);
+      Ff[i * ld + j] = a;
+      Xf[i * ld + j] = i == j ? 1.0f : 0.0f;
+    }
+    for (int o = 16; o; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (lane == 0) fred[warp] = tot;
+    __syncthreads();
+    tot = 0.0f;
+    for (int w = 0; w < nw; ++w) tot += fred[w];
+    inv = rsqrtf(tot);  // an infinity or NaN when the scale is outside FP32: no step passes then
+  }
+  // Rotations.  Lane i of every warp has pair i and takes its angle from the old matrix, so all warps know
+  // the round's angles without an exchange; warp w turns the blocks (i, j), j = w, w + 8, ..
+  // from the old into the new matrix and the rows w, w + 8, .. of the vectors: one
+  // synchronisation per round, none for a round without rotations.
+  const int me = m + (m & 1), npair = me / 2;
+  const float thr = 2e-7f * (1.0f / inv);
+  int cur = 0;
+  for (int sweep = 0; sweep < 6; ++sweep) {
+    int any = 0;
+    for (int i = warp; i < m; i += nw)
+      for (int j = lane; j < i; j += 32) any |= fabsf(Ff[cur + i * ld + j]) > thr ? 1 : 0;
+    if (!__syncthreads_or(any)) break;
+    for (int r = 0; r < me - 1; ++r) {
+      int p = 0, q = 0;
+      float c = 1.0f, s = 0.0f;
+      const float* O = Ff + cur;
+      if (lane < npair) {
+        int a = lane - 1 + r, b = me - 2 - lane + r;
+        a = lane == 0 ? 0 : (a >= me - 1 ? a - (me - 1) : a) + 1;
+        b = (b >= me - 1 ? b - (me - 1) : b) + 1;
+        p = min(a, b);
+        q = max(a, b);
+        if (q < m) {
+          const float apq = O[p * ld + q];
+          if (fabsf(apq) > thr) {
+            const float tau = __fdividef((O[q * ld + q] - O[p * ld + p]) * inv, 2.0f * apq * inv);
+            const float t = copysignf(__fdividef(1.0f, fabsf(tau) + sqrtf(fmaf(tau, tau, 1.0f))), tau);
+            c = rsqrtf(fmaf(t, t, 1.0f));
+            s = t * c;
+          }
+        }
+      }
+      if (!__any_sync(0xffffffffu, s != 0.0f)) continue;
+      float* N = Ff + (m * ld - cur);
+      for (int j = warp; j < npair; j += nw) {
+        const float cj = __shfl_sync(0xffffffffu, c, j), sj = __shfl_sync(0xffffffffu, s, j);
+        const int u = __shfl_sync(0xffffffffu, p, j), v = __shfl_sync(0xffffffffu, q, j);
+        if (lane > j) continue;
+        const bool hq = q < m, hv = v < m;
+        const float b11 = O[p * ld + u], b12 = hv ? O[p * ld + v] : 0.0f, b21 = hq ? O[q * ld + u] : 0.0f,
+                    b22 = hq && hv ? O[q * ld + v] : 0.0f;
+        const float r11 = c * b11 - s * b21, r12 = c * b12 - s * b22;
+        const float r21 = s * b11 + c * b21, r22 = s * b12 + c * b22;
+        const float x11 = cj * r11 - sj * r12, x22 = sj * r21 + cj * r22;
+        float x12 = sj * r11 + cj * r12, x21 = cj * r21 - sj * r22;
+        if (lane == j) x12 = x21 = 0.5f * (x12 + x21);
+        N[p * ld + u] = N[u * ld + p] = x11;
+        if (hv) N[p * ld + v] = N[v * ld + p] = x12;
+        if (hq && lane != j) N[q * ld + u] = N[u * ld + q] = x21;
+        if (hq && hv) N[q * ld + v] = N[v * ld + q] = x22;
+      }
+      if (s != 0.0f)
+        for (int row = warp; row < m; row += nw) {
+          const float yp = Xf[row * ld + p], yq = Xf[row * ld + q];
+          Xf[row * ld + p] = c * yp - s * yq;
+          Xf[row * ld + q] = s * yp + c * yq;
+        }
+      cur = m * ld - cur;
+      __syncthreads();
+    }
+  }
+  __syncthreads();
+  for (int t = tid; t < mm; t += nt) {
+    const int i = t / m;
+    X[t] = (double)Xf[i * ld + t - i * m];
+  }
+  __syncthreads();
+  float* Ef = Ff;
+  const int pairs = m * (m + 1) / 2;
+  for (int step = 0; step < 5; ++step) {
+    for (int t = tid; t < mm; t += nt) {
+      const int i = t / m, j = t - i * m;
+      double a = 0.0;
+      if (i < m0) {
+        a = A[i * m + i] * X[t];
+        for (int l = m0; l < m; ++l) a = fma(A[i * m + l], X[l * m + j], a);
+      } else {
+        for (int l = 0; l < m; ++l) a = fma(A[i * m + l], X[l * m + j], a);
+      }
+      AX[t] = a;
+    }
+    if (tid == 0) emax_s = 0u;
+    __syncthreads();
+    for (int t = tid; t < pairs; t += nt) {
+      // t = j (j + 1) / 2 + i, i <= j
+      int j = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+      if ((j + 1) * (j + 2) / 2 <= t) ++j;
+      if (j * (j + 1) / 2 > t) --j;
+      const int i = t - j * (j + 1) / 2;
+      double x = i == j ? -1.0 : 0.0, a = 0.0;
+      for (int l = 0; l < m; ++l) {
+        const double xi = X[l * m + i];
+        x = fma(xi, X[l * m + j], x);
+        a = fma(xi, AX[l * m + j], a);
+      }
+      RT[i * m + j] = a;
+      if (i == j) {
+        rdiag[i] = -x;
+        lam[i] = fma(a, -x * fma(-x, 1.0 - x, 1.0), a);  // a / (1 - r), r = -x
+      } else {
+        RT[j * m + i] = -x;
+      }
+    }
+    __syncthreads();
+    float em = 0.0f;
+    for (int t = tid; t < mm; t += nt) {
+      const int i = t / m, j = t - i * m;
+      float e;
+      if (i == j) {
+        e = (float)(0.5 * rdiag[i]);
+      } else {
+        const int lo = min(i, j), hi = max(i, j);
+        const double num = fma(lam[j], RT[hi * m + lo], RT[lo * m + hi]);
+        e = __fdividef((float)num * inv, (float)(lam[j] - lam[i]) * inv);
+      }
+      Ef[t] = e;
+      em = fabsf(e) <= em ? em : fabsf(e);  // (a NaN stays)
+      if (!(em < 3e38f)) em = 3e38f;
+    }
+    em = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(em)));
+    if ((tid & 31) == 0) atomicMax(&emax_s, __float_as_uint(em));
+    __syncthreads();
+    const float emax = __uint_as_float(emax_s);
+    if (!(emax < 0.03f)) return false;
+    for (int t = tid; t < mm; t += nt) {
+      const int i = t / m, j = t - i * m;
+      float d = 0.0f;
+      for (int l = 0; l < m; ++l) d = fmaf(Xf[i * ld + l], Ef[l * m + j], d);
+      X[t] += (double)d;
+    }
+    if (emax < 3e-9f) {
+      __syncthreads();
+      return true;
+    }
+    __syncthreads();
+    for (int t = tid; t < mm; t += nt) {
+      const int i = t / m;
+      Xf[i * ld + t - i * m] = (float)X[t];
+    }
+    __syncthreads();
+  }
+  return false;
+}
+
 // Symmetric eigen-decomposition of S[0:m][0:m] by cyclic Jacobi rotations
 // (Golub & Van Loan, "Matrix Computations", Sec. 8.5) in the parallel
 // round-robin order of Brent and Luk: each round rotates m/2 disjoint (p, q)
@@ -647,47 +841,98 @@ __global__ void k_dav_request_restart(DavCtl* __restrict__ ctl, int nkeep) {
 //     two Newton steps, so that the rotation is orthogonal to FP64 rounding;
 //   * a thread turns a 2 x 2 block (rows of pair i, columns of pair j >= i) from
 //     both sides and writes its mirror image: half the products, one pass.
-// Basis of 12 to 24, two roots: 330 -> 228 us on average.
+// Basis of 12 to 24, two roots: 330 -> 228 us on average.  Up to order kEighRefine the rotations
+// run in FP32 and the vectors are refined (eigh_refined): 228 -> 66 us; the FP64 rotations
+// below then only serve what that leaves.
 __global__ void __launch_bounds__(256) k_dav_eigh(DavCtl* __restrict__ ctl, const double* __restrict__ S, int lds,
                                                   double* gA, double* gQ, double* Y, int ldy,
-                                                  double* theta_all, int use_smem) {
+                                                  double* theta_all, int use_smem, int refine) {
   extern __shared__ double dyn[];
   __shared__ double cs[192], sn[192];
-  __shared__ int pp[192], qq[192];
+  __shared__ int pp[192], qq[192], order[384];
   __shared__ double red[8], thr_s, inv_s;
   const int m = ctl->m, m0 = ctl->m_eig > 0 && ctl->m_eig <= m ? ctl->m_eig : 0;
   double* A = use_smem ? dyn : gA;
   double* Q = use_smem ? dyn + m * m : gQ;
   const int me = m + (m & 1);
   const int npair = me / 2;
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    const int i = t / m, j = t % m;
-    double a;
-    if (i < m0 && j < m0) {
-      a = i == j ? theta_all[i] : 0.0;
-    } else if (i < m0 || j < m0) {
-      const int o = min(i, j), x = max(i, j);  // old vector o, new row x
-      a = 0.0;
-      for (int l = 0; l < m0; ++l) a = fma(Y[(long long)l * ldy + o], S[(long long)l * lds + x], a);
-    } else {
-      a = S[(long long)i * lds + j];
+  bool done = false;
+  // the last eigenvectors and the new columns, read once (refine: shared memory for them)
+  double* Ys = refine ? dyn + 3 * m * m : nullptr;
+  if (refine) {
+    for (int t = threadIdx.x; t < m0 * m0; t += blockDim.x) Ys[t] = Y[(long long)(t / m0) * ldy + t % m0];
+    for (int t = threadIdx.x; t < m * (m - m0); t += blockDim.x)
+      Q[t] = S[(long long)(t / (m - m0)) * lds + m0 + t % (m - m0)];
+    __syncthreads();
+    const int sub = threadIdx.x & 3;  // four lanes per element between old vector o and new row x
+    for (int t = threadIdx.x >> 2; t < (m0 * (m - m0) + 7) / 8 * 8; t += blockDim.x >> 2) {
+      const bool on = t < m0 * (m - m0);
+      const int o = on ? t / (m - m0) : 0, x = on ? t - o * (m - m0) : 0;
+      double a = 0.0;
+      for (int l = sub; l < m0; l += 4) a = fma(Ys[l * m0 + o], Q[l * (m - m0) + x], a);
+      a += __shfl_xor_sync(0xffffffffu, a, 1);
+      a += __shfl_xor_sync(0xffffffffu, a, 2);
+      if (on && sub == 0) A[o * m + m0 + x] = A[(m0 + x) * m + o] = a;
     }
-    A[t] = a;
-    Q[t] = i < m0 && j < m0 ? Y[(long long)i * ldy + j] : i == j ? 1.0 : 0.0;
+    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+      const int i = t / m, j = t - i * m;
+      if (i < m0 && j < m0) A[t] = i == j ? theta_all[i] : 0.0;
+      else if (i >= m0 && j >= m0) A[t] = Q[i * (m - m0) + j - m0];
+    }
+  } else {
+    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+      const int i = t / m, j = t % m;
+      double a;
+      if (i < m0 && j < m0) {
+        a = i == j ? theta_all[i] : 0.0;
+      } else if (i < m0 || j < m0) {
+        const int o = min(i, j), x = max(i, j);
+        a = 0.0;
+        for (int l = 0; l < m0; ++l) a = fma(Y[(long long)l * ldy + o], S[(long long)l * lds + x], a);
+      } else {
+        a = S[(long long)i * lds + j];
+      }
+      A[t] = a;
+    }
   }
   __syncthreads();
-  {
+  if (refine && m > 1) {
+    double *X = dyn + 2 * m * m, *AX = X + 2 * m * m, *lam = cs;
+    float *Xf = reinterpret_cast<float*>(AX + m * m), *Ff = Xf + m * (m | 1);
+    done = eigh_refined(dyn, m, m0, X, AX, dyn + m * m, Xf, Ff, lam);
+    if (done) {
+      // back from the warm start's vectors
+      for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+        const int i = t / m, j = t - i * m;
+        double a = 0.0;
+        if (i < m0)
+          for (int l = 0; l < m0; ++l) a = fma(Ys[i * m0 + l], X[l * m + j], a);
+        else
+          a = X[t];
+        Q[t] = a;
+        if (i == j) A[t] = lam[i];
+      }
+    }
+    __syncthreads();
+  }
+  double thr = 0.0, inv = 0.0;
+  if (!done) {
     double tot = 0.0;
-    for (int t = threadIdx.x; t < m * m; t += blockDim.x) tot = fma(A[t], A[t], tot);
+    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+      const int i = t / m, j = t - i * m;
+      Q[t] = i < m0 && j < m0 ? Y[(long long)i * ldy + j] : i == j ? 1.0 : 0.0;
+      tot = fma(A[t], A[t], tot);
+    }
     tot = block_sum(tot, red);
     if (threadIdx.x == 0) {
       thr_s = 1e-15 * sqrt(tot) / m;
       inv_s = tot > 0.0 ? 1.0 / sqrt(tot) : 0.0;  // the angles' FP32 sees numbers between 1e-18 and 2
     }
     __syncthreads();
+    thr = thr_s;
+    inv = inv_s;
   }
-  const double thr = thr_s, inv = inv_s;
-  for (int sweep = 0; sweep < 60 && m > 1; ++sweep) {
+  for (int sweep = 0; sweep < 60 && m > 1 && !done; ++sweep) {
     bool any = false;
     for (int r = 0; r < me - 1; ++r) {
       int rot = 0;
@@ -760,16 +1005,26 @@ __global__ void __launch_bounds__(256) k_dav_eigh(DavCtl* __restrict__ ctl, cons
     }
     if (!any) break;
   }
-  // ascending order: rank of each eigenvalue (ties by index)
+  // ascending order: rank of each eigenvalue (ties by index), compared as integers of the same order
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     const double li = A[i * m + i];
+    auto key = [](double x) {
+      const long long b = __double_as_longlong(x);
+      return b < 0 ? b ^ 0x7FFFFFFFFFFFFFFFll : b;
+    };
+    const long long ki = key(li);
     int rank = 0;
     for (int j = 0; j < m; ++j) {
-      const double lj = A[j * m + j];
-      rank += (lj < li) || (lj == li && j < i);
+      const long long kj = key(A[j * m + j]);
+      rank += (kj < ki) || (kj == ki && j < i);
     }
     theta_all[rank] = li;
-    for (int row = 0; row < m; ++row) Y[(long long)row * ldy + rank] = Q[row * m + i];
+    order[i] = rank;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+    const int row = t / m;
+    Y[(long long)row * ldy + order[t - row * m]] = Q[t];
   }
   __syncthreads();
   for (int j = threadIdx.x; j < ctl->k && j < m; j += blockDim.x) ctl->theta[j] = theta_all[j];
@@ -843,7 +1098,9 @@ struct Dav {
     parts = 152 * (int)std::min<long long>(kVecBlocks / 152, std::max<long long>(1, (N + per_wave - 1) / per_wave));
     parts = (int)std::min<long long>(parts, (N + kVecThreads - 1) / kVecThreads);  // no block without elements
     rows_cap = maxsub + k;
-    const int eb = 2 * maxsub * maxsub * (int)sizeof(double);
+    const int eb = maxsub <= kEighRefine
+                       ? maxsub * (5 * maxsub * (int)sizeof(double) + 3 * (maxsub | 1) * (int)sizeof(float))
+                       : 2 * maxsub * maxsub * (int)sizeof(double);
     eig_smem = eb <= 160 * 1024 ? eb : 0;
   }
 
@@ -1017,7 +1274,7 @@ struct Dav {
   // eigen-decomposition of S, Ritz vectors and residuals, convergence check
   int evaluate() {
     k_dav_eigh<<<1, 256, eig_smem, st>>>(ctl, S.as<double>(), maxsub, eigA.as<double>(), eigQ.as<double>(),
-                                         Y.as<double>(), maxsub, thetas.as<double>(), eig_smem ? 1 : 0); ISCSI_COUNT_LAUNCH();
+                                         Y.as<double>(), maxsub, thetas.as<double>(), eig_smem ? 1 : 0, maxsub <= kEighRefine ? 1 : 0); ISCSI_COUNT_LAUNCH();
     ritz();
     k_dav_check<<<1, 32 * kMaxRoots, 0, st>>>(ctl, rr_part.as<double>(), parts); ISCSI_COUNT_LAUNCH();
     ISCSI_CUDA(cudaGetLastError());
