@@ -353,7 +353,7 @@ def run_ours(args, wl, ws, rank, local):
         # FP32 form: 6 of the 9 products of three bf16 terms per operand
         flops = (st["opposite_tc_bf16_flops"] + (st.get("samespin_tc_bf16_flops", 0.0) if both else 0.0)) * 6.0 / 28.0
         peak, peak_src = bf16_peak()
-        bound, kname, kkey = "tensor", "k_tc32w_gemm (tcgen05, FP32-accurate %s, 128 x 128 tiles)" % what, \
+        bound, kname, kkey = "tensor", "k_tc32w_gemm (tcgen05, FP32-accurate %s, 128-row tiles)" % what, \
             "k_tc32w_gemm%s_%s" % (tag, args.workload)
     else:
         flops = st["opposite_gemm_flops"]

@@ -45,6 +45,7 @@ int merge_jobs(MergedJob& mj, const std::vector<const OzJob*>& jobs, const std::
     mj.sh.insert(mj.sh.end(), J.sh.begin(), J.sh.end());
     mj.tiles += J.tiles;
   }
+  if (prec != 64) mj.tiles = t3_tiles(mj.probs, mj.segs, mj.bn);
   ISCSI_TRY(mj.d_probs.grow(sizeof(OzProblem) * std::max<size_t>(1, mj.probs.size())));
   ISCSI_TRY(mj.d_segs.grow(sizeof(OzSeg) * std::max<size_t>(1, mj.segs.size())));
   ISCSI_TRY(mj.d_maps.grow(sizeof(OzMaps) * std::max<size_t>(1, mj.maps.size())));
@@ -74,7 +75,7 @@ int merge_jobs(MergedJob& mj, const std::vector<const OzJob*>& jobs, const std::
 int launch_merged(const MergedJob& mj, int prec, int* err, cudaStream_t st) {
   if (mj.tiles == 0) return kOk;
   return launch_tc_problems(mj.d_probs.as<OzProblem>(), (int)mj.probs.size(), mj.d_segs.as<OzSeg>(),
-                            mj.d_maps.as<OzMaps>(), mj.d_tbases.as<void*>(), mj.tiles, &mj.plan, prec, err, st);
+                            mj.d_maps.as<OzMaps>(), mj.d_tbases.as<void*>(), mj.tiles, mj.bn, &mj.plan, prec, err, st);
 }
 
 struct BatchState {

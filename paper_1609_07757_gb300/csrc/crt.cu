@@ -641,21 +641,10 @@ static void crt_schedule(const std::vector<CrtHostProblem>& probs, int npairs, s
   }
 }
 
-static int crt_sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 2)
-      n = 148;
-  }
-  return n;
-}
-
 int CrtJob::upload(cudaStream_t st) {
   std::vector<CrtItem> items;
   std::vector<int> start;
-  crt_schedule(probs, crt_sm_count() / 2, items, start, flops);
+  crt_schedule(probs, tc_sm_count() / 2, items, start, flops);
   grid = 2 * ((int)start.size() - 1);
   nitems = (int)items.size();
   std::vector<CrtProblem> pr;
@@ -1328,7 +1317,7 @@ int crt_operands(Context& ctx, const double* c, int nvec, int parts) {
     }
     ISCSI_TRY(rc);
   }
-  const int vb = (int)std::min<long long>(2 * crt_sm_count(), (ctx.ndet + 1023) / 1024);
+  const int vb = (int)std::min<long long>(2 * tc_sm_count(), (ctx.ndet + 1023) / 1024);
   k_crt_cmax<<<dim3(vb, nvec), 256, 0, st>>>(c, ctx.ndet, S.ops.cmax); ISCSI_COUNT_LAUNCH();
   k_crt_operands<<<S.ops_blocks, 256, S.ops_smem, st>>>(S.ops, S.mods, c); ISCSI_COUNT_LAUNCH();
   ISCSI_CUDA(cudaGetLastError());

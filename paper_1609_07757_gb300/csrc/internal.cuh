@@ -178,6 +178,7 @@ struct OzJob {
   OzPlan plan;               // FP64-accurate jobs: the persistent launch's schedule
   DevBuf d_probs, d_segs, d_maps;
   int tiles = 0;
+  int bn = 128;              // FP32-form jobs: columns per tile
   int nvec = -1;
   const void* tbase = nullptr;
   long long version = 0;  // bumped at every rebuild (launches over several contexts re-merge)
@@ -368,8 +369,11 @@ const OzJob* both_tc_job(Context& ctx, int prec);  // that combined job (built w
 // table tbases: the FP64-accurate kernel on plan's schedule (prec 64), else
 // the FP32-form kernel over `tiles` tiles
 int launch_tc_problems(const OzProblem* probs, int nprobs, const OzSeg* segs, const OzMaps* maps,
-                       void* const* tbases, int tiles, const OzPlan* plan, int prec, int* err, cudaStream_t st);
+                       void* const* tbases, int tiles, int bn, const OzPlan* plan, int prec, int* err, cudaStream_t st);
+// FP32-form launches: numbers the problems' tiles for the better tile width (bn), returns the tiles
+int t3_tiles(std::vector<OzProblem>& probs, const std::vector<OzSeg>& segs, int& bn);
 int tc_check(Context& ctx);
+int tc_sm_count();
 int tc_err_buf(Context& ctx);  // the context's error word (allocated and cleared when missing)
 int tc_wait_selftest(Context& ctx, long long polls);
 int tc_wait_status(int* err, const char* what);
@@ -454,6 +458,7 @@ struct MergedJob {
   std::vector<long long> ver;
   std::vector<void*> tbases;
   int tiles = 0;
+  int bn = 128;
 };
 // sigma_i = H(ctxs[i]) cs[i] for several contexts, contractions merged
 struct SigmaBatch {

@@ -107,11 +107,11 @@ struct OzSeg {
 };
 
 // TMA descriptors of a segment's two slice arrays: dims (ld, rows, S), box
-// (16, 128 or 64, S), 32-byte swizzle.  Kept in global memory beside the
+// (16, 128 or 64, S) with the 32-byte swizzle, or for the FP32 form (tc32w.cuh)
+// (32, 128, S) with the 64-byte one.  Kept in global memory beside the
 // segment list (one entry per segment; unused for tiled segments).
 struct OzMaps {
   CUtensorMap a, b;
-  CUtensorMap bw;  // B in boxes of 16 x OZ_BW_ROWS rows x all slices (128-column tiles, tc32w.cuh)
 };
 
 // T[M][N] (FP64, ldt) (+)= sum over segments of A_seg B_seg^T; T is the

@@ -262,10 +262,22 @@ static int tc_attr() {
   static bool done = false;
   if (!done) {
     ISCSI_CUDA(cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM_BYTES));
-    ISCSI_CUDA(cudaFuncSetAttribute(k_tc32w_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, T3W_SMEM_BYTES));
+    ISCSI_CUDA(cudaFuncSetAttribute(k_tc32w_gemm<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, T3wShape<128>::SMEM));
+    ISCSI_CUDA(cudaFuncSetAttribute(k_tc32w_gemm<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, T3wShape<256>::SMEM));
     done = true;
   }
   return kOk;
+}
+
+int tc_sm_count() {
+  static int n = 0;
+  if (n == 0) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 2)
+      n = 148;
+  }
+  return n;
 }
 
 int tc_err_buf(Context& ctx) {
@@ -376,9 +388,9 @@ static int add_seg(OzJob& job, const SliceArray& A, int a_row0, int a_k0, const 
   sg.nrows_b = nrows_b;
   OzMaps m;
   std::memset(&m, 0, sizeof(m));
-  if (oz_encode_map(&m.a, A.base, A.ld, A.rows, nslice, A.slice, OZ_BM) ||
-      oz_encode_map(&m.b, B.base, B.ld, B.rows, nslice, B.slice, OZ_BN) ||
-      oz_encode_map(&m.bw, B.base, B.ld, B.rows, nslice, B.slice, OZ_BW_ROWS)) {
+  const bool t3 = nslice == T3_S;  // the FP32 form's kernel reads T3_STAGE_K columns at once, of B 128 rows of a term
+  if (oz_encode_map(&m.a, A.base, A.ld, A.rows, nslice, A.slice, OZ_BM, 0, t3 ? T3_STAGE_K : OZ_BK) ||
+      oz_encode_map(&m.b, B.base, B.ld, B.rows, nslice, B.slice, t3 ? OZ_BW_ROWS : OZ_BN, t3 ? 1 : 0, t3 ? T3_STAGE_K : OZ_BK)) {
     set_error("tensor-core sigma: TMA descriptor rejected");
     return kErrCuda;
   }
@@ -434,6 +446,34 @@ static int add_tiles(std::vector<OzProblem>& probs, int bn = OZ_BN) {
     tiles += (round_up(p.M, OZ_BM) / OZ_BM) * p.tiles_n;
   }
   return tiles;
+}
+
+// Tile width of an FP32-form launch over these problems, which are numbered for it: returns the tiles.
+// Half as many tiles fill the SMs less evenly, so narrow ones win up to one wave of them
+// and just above whole waves of wide ones.  Measured, K = 3584: 152 / 80 tiles 84 us narrow, 119 wide;
+// 171 / 90: 157, 118; 304 / 160: 164, 231; 480 / 240: 309, 239; 784 / 392: 461, 361 (K = 512: 20, 26; 34, 27;
+// 36, 47; 65, 49; 94, 70), which waves x the cycles of a K step below order as they came out.  A segment
+// that reaches only the first half of a wide tile of its problem would move the chunk
+// boundaries of the second half: such lists stay narrow.
+constexpr int kT3Step256 = 850, kT3Step128 = 575;
+int t3_tiles(std::vector<OzProblem>& probs, const std::vector<OzSeg>& segs, int& bn) {
+  bool wide = true;
+  for (const OzProblem& p : probs)
+    for (int g = 0; g < p.seg_count; ++g) {
+      const OzSeg& sg = segs[p.seg_begin + g];
+      if (sg.K > 0 && sg.nrows_b < p.N && round_up(sg.nrows_b, OZ_BW_ROWS) % 256 != 0) wide = false;
+    }
+  const int sms = tc_sm_count();
+  auto waves = [&](int t) { return (t + sms - 1) / sms; };
+  const int narrow_tiles = add_tiles(probs, 128);
+  bn = 128;
+  if (!wide) return narrow_tiles;
+  const int wide_tiles = add_tiles(probs, 256);
+  if (waves(wide_tiles) * kT3Step256 < waves(narrow_tiles) * kT3Step128) {
+    bn = 256;
+    return wide_tiles;
+  }
+  return add_tiles(probs, 128);
 }
 
 // ---------------------------------------------------------------------------
@@ -779,16 +819,22 @@ static int t3_slice_matrix(const V* X, int rows, int cols, long long ld, int tra
 }
 
 // k_tc32w_gemm over a problem list
-static int launch_t3(int tiles, const OzProblem* probs, int nprobs, const OzSeg* segs, const OzMaps* maps,
+static int launch_t3(int tiles, int bn, const OzProblem* probs, int nprobs, const OzSeg* segs, const OzMaps* maps,
                      float* tbase, float* const* tbases, int* err, cudaStream_t st) {
   if (tiles == 0) return kOk;
-  k_tc32w_gemm<<<tiles, T3W_THREADS, T3W_SMEM_BYTES, st>>>(probs, nprobs, segs, maps, tbase, tbases, err); ISCSI_COUNT_LAUNCH();
+  if (bn == 256)
+    k_tc32w_gemm<256><<<tiles, T3wShape<256>::THREADS, T3wShape<256>::SMEM, st>>>(probs, nprobs, segs, maps, tbase,
+                                                                                  tbases, err);
+  else
+    k_tc32w_gemm<128><<<tiles, T3wShape<128>::THREADS, T3wShape<128>::SMEM, st>>>(probs, nprobs, segs, maps, tbase,
+                                                                                  tbases, err);
+  ISCSI_COUNT_LAUNCH();
   ISCSI_CUDA(cudaGetLastError());
   return kOk;
 }
 
 static int t3_launch(Context& ctx, const OzJob& job, float* tbase, cudaStream_t st) {
-  return launch_t3(job.tiles, job.d_probs.as<OzProblem>(), (int)job.probs.size(), job.d_segs.as<OzSeg>(),
+  return launch_t3(job.tiles, job.bn, job.d_probs.as<OzProblem>(), (int)job.probs.size(), job.d_segs.as<OzSeg>(),
                    job.d_maps.as<OzMaps>(), tbase, nullptr, ctx.oz_err.as<int>(), st);
 }
 
@@ -841,7 +887,7 @@ int opposite_tc32_operands(Context& ctx, const float* c, float* ttw, int nvec) {
       ISCSI_TRY(add_seg(job, GA, 0, 0, nullptr, CB, 0, 0, nullptr, C.kpad, C.ncols, T3_S));
       job.probs.push_back(P);
     }
-    job.tiles = add_tiles(job.probs, T3W_BN);
+    job.tiles = t3_tiles(job.probs, job.segs, job.bn);
     ISCSI_TRY(upload_job(job, st, false));
     job.nvec = nvec;
     job.tbase = ttw;
@@ -957,7 +1003,7 @@ int samespin_tc32_operands(Context& ctx, const float* c, float* sigma, int nvec)
         }
         if (P.seg_count > 0) job.probs.push_back(P);
       }
-    job.tiles = add_tiles(job.probs, T3W_BN);
+    job.tiles = t3_tiles(job.probs, job.segs, job.bn);
     ISCSI_TRY(upload_job(job, st, false));
     job.nvec = nvec;
   }
@@ -984,7 +1030,7 @@ int samespin_tc32_gemm(Context& ctx, float* sigma) { return t3_launch(ctx, ctx.t
 // The opposite-spin and same-spin problem lists of a context as one list
 // (one launch fills the GPU's waves better than two).  Rebuilt when either
 // source job changed.
-static int build_both(OzJob& both, const OzJob& ab, const OzJob& ss, int bn, cudaStream_t st) {
+static int build_both(OzJob& both, const OzJob& ab, const OzJob& ss, bool fp64, cudaStream_t st) {
   if (both.src_ver[0] == ab.version && both.src_ver[1] == ss.version) return kOk;
   both.probs = ab.probs;
   both.segs = ab.segs;
@@ -998,8 +1044,8 @@ static int build_both(OzJob& both, const OzJob& ab, const OzJob& ss, int bn, cud
   both.maps.insert(both.maps.end(), ss.maps.begin(), ss.maps.end());
   both.sh = ab.sh;
   both.sh.insert(both.sh.end(), ss.sh.begin(), ss.sh.end());
-  both.tiles = add_tiles(both.probs, bn);
-  ISCSI_TRY(upload_job(both, st, bn == OZ_BN));
+  both.tiles = fp64 ? add_tiles(both.probs) : t3_tiles(both.probs, both.segs, both.bn);
+  ISCSI_TRY(upload_job(both, st, fp64));
   both.src_ver[0] = ab.version;
   both.src_ver[1] = ss.version;
   return kOk;
@@ -1008,34 +1054,35 @@ static int build_both(OzJob& both, const OzJob& ab, const OzJob& ss, int bn, cud
 const OzJob* both_tc_job(Context& ctx, int prec) {
   OzJob& both = prec == 64 ? ctx.oz_both : ctx.t3_both;
   if (build_both(both, prec == 64 ? ctx.oz_ab : ctx.t3_ab, prec == 64 ? ctx.oz_ss : ctx.t3_ss,
-                 prec == 64 ? OZ_BN : T3W_BN, stream()) != kOk)
+                 prec == 64, stream()) != kOk)
     return nullptr;
   return &both;
 }
 
 int both_tc_gemm(Context& ctx, double* sigma) {
   cudaStream_t st = stream();
-  ISCSI_TRY(build_both(ctx.oz_both, ctx.oz_ab, ctx.oz_ss, OZ_BN, st));
+  ISCSI_TRY(build_both(ctx.oz_both, ctx.oz_ab, ctx.oz_ss, true, st));
   return launch_job(ctx, ctx.oz_both, sigma, st);
 }
 
 int both_tc32_gemm(Context& ctx, float* sigma) {
   cudaStream_t st = stream();
-  ISCSI_TRY(build_both(ctx.t3_both, ctx.t3_ab, ctx.t3_ss, T3W_BN, st));
+  ISCSI_TRY(build_both(ctx.t3_both, ctx.t3_ab, ctx.t3_ss, false, st));
   return t3_launch(ctx, ctx.t3_both, sigma, st);
 }
 
 // one launch of the FP64-accurate (prec 64) or FP32-form (prec 32) contraction
 // over a device problem list whose relative outputs use the base table tbases
 int launch_tc_problems(const OzProblem* probs, int nprobs, const OzSeg* segs, const OzMaps* maps,
-                       void* const* tbases, int tiles, const OzPlan* plan, int prec, int* err, cudaStream_t st) {
+                       void* const* tbases, int tiles, int bn, const OzPlan* plan, int prec, int* err,
+                       cudaStream_t st) {
   ISCSI_TRY(tc_attr());
   if (prec == 64) {
     if (!plan) return kOk;
     return launch_oz(*plan, probs, segs, maps, nullptr, reinterpret_cast<double* const*>(tbases), err, st);
   }
   if (tiles == 0) return kOk;
-  return launch_t3(tiles, probs, nprobs, segs, maps, nullptr, reinterpret_cast<float* const*>(tbases), err, st);
+  return launch_t3(tiles, bn, probs, nprobs, segs, maps, nullptr, reinterpret_cast<float* const*>(tbases), err, st);
 }
 
 // the same-spin string matrices changed in place: cut the slices prepared so far again

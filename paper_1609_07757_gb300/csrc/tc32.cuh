@@ -21,7 +21,7 @@ namespace iscsi {
 
 constexpr int T3_S = 3;             // bf16 terms per element
 constexpr int T3_BM = 128, T3_BK = 16;
-constexpr int T3_A_SLICE_BYTES = T3_BM * T3_BK * 2;  // 4096
+constexpr int T3_STAGE_K = 32;      // K per TMA box
 constexpr int T3_CHUNK_STEPS = 32;  // K = 512 per tensor-memory chunk
 
 // the three bf16 terms of x, slice s at out[s * slice_stride]

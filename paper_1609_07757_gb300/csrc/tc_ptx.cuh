@@ -110,6 +110,14 @@ TC_DEVI void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t 
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// the same from the low words of two smem_desc_sw64 descriptors (the high word is a constant)
+TC_DEVI void mma_bf16_sw64(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 a, b;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"((512 >> 4) | (1 << 14) | (4 << 29))
+      : "memory");
+}
 // arrive on an mbarrier once all previously issued MMAs of this thread complete
 TC_DEVI void mma_commit(uint32_t mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar) : "memory");
@@ -252,6 +260,14 @@ TC_DEVI unsigned long long add2(unsigned long long a, unsigned long long b) {
 // layout TMA writes for a box whose rows are 128 bytes under
 // CU_TENSOR_MAP_SWIZZLE_128B): 8-row groups 1024 bytes apart; the 16-deep K
 // steps inside the 128-byte row start 32 bytes apart.
+TC_DEVI uint64_t smem_desc_sw64(uint32_t saddr) {
+  uint64_t d = (uint64_t)((saddr & 0x3FFFF) >> 4);
+  d |= (uint64_t)1 << 16;             // leading byte offset: unused for this layout
+  d |= (uint64_t)(512 >> 4) << 32;    // stride byte offset
+  d |= (uint64_t)1 << 46;             // descriptor version
+  d |= (uint64_t)4 << 61;             // swizzle mode: 64 bytes
+  return d;
+}
 TC_DEVI uint64_t smem_desc_sw128(uint32_t saddr) {
   uint64_t d = (uint64_t)((saddr & 0x3FFFF) >> 4);
   d |= (uint64_t)1 << 16;             // leading byte offset: unused for this layout
