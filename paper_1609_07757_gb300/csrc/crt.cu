@@ -258,8 +258,8 @@ __device__ __forceinline__ double crt_lift_value(const CrtLiftView& L, int qs, c
   if (ea < 0 || eb < 0) return 0.0;
   const int Bp = eb >> 1;
   if (Bp >= L.lim[q]) return 0.0;
-  const double x = cv[L.off[q] + Bp];
-  return ((ea ^ eb) & 1) ? -x : x;
+  // (the sign by the integer units: a negation on the FP64 pipe takes 64 cycles a warp)
+  return __longlong_as_double(__double_as_longlong(cv[L.off[q] + Bp]) ^ ((long long)((ea ^ eb) & 1) << 63));
 }
 
 // Blocks of lift columns first (eight warps: one, two, four or eight per
@@ -791,8 +791,11 @@ static FoldShape fold_shape(const Context& ctx, const CrtState& S, int lev) {
   f.hole = f.base1 + (ctx.n - nob) * f.stride1;
   const long long units = 8ll * (f.hole / 8 + 8);
   const int together = ctx.na * ctx.nb <= 25 ? ctx.na : 1;  // (at most 26 residues per pass: sums below 2^64)
+  // two blocks per SM (113 KB) before all holes in one pass: 4 + 4 electrons in 16 orbitals 182 KB in one
+  // pass 710 us, 91 KB in two passes 545; but one hole per pass is slower (CISDT, 100 orbitals: 302 against 279)
   const struct { int ni, nbuf; long long limit; } tries[] = {
-      {together, 4, 56 * 1024}, {together, 3, 75 * 1024}, {together, 2, kFoldMaxSmem}, {1, 2, kFoldMaxSmem}};
+      {together, 4, 56 * 1024}, {together, 3, 75 * 1024}, {together, 2, 113 * 1024},
+      {(together + 1) / 2, 2, together > 2 ? 113 * 1024 : 0}, {together, 2, kFoldMaxSmem}, {1, 2, kFoldMaxSmem}};
   for (const auto& t : tries) {
     const long long b = t.ni * (t.nbuf * 2ll * f.hole + units);
     if (b <= t.limit) {
