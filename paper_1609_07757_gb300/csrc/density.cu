@@ -26,7 +26,7 @@
 // slices of ozaki.cuh instead.
 // An expansion kernel writes the n^4 tensors from the pair-indexed results.
 // d1 comes from d2's partial trace when d2 is computed for that spin (sum_r
-// d2_ss[p,q,r,r] = (N_s - 1) d1_s[p,q], summed by the expansion kernel), else
+// d2_ss[p,q,r,r] = (N_s - 1) d1_s[p,q]), else
 // from a direct kernel over the one-hole strings.
 #include <algorithm>
 #include <climits>
@@ -328,13 +328,25 @@ struct DmGather {
   const int8_t* alevel;
   const int* nballow;
   const long long* off;
+  unsigned div_mul;               // 2^div_shift / nholeB rounded up
+  int div_shift;
 };
+
+// xy / nholeB for 0 <= xy < 2^31 by one wide product (div_mul, div_shift of gather_of)
+__device__ __forceinline__ int dm_div(const DmGather& g, int xy) {
+  return (int)(((unsigned long long)(unsigned)xy * g.div_mul) >> g.div_shift);
+}
+
+// x, or -x when bit 0 of neg is set, on the integer units (a negation by the FP64 pipe takes 64 cycles a warp)
+__device__ __forceinline__ double dm_signed(double x, int neg) {
+  return __longlong_as_double(__double_as_longlong(x) ^ ((long long)(neg & 1) << 63));
+}
 
 __device__ __forceinline__ double dm_value(const DmGather& g, int col, int row, const double* __restrict__ c) {
   int A, B, neg;
   if (g.kind == 0) {
     int xy = g.hp_inv[col];
-    int X = xy / g.nholeB, Y = xy - X * g.nholeB;
+    int X = dm_div(g, xy), Y = xy - X * g.nholeB;
     int qt = g.pair_of[row];
     int q = qt / g.n, t = qt - q * g.n;
     int ea = g.liftA[q * g.nholeA + X], eb = g.liftB[t * g.nholeB + Y];
@@ -351,8 +363,7 @@ __device__ __forceinline__ double dm_value(const DmGather& g, int col, int row, 
     neg = e & 1;
   }
   if (B >= g.nballow[g.alevel[A]]) return 0.0;
-  double x = c[g.off[A] + B];
-  return neg ? -x : x;
+  return dm_signed(c[g.off[A] + B], neg);
 }
 
 // One block per row of L (rows_pad rows, ld columns): gathers the row once
@@ -376,13 +387,12 @@ __device__ __forceinline__ double dm_row_value(const DmGather& g, const DmStageR
                                                const double* __restrict__ c) {
   if (!STAGED) return dm_value(g, col, row, c);
   const int xy = g.hp_inv[col];
-  const int X = xy / g.nholeB, Y = xy - (xy / g.nholeB) * g.nholeB;
+  const int X = dm_div(g, xy), Y = xy - X * g.nholeB;
   const int ea = S.a[X], eb = S.b[Y];
   if (ea < 0 || eb < 0) return 0.0;
   const int B = eb >> 1;
   if (B >= S.lim[X]) return 0.0;
-  const double x = c[S.off[X] + B];
-  return ((ea ^ eb) & 1) ? -x : x;
+  return dm_signed(c[S.off[X] + B], ea ^ eb);
 }
 
 template <bool STAGED>
@@ -511,10 +521,10 @@ __global__ void __launch_bounds__(256) k_dm_norm(const double* __restrict__ c, l
 // Residues of one part's columns, one block per row of L: 8 consecutive columns
 // per thread (row entries staged as in k_dm_lift_slice).  Rows the part does not
 // reach and padding are zero from the buffer's first clearing on.  26 bytes written per
-// element: full CI in 60 orbitals 495 MB in 206 us (the slices: 187 us), latency of the
-// gathers and the row staging.
+// element: full CI in 60 orbitals 495 MB in 184 us (the slices: 187 us), latency of the
+// gathers and the row staging; five blocks per SM for the staged rows (106 us against 118), four otherwise (78, 92).
 template <bool STAGED>
-__global__ void __launch_bounds__(256) k_dm_cut(DmGather g, int col_start, int ncol, int kb0, int nkb, int nkb_all,
+__global__ void __launch_bounds__(256, STAGED ? 5 : 4) k_dm_cut(DmGather g, int col_start, int ncol, int kb0, int nkb, int nkb_all,
                                                 long long mod_stride, const int* __restrict__ scale,
                                                 const __grid_constant__ CrtMods M, const double* __restrict__ c,
                                                 __nv_bfloat16* __restrict__ out) {
@@ -665,68 +675,68 @@ struct DmExpand {
   const int* pp_row[2];   // aa / bb: {u < v} -> row
 };
 
-// One block per (p, q) and d2 block b writes d2[b][p][q][r][t] for all (r, t): b = 1 (ab)
-// Q[(p,r)][(q,t)], b = 0 (aa) or 2 (bb) s(p,r) s(q,t) Q[{p,r}][{q,t}].  A row's index, a
-// column's index and their signs are taken once per block into shared memory
-// (twice the row, 1 for the sign; -1: no row), so an element costs one read of
-// Q (mostly consecutive in t within a level group) and one store; lanes run over
-// t, a warp over the rows r, eight reads in flight.  3 n^4 stores; n = 60: 157 us
-// (indices and a division per element: 173).
-// A same-spin block's (p, q) block also yields d1_s[p][q] = sum_r d2_ss[p,q,r,r]
-// / (N_s - 1) (written when d1 is given and N_s >= 2).
-__global__ void __launch_bounds__(256) k_dm_expand(DmExpand E, double* __restrict__ d2, double* __restrict__ d1) {
-  extern __shared__ int dm_idx[];
-  const int n = E.n, p = blockIdx.x / n, q = blockIdx.x - (blockIdx.x / n) * n, b = blockIdx.y;
+// One block per (p, r) and d2 block b writes d2[b][p][q][r][t] for all (q, t): b = 1 (ab)
+// Q[(p,r)][(q,t)], b = 0 (aa) or 2 (bb) s(p,r) s(q,t) Q[{p,r}][{q,t}].  A block reads one row
+// of Q, which stays in L1 however the pairs {q,t} jump about in it (blocks over (p, q) read columns
+// t < q of it one sector per element); a warp takes a q, lanes run over t, eight q
+// in flight.  Bound by the 3 n^4 stores; n = 60: 157 us by (p, q), 101 now.
+__global__ void __launch_bounds__(256) k_dm_expand(DmExpand E, double* __restrict__ d2) {
+  const int n = E.n, p = blockIdx.x / n, r = blockIdx.x - (blockIdx.x / n) * n, b = blockIdx.y;
   const long long n2 = (long long)n * n;
-  double* __restrict__ out = d2 + (long long)b * n2 * n2 + (long long)blockIdx.x * n2;
   const bool ab = b == 1 && E.na > 0 && E.nb > 0;
   const bool ss = b != 1 && (b == 0 ? E.na : E.nb) >= 2;
   const DmResult& Q = E.blk[b];
-  for (int i = threadIdx.x; i < 2 * n; i += 256) {
-    const int u = i < n ? p : q, w = i < n ? i : i - n;
-    int x = -1, sg = 0;
-    if (ab) {
-      x = E.pair_index[u * n + w];
-    } else if (ss && u != w) {
-      x = E.pp_row[b == 0 ? 0 : 1][min(u, w) * n + max(u, w)];
-      sg = u < w ? 1 : 0;
-    }
-    dm_idx[i] = x >= 0 && x < Q.R ? 2 * x + sg : -1;
-  }
-  __syncthreads();
+  const int* __restrict__ rows = ab ? E.pair_index : ss ? E.pp_row[b == 0 ? 0 : 1] : nullptr;
+  int x = -1;
+  if (ab) x = rows[p * n + r];
+  else if (ss && p != r) x = rows[min(p, r) * n + max(p, r)];
+  const double* __restrict__ row = x >= 0 && x < Q.R ? Q.q + (long long)x * Q.R : nullptr;
+  double* __restrict__ out = d2 + (((long long)b * n + p) * n2 + r) * n;  // + q n^2 + t
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double tr = 0.0;
-  for (int t = lane; t < n; t += 32) {
-    const int y = dm_idx[n + t];
-    const double* __restrict__ col = Q.q + (y >> 1);
-    for (int r0 = warp; r0 < n; r0 += 64) {
+  const int sx = p < r ? 1 : 0;
+  for (int q0 = warp; q0 < n; q0 += 64)
+    for (int t = lane; t < n; t += 32) {
+      int y[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int q = q0 + 8 * j;
+        const bool on = row && q < n && (ab || q != t);
+        y[j] = on ? __ldg(rows + (ab ? q * n + t : min(q, t) * n + max(q, t))) : -1;
+      }
       long long v[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int r = r0 + 8 * j, x = r < n ? dm_idx[r] : -1;
-        v[j] = x >= 0 && y >= 0
-                   ? __double_as_longlong(__ldg(col + (long long)(x >> 1) * Q.R)) ^ ((long long)((x ^ y) & 1) << 63)
-                   : 0;
-      }
+      for (int j = 0; j < 8; ++j) v[j] = y[j] >= 0 && y[j] < Q.R ? __double_as_longlong(__ldg(row + y[j])) : 0;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const int r = r0 + 8 * j;
-        if (r < n) __stcs(out + r * n + t, __longlong_as_double(v[j]));
-        if (r == t) tr += __longlong_as_double(v[j]);
+        const int q = q0 + 8 * j;
+        if (q >= n) continue;
+        const int sg = ss ? sx ^ (q < t ? 1 : 0) : 0;
+        const long long w = v[j] == 0 ? 0 : v[j] ^ ((long long)sg << 63);
+        __stcs(out + q * n2 + t, __longlong_as_double(w));
       }
     }
+}
+
+// d1_s[p][q] = sum_r d2_ss[p,q,r,r] / (N_s - 1) of a spin with N_s >= 2, a warp per (p, q)
+__global__ void __launch_bounds__(256) k_dm_trace(DmExpand E, double* __restrict__ d1) {
+  const int spin = blockIdx.y;
+  if ((spin == 0 ? E.na : E.nb) < 2) return;
+  const int n = E.n, lane = threadIdx.x & 31;
+  const int pq = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (pq >= n * n) return;
+  const int p = pq / n, q = pq - p * n;
+  const DmResult& Q = E.blk[2 * spin];
+  const int* __restrict__ rows = E.pp_row[spin];
+  double s = 0.0;
+  for (int r = lane; r < n; r += 32) {
+    if (r == p || r == q) continue;
+    const int x = rows[min(p, r) * n + max(p, r)], y = rows[min(q, r) * n + max(q, r)];
+    if (x < 0 || y < 0 || x >= Q.R || y >= Q.R) continue;
+    const double v = Q.q[(long long)x * Q.R + y];
+    s += (p < r) == (q < r) ? v : -v;
   }
-  if (!ss || !d1) return;
-  __shared__ double red[8];
-  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-  if (lane == 0) red[warp] = tr;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sum = 0.0;
-    for (int w = 0; w < 8; ++w) sum += red[w];
-    const int spin = b == 0 ? 0 : 1;
-    d1[(long long)spin * n2 + blockIdx.x] = sum / (double)((spin == 0 ? E.na : E.nb) - 1);
-  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) d1[(long long)spin * n * n + pq] = s / (double)((spin == 0 ? E.na : E.nb) - 1);
 }
 
 // d1_s[p][q] = sum_X s(p,X) s(q,X) sum_O bra[X u p, O] ket[X u q, O] over the
@@ -791,6 +801,11 @@ static DmGather gather_of(const Context& ctx, const DensityPlan& P, int b) {
   g.alevel = ctx.sp[0].level.as<int8_t>();
   g.nballow = ctx.nballow.as<int>();
   g.off = ctx.off.as<long long>();
+  const int d = std::max(1, g.nholeB);
+  int l = 0;
+  while ((1ll << l) < d) ++l;
+  g.div_shift = 31 + l;
+  g.div_mul = (unsigned)(((1ull << (31 + l)) + d - 1) / d);
   return g;
 }
 
@@ -1068,14 +1083,17 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
         dim3 grid((R.R + 31) / 32, (R.R + 31) / 32);
         k_dm_mirror<<<grid, 256, 0, st>>>(R, const_cast<double*>(R.q)); ISCSI_COUNT_LAUNCH();
       }
-    k_dm_expand<<<dim3(n * n, 3), 256, 2 * n * sizeof(int), st>>>(E, d2, d1); ISCSI_COUNT_LAUNCH();
+    k_dm_expand<<<dim3(n * n, 3), 256, 0, st>>>(E, d2); ISCSI_COUNT_LAUNCH();
+    if (d1) {
+      k_dm_trace<<<dim3((n * n + 7) / 8, 2), 256, 0, st>>>(E, d1); ISCSI_COUNT_LAUNCH();
+    }
     ISCSI_CUDA(cudaGetLastError());
   }
   if (d1) {
     for (int s = 0; s < 2; ++s) {
       const int ne = s == 0 ? ctx.na : ctx.nb;
       if (d2 && ne >= 2) {
-        // written by the expansion
+        // k_dm_trace above
       } else if (ne == 0) {
         ISCSI_CUDA(cudaMemsetAsync(d1 + (size_t)s * n * n, 0, sizeof(double) * n * n, st));
       } else {
