@@ -124,3 +124,13 @@ def test_density_residues(n, na, nb, k, transition):
     r1, r2 = Oracle(n, na, nb, k, 0.0, h1, eri).density(bra, ket)
     for got, ref in [(d1.cpu().numpy(), np.asarray(r1))] + list(zip(d2.cpu().numpy(), np.asarray(r2))):
         assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+# four strings' holes beyond the shared memory of half an SM: two holes per pass, without and with runs of levels
+@pytest.mark.parametrize("kmax", [8, 5])
+def test_residues_fold_in_passes(kmax):
+    n = 15
+    h1, eri = make_integrals(n, 7300, ell=4.0, nchol=12)
+    L.iscsi_init(n, 4, 4, kmax, h1, eri, 1e-14)
+    s, ref = both(unit_vector(L.iscsi_ndet(), 3)[None], 1)
+    check(s[0], ref[0])
