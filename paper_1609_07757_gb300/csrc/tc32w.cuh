@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(T3wShape<BN>::THREADS, 1)
       }
       ph ^= 1u;
     }
-    if (abort_s) {
+    if (__any_sync(0xffffffffu, abort_s != 0)) {
       if (tc::elect_one()) tc::mma_commit(tc::smem_u32(&drain_b));
       __syncwarp();
       tc::mbar_wait_bounded(tc::smem_u32(&drain_b), 0, OZ_SPIN);
