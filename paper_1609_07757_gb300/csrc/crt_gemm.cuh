@@ -113,7 +113,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CRT_THREADS, 1)
       int g = 0, st = 0, chunk = 0;
       uint32_t ph = 0;
       bool ok = true;
-      const uint64_t dA0 = tc::smem_desc_sw128(s0), dB0 = tc::smem_desc_sw128(s0 + CRT_A_BYTES);
+      const uint32_t dA0 = (uint32_t)tc::smem_desc_sw128(s0), dB0 = dA0 + (CRT_A_BYTES >> 4);
       for (int it = it0; it < it1 && ok; ++it) {
         const int nkb = __ldg(&items[it].nkb) + __ldg(&items[it].nkbb);
         const uint32_t idesc = tc::idesc_bf16_f32(2 * CRT_BM, __ldg(&items[it].ntile));
@@ -134,12 +134,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CRT_THREADS, 1)
           }
           tc::fence_after_sync();
           if (tc::elect_one()) {
-            const uint64_t off = (uint64_t)(st * (CRT_STAGE_BYTES >> 4));
+            const uint32_t off = (uint32_t)(st * (CRT_STAGE_BYTES >> 4));
             const uint32_t d = tmem + (uint32_t)(buf * CRT_MAXN);
 #pragma unroll
             for (int j = 0; j < CRT_BK / 16; ++j)
-              tc::mma_bf16_pair(d, dA0 + off + (uint64_t)(2 * j), dB0 + off + (uint64_t)(2 * j), idesc,
-                                first && j == 0 ? 0u : 1u);
+              tc::mma_bf16_pair_sw128(d, dA0 + off + 2 * j, dB0 + off + 2 * j, idesc, first && j == 0 ? 0u : 1u);
             tc::mma_commit_pair(tc::smem_u32(&empty_b[st]));
             if (last) tc::mma_commit_pair(tc::smem_u32(&accf_b[buf]));
           }
