@@ -132,14 +132,14 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 
 // Thin problems (N <= 16 columns, e.g. the single allowed beta string of the
 // highest-level CISD block): one warp per output row, lanes split K, the
-// per-column partial sums are reduced with shuffles (of the columns there are: FP64 adds at 64
-// cycles a warp).  The column count is a
-// template parameter so no FMA is spent on absent columns.  All 16 columns reduced and one load in
-// flight per lane took CISD, 100 orbitals (4950 x 4950 by one column, twice) from 675 to 692 us.
+// per-column partial sums are reduced with shuffles, of the columns there are only (an FP64
+// addition takes 64 cycles a warp; all 16 and a serial sum of the chunks in k_mthin_reduce:
+// CISD, 100 orbitals 0.710 ms, 200 orbitals 4.76, now 0.687 and 4.71).  The column count is
+// a template parameter so no FMA is spent on absent columns.  The K loops stay rolled: four to sixteen
+// loads in flight cost occupancy (200 orbitals: 4.87 to 5.02 ms).
 template <typename T, int NB>
 __device__ __forceinline__ void thin_row_seg(T (&acc)[16], const T* __restrict__ Ap, const T* __restrict__ Bp,
                                              int K, long long ldb, int lane) {
-#pragma unroll(NB <= 4 ? 8 : 2)
   for (int k = lane; k < K; k += 32) {
     T a = Ap[k];
     const T* br = Bp + (long long)k * ldb;
@@ -151,7 +151,6 @@ __device__ __forceinline__ void thin_row_seg(T (&acc)[16], const T* __restrict__
 template <typename T, int MB>
 __device__ __forceinline__ void mthin_col_seg(T (&acc)[16], const T* __restrict__ Ap, long long lda,
                                               const T* __restrict__ Bp, long long ldb, int k0, int k1) {
-#pragma unroll(MB <= 4 ? 16 : 4)
   for (int k = k0; k < k1; ++k) {
     T b = Bp[(long long)k * ldb];
 #pragma unroll
@@ -862,7 +861,14 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
   return kOk;
 }
 
+// The slices skip screened blocks of the integrals, the residue products do not.  One sigma,
+// slices / residues, by the share of opposite-spin integrals kept (CISDT in a box): 0.98 3.17 / 1.39 ms,
+// 0.78 16.3 / 8.2, 0.55 50.7 / 38.7; the square of a one-body operator (full CI, 60 orbitals, 0.004)
+// 1.02 / 1.26.  The line through these meets 1 between 0.3 and 0.45.
+constexpr double kCrtMinKept = 0.45;
+
 int crt_parts(Context& ctx, int nvec) {
+  if (ctx.units_opposite_total > 0 && (double)ctx.units_opposite < kCrtMinKept * (double)ctx.units_opposite_total) return 0;
   int parts = 0;
   if (ctx.have_ab && ab_on_tc(ctx, 64) && crt_ab_active(ctx, nvec)) parts |= 1;
   if (ctx.route[0].ss_min <= kThinN && samespin_tc_active(ctx) && crt_ss_active(ctx)) parts |= 2;
