@@ -341,7 +341,15 @@ def run_ours(args, wl, ws, rank, local):
     both = st.get("both_tc_fp%d" % args.precision, 0) == 1
     what = "opposite- and same-spin contractions in one launch" if both else "opposite-spin contraction"
     tag = "_both" if both else ""
-    if tc and args.precision == 64:
+    res = st.get("residues", {})
+    residues = bool(tc and args.precision == 64 and res.get("items", 0) > 0)
+    if residues:
+        # residue numbers: one bf16 product per modulus over whole tiles
+        flops = res["bf16_flops"]
+        peak, peak_src = bf16_peak()
+        bound, kname, kkey = "tensor", "k_crt_gemm (tcgen05 CTA pairs, one bf16 product per modulus, %d moduli)" % (
+            res["moduli"]), "k_crt_gemm_%s" % args.workload
+    elif tc and args.precision == 64:
         # tensor-core kernel: bf16 MMA flops its schedule issues (the exact slice
         # products of live slices of non-screened blocks, over whole tiles)
         flops = st.get("tc_schedule_fp64", {}).get("issued_bf16_flops") or (
@@ -382,7 +390,8 @@ def run_ours(args, wl, ws, rank, local):
         "higher_is_better": True,
         "scaling": "weak",
         "vs_baseline": None,
-        "dtype": ("f64 (tcgen05 bf16 exact slices, int64/f64 accumulation)" if tc else "f64")
+        "dtype": ("f64 (tcgen05 bf16 residues, exact integer sums)" if residues
+                  else "f64 (tcgen05 bf16 exact slices, int64/f64 accumulation)" if tc else "f64")
         if args.precision == 64 else ("f32 (tcgen05, three bf16 terms, f32 accumulation)" if tc else "f32"),
         "data": "synthetic (seeded integrals shaped like the paper's Be-in-a-box sets)",
         "config": {"workload": args.workload, "norb": wl["n"], "nalpha": wl["na"], "nbeta": wl["nb"],
@@ -402,7 +411,8 @@ def run_ours(args, wl, ws, rank, local):
                      "method_tflops": round(2.0 * updates / (gemm_ms * 1e-3) / 1e12, 3) if gemm_ms > 0 else None,
                      "method_frac": round(2.0 * updates / (gemm_ms * 1e-3) / 1e12 / peak, 5) if gemm_ms > 0 else None,
                      "emulation_factor": round(flops / (2.0 * updates), 3) if updates > 0 else None,
-                     "schedule": st.get("tc_schedule_fp64") if (tc and args.precision == 64) else None,
+                     "schedule": res if residues else st.get("tc_schedule_fp64")
+                     if (tc and args.precision == 64) else None,
                      "peak_source": peak_src},
         "hbm": {"compulsory_bytes_per_step": comp_bytes,
                 "achieved_gbs": round(comp_bytes / (ms * 1e-3) / 1e9, 2),
@@ -463,12 +473,12 @@ def run_tau_sweep(L, wl, taus, steps=5, warmup=3):
         L.iscsi_set_option("phase_timing", 0)
         ms = sum(a.elapsed_time(b) for a, b in ev) / steps
         upd = L.iscsi_updates_per_sigma()
-        sched = st.get("tc_schedule_fp64", {})
+        issued = st.get("residues", {}).get("bf16_flops") or st.get("tc_schedule_fp64", {}).get("issued_bf16_flops")
         out.append({"tau": tau, "sigma_ms": round(ms, 4), "gupdates_per_s": round(upd / (ms * 1e-3) / 1e9, 1),
                     "updates_per_sigma": upd,
                     "opposite_units_kept": round(st["units_kept_opposite"] / max(1, st["units_total"]["opposite"]), 6),
                     "contraction_ms": round(st["phase_ms"]["opposite_gemm"] / max(1, st["timed_calls"]), 4),
-                    "issued_bf16_flops": sched.get("issued_bf16_flops")})
+                    "issued_bf16_flops": issued})
         L.iscsi_finalize()
     return out
 
@@ -758,8 +768,9 @@ def run_density(name, steps=10, warmup=3, with_cpu=True, tau=None):
            "contraction_bf16_flops": bf16, "contraction_fp64_flops": fp64,
            "roofline": {"bound": "tensor", "achieved": round(bf16 / (gemm_ms * 1e-3) / 1e12, 4), "peak": peak,
                         "unit": "TFLOP/s", "frac": round(bf16 / (gemm_ms * 1e-3) / 1e12 / peak, 4),
-                        "traffic": profile_traffic("k_oz_gemm_density_%s" % name)[0],
-                        "kernel": "k_oz_gemm<1> (tcgen05, FP64-accurate Gram products of lifted vectors, ket = bra)",
+                        "traffic": profile_traffic("k_crt_gemm_density_%s" % name)[0],
+                        "kernel": "k_crt_gemm (tcgen05 CTA pairs, Gram products of lifted vectors, ket = bra, "
+                                  "one bf16 product per modulus)",
                         "peak_source": peak_src},
            "fp64_equivalent_tflops": round(fp64 / (gemm_ms * 1e-3) / 1e12, 3),
            "output_bytes": 8 * (2 * n * n + 3 * n ** 4), "l2": "flushed between calls", "checks": checks}
@@ -1058,13 +1069,18 @@ def run_gas(name, steps=10, warmup=3, with_cpu=True, projected=True):
     both = st_t.get("both_tc_fp64", 0) == 1
     route = st_t.get("route_fp64", {})
     if st_t.get("fp64_tc", 0) == 1 and route.get("ab_tc", 1) == 1 and gemm_ms > 0:
-        flops = st_t["opposite_tc_bf16_flops"] + (st_t.get("samespin_tc_bf16_flops", 0.0) if both else 0.0)
+        res = st_t.get("residues", {})
+        residues = res.get("items", 0) > 0
+        flops = res["bf16_flops"] if residues else (
+            st_t["opposite_tc_bf16_flops"] + (st_t.get("samespin_tc_bf16_flops", 0.0) if both else 0.0))
         peak, peak_src = bf16_peak()
         ach = flops / (gemm_ms * 1e-3) / 1e12
         roof = {"bound": "tensor", "achieved": round(ach, 4), "peak": peak, "unit": "TFLOP/s",
                 "frac": round(ach / peak, 4),
-                "traffic": profile_traffic("k_oz_gemm%s_gas_%s" % ("_both" if both else "", name))[0],
-                "kernel": "k_oz_gemm (tcgen05, FP64-accurate, %s)" % (
+                "traffic": None if residues else
+                profile_traffic("k_oz_gemm%s_gas_%s" % ("_both" if both else "", name))[0],
+                "kernel": "k_crt_gemm (tcgen05 CTA pairs, one bf16 product per modulus)" if residues else
+                "k_oz_gemm (tcgen05, FP64-accurate, %s)" % (
                     "opposite- and same-spin contractions in one launch" if both else "opposite-spin"),
                 "kernel_ms": round(gemm_ms, 4), "flops_per_launch": flops, "peak_source": peak_src}
     else:
