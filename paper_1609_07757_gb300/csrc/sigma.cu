@@ -132,7 +132,7 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 
 // Thin problems (N <= 16 columns, e.g. the single allowed beta string of the
 // highest-level CISD block): one warp per output row, lanes split K, the
-// per-column partial sums are reduced with shuffles, of the columns there are only (an FP64
+// per-column partial sums are reduced with shuffles, of the columns there are only, in fours (an FP64
 // addition takes 64 cycles a warp; all 16 and a serial sum of the chunks in k_mthin_reduce:
 // CISD, 100 orbitals 0.710 ms, 200 orbitals 4.76, now 0.687 and 4.71).  The column count is
 // a template parameter so no FMA is spent on absent columns.  The K loops stay rolled: four to sixteen
@@ -197,9 +197,12 @@ __global__ void __launch_bounds__(256)
     }
   }
 #pragma unroll
-  for (int n = 0; n < kThinN; ++n) {
-    if (n >= P.N) break;
-    for (int o = 16; o; o >>= 1) acc[n] += __shfl_xor_sync(0xffffffffu, acc[n], o);
+  for (int n0 = 0; n0 < kThinN; n0 += 4) {  // (four columns' chains side by side)
+    if (n0 >= P.N) break;
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+#pragma unroll
+      for (int n = n0; n < n0 + 4; ++n) acc[n] += __shfl_xor_sync(0xffffffffu, acc[n], o);
   }
   T* Cp = const_cast<T*>(resolve(P.c, P.csrc)) + (long long)row * P.ldc;
 #pragma unroll
