@@ -61,27 +61,6 @@ __global__ void k_oz_row_exp(const double* __restrict__ X, int rows, int cols, l
   }
 }
 
-// slices of X into out[s][row][k] (row stride ldo, rows_pad rows, zero padded).
-// Source column of k: colmap[k] (-1: zero) if colmap, else k (zero beyond cols).
-__global__ void k_oz_slice(const double* __restrict__ X, int rows, int cols, long long ld, int trans,
-                           const int* __restrict__ colmap, const int* __restrict__ e,
-                           __nv_bfloat16* __restrict__ out, long long slice_stride, int ldo, int rows_pad) {
-  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long total = (long long)rows_pad * ldo;
-  if (t >= total) return;
-  int r = (int)(t / ldo), k = (int)(t % ldo);
-  int src = colmap ? colmap[k] : (k < cols ? k : -1);
-  double x = 0.0;
-  int ex = 0;
-  if (r < rows && src >= 0) {
-    x = trans ? X[(long long)src * ld + r] : X[(long long)r * ld + src];
-    ex = e[r];
-  }
-  int a[OZ_S];
-  oz_digits(x, ex, a);
-  oz_store_digits(a, out + t, slice_stride);
-}
-
 // Tiled slices of an FP64 matrix, one thread per tiled row r and 8-wide K
 // chunk (8 threads of consecutive rows write one 128-byte run per slice).
 // X(row, k) = X[row * ld + k], or X[k * ld + row] when trans; tiled row r

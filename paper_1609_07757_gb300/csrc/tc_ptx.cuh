@@ -23,12 +23,6 @@ TC_DEVI void cp_async_wait() {
 // generic-proxy shared-memory writes become visible to the tensor core (async proxy)
 TC_DEVI void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
-// arrive on the mbarrier when all earlier cp.async of this thread completed
-// (the barrier's expected count includes this arrival)
-TC_DEVI void cp_async_mbar_arrive(uint32_t mbar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(mbar) : "memory");
-}
-TC_DEVI void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 TC_DEVI void mbar_arrive(uint32_t mbar) {
   asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(mbar) : "memory");
 }
@@ -57,10 +51,6 @@ TC_DEVI void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t m
                "l"(src), "r"(bytes), "r"(mbar)
                : "memory");
 }
-TC_DEVI void prefetch_map(const void* map) {
-  asm volatile("prefetch.tensormap [%0];\n" ::"l"(map) : "memory");
-}
-
 TC_DEVI void mbar_init(uint32_t a, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(a), "r"(count) : "memory");
 }
@@ -144,12 +134,6 @@ TC_DEVI void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 TC_DEVI void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"r"(taddr), "r"(r[0]),
                "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
-// 32 lanes x 8 consecutive 32-bit columns of TMEM set to zero
-TC_DEVI void tmem_zero8(uint32_t taddr) {
-  const uint32_t z = 0u;
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};\n" ::"r"(taddr), "r"(z)
                : "memory");
 }
 TC_DEVI void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
