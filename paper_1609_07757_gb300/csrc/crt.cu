@@ -272,7 +272,8 @@ __global__ void __launch_bounds__(256) k_crt_operands(const __grid_constant__ Cr
                                                       const double* __restrict__ c) {
   extern __shared__ __align__(16) unsigned char crt_dyn[];
   const int nlift = O.blk_start[O.ngroups];
-  if (blockIdx.x == 0 && (int)threadIdx.x < O.nvec) O.cexp[threadIdx.x] = O.cmax[threadIdx.x];
+  if (blockIdx.x == 0)
+    for (int v = threadIdx.x; v < O.nvec; v += 256) O.cexp[v] = O.cmax[v];
   if ((int)blockIdx.x < nlift) {
     int gi = 0;
     while ((int)blockIdx.x >= O.blk_start[gi + 1]) ++gi;
@@ -815,9 +816,10 @@ static FoldShape fold_shape(const Context& ctx, const CrtState& S, int lev) {
 // to fit k_crt_fold's shared memory.
 constexpr int kCrtMinCols = 64;
 constexpr int kCrtMinRows = 16;
+constexpr int kCrtMaxVecs = 65535;  // vectors are a grid dimension of k_crt_cmax and k_crt_fold
 
 bool crt_ab_active(Context& ctx, int nvec) {
-  if (!ctx.have_ab) return false;
+  if (!ctx.have_ab || nvec > kCrtMaxVecs) return false;
   CrtState& S = crt_state(ctx);
   if (S.off || S.groups.empty() || fold_shape(ctx, S, 0).ni == 0) return false;
   double heavy = 0.0, good = 0.0;
@@ -831,9 +833,9 @@ bool crt_ab_active(Context& ctx, int nvec) {
 }
 
 // the same-spin products, all levels at once, when the strings fill a tile or so
-bool crt_ss_active(Context& ctx) {
+bool crt_ss_active(Context& ctx, int nvec) {
   CrtState& S = crt_state(ctx);
-  return !S.off && ctx.sp[0].count >= kCrtMinRows && ctx.sp[1].count >= kCrtMinRows;
+  return !S.off && nvec <= kCrtMaxVecs && ctx.sp[0].count >= kCrtMinRows && ctx.sp[1].count >= kCrtMinRows;
 }
 
 int crt_encode(CrtProblem& P, const void* a, const void* b, int nm) {

@@ -390,7 +390,7 @@ int oz_job_launch(Context& ctx, const OzJob& job, cudaStream_t st);
 // crt.cu: the FP64 contractions through residue numbers.  parts: 1 opposite
 // spin, 2 same spin (all levels); crt_parts: what the current routing sends there
 bool crt_ab_active(Context& ctx, int nvec);
-bool crt_ss_active(Context& ctx);
+bool crt_ss_active(Context& ctx, int nvec);
 int crt_parts(Context& ctx, int nvec);
 int crt_operands(Context& ctx, const double* c, int nvec, int parts);
 int crt_gemm(Context& ctx);

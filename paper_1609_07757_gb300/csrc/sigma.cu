@@ -878,7 +878,7 @@ int crt_parts(Context& ctx, int nvec) {
   // the same-spin part follows the opposite-spin part; alone (a thin column class keeps that one on the
   // slices) it pays while the string matrices are small: CISD, slices / residues, 50 orbitals (1225 strings)
   // 0.219 / 0.189 ms, 70 (2415) 0.307 / 0.308, 100 (4950) 0.66 / 0.69, 150 2.02 / 2.35
-  if (ctx.route[0].ss_min <= kThinN && samespin_tc_active(ctx) && crt_ss_active(ctx) &&
+  if (ctx.route[0].ss_min <= kThinN && samespin_tc_active(ctx) && crt_ss_active(ctx, nvec) &&
       ((parts & 1) || !ctx.have_ab || std::max(ctx.sp[0].count, ctx.sp[1].count) <= kCrtSsAlone))
     parts |= 2;
   return parts;
@@ -988,7 +988,7 @@ int sigma_autotune(Context& ctx, const double* c, double* sigma, int nvec, int p
           same = (rows > q.ss && nba > q.ss) == (rows > ss && nba > ss);
         }
         // the lowest threshold is the residue products (all blocks at once), the others slices
-        if (prec == 64 && crt_ss_active(ctx) && (q.ss == kThinN) != (ss == kThinN)) same = false;
+        if (prec == 64 && crt_ss_active(ctx, nvec) && (q.ss == kThinN) != (ss == kThinN)) same = false;
         if (same) dup = true;
       }
       if (!dup) cands.push_back({ab, ss, route_model_ms(ctx, prec, ab, ss, nvec), -1.0});

@@ -134,3 +134,24 @@ def test_residues_fold_in_passes(kmax):
     L.iscsi_init(n, 4, 4, kmax, h1, eri, 1e-14)
     s, ref = both(unit_vector(L.iscsi_ndet(), 3)[None], 1)
     check(s[0], ref[0])
+
+
+# more vectors than a thread block has threads, in both parts and in the string matrices' part alone (no
+# two-electron part), single and in a batch; sizes over six decades, so that each vector's own exponent counts
+@pytest.mark.parametrize("n,kmax,parts", [(10, 4, 3), (12, 4, 2)])
+@pytest.mark.parametrize("batch", [False, True])
+def test_residues_many_vectors(n, kmax, parts, batch):
+    nvec = 300
+    h1, eri = make_integrals(n, 7400, ell=3.0, nchol=12)
+    L.iscsi_init(n, 2, 2, kmax, h1, eri if parts == 3 else None, 1e-14)
+    nd = L.iscsi_ndet()
+    C = np.stack([unit_vector(nd, 10 + v) * 10.0 ** (v % 7 - 3) for v in range(nvec)])
+    s, ref = both(C, nvec)
+    if batch:
+        c = torch.as_tensor(C, device="cuda")
+        out = torch.full_like(c, float("nan"))
+        L.iscsi_batch_sigma([L.iscsi_ctx_current()], [c], [out], nvec)
+        torch.cuda.synchronize()
+        s = out.cpu().numpy()
+    for v in range(nvec):
+        check(s[v], ref[v])
