@@ -128,7 +128,7 @@ struct ProblemList {
   // problems with at most kThinN rows run one thread per output column
   std::vector<Problem<T>> mthin;
   DevBuf d_mthin, d_part_off, d_part;
-  int mthin_cols = 0;
+  int mthin_cols = 0, mthin_rows = 0;  // columns in all, most rows of a problem
   int mthin_chunks = 1;
   long long mthin_part_stride = 0;
 };

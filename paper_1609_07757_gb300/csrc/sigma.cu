@@ -269,6 +269,9 @@ __global__ void __launch_bounds__(256)
     if (m < P.M) out[(long long)m * P.N + n] = acc[m];
 }
 
+// sigma's elements from the chunks' partial sums, in chunk order; a thread per column and row (grid.y).
+// Bound by the latency of the chunks' loads: eight in flight, rows side by side (a thread per column for all rows:
+// FP32 sigma of 4 + 3 electrons in 10 orbitals, 5 chunks, 139 us; now 121).
 template <typename T>
 __global__ void k_mthin_reduce(const Problem<T>* __restrict__ probs, int nprobs, const long long* __restrict__ part_off,
                                T* sbase, const T* __restrict__ cbase, int total_cols, int nchunks,
@@ -282,17 +285,16 @@ __global__ void k_mthin_reduce(const Problem<T>* __restrict__ probs, int nprobs,
     else hi = mid - 1;
   }
   const Problem<T> P = probs[lo];
-  int n = item - P.tile_begin;
-  T* Cp = (P.csrc == kSrcC ? const_cast<T*>(cbase) + P.c : P.csrc == kSrcSigma ? sbase + P.c
-                                                                              : reinterpret_cast<T*>(P.c)) + n;
-  for (int m = 0; m < P.M; ++m) {
-    T acc = T(0);
-    const T* src = part + part_off[lo] + (long long)m * P.N + n;
+  const int n = item - P.tile_begin, m = blockIdx.y;
+  if (m >= P.M) return;
+  T* dst = (P.csrc == kSrcC ? const_cast<T*>(cbase) + P.c : P.csrc == kSrcSigma ? sbase + P.c
+                                                                               : reinterpret_cast<T*>(P.c)) +
+           n + (long long)m * P.ldc;
+  T acc = T(0);
+  const T* src = part + part_off[lo] + (long long)m * P.N + n;
 #pragma unroll 8
-    for (int c = 0; c < nchunks; ++c) acc += src[c * part_stride];
-    T* dst = Cp + (long long)m * P.ldc;
-    *dst = P.accumulate ? *dst + acc : acc;
-  }
+  for (int c = 0; c < nchunks; ++c) acc += src[c * part_stride];
+  *dst = P.accumulate ? *dst + acc : acc;
 }
 
 template <typename T>
@@ -314,7 +316,7 @@ static int upload_problems(ProblemList<T>& pl, cudaStream_t st) {
   pl.mthin.clear();
   std::vector<Problem<T>> wide;
   pl.thin_rows = 0;
-  pl.mthin_cols = 0;
+  pl.mthin_cols = pl.mthin_rows = 0;
   std::vector<long long> part_off;
   long long part_elems = 0;
   int max_k = 0;
@@ -323,6 +325,7 @@ static int upload_problems(ProblemList<T>& pl, cudaStream_t st) {
       Problem<T> q = p;
       q.tile_begin = pl.mthin_cols;
       pl.mthin_cols += q.N;
+      pl.mthin_rows = std::max(pl.mthin_rows, q.M);
       pl.mthin.push_back(q);
       part_off.push_back(part_elems);
       part_elems += (long long)q.M * q.N;
@@ -385,7 +388,7 @@ static int launch_grouped(const ProblemList<T>& pl, const T* cbase, T* sbase, cu
                                              pl.d_segs.template as<Segment<T>>(), pl.d_part_off.template as<long long>(),
                                              cbase, sbase, pl.mthin_cols, pl.mthin_part_stride,
                                              pl.d_part.template as<T>()); ISCSI_COUNT_LAUNCH();
-    k_mthin_reduce<T><<<(pl.mthin_cols + 255) / 256, 256, 0, st>>>(
+    k_mthin_reduce<T><<<dim3((pl.mthin_cols + 255) / 256, pl.mthin_rows), 256, 0, st>>>(
         pl.d_mthin.template as<Problem<T>>(), (int)pl.mthin.size(), pl.d_part_off.template as<long long>(), sbase,
         cbase, pl.mthin_cols, pl.mthin_chunks, pl.mthin_part_stride, pl.d_part.template as<T>()); ISCSI_COUNT_LAUNCH();
     ISCSI_CUDA(cudaGetLastError());
