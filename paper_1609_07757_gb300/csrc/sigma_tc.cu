@@ -24,6 +24,8 @@
 #include <algorithm>
 #include <climits>
 #include <cstring>
+#include <functional>
+#include <queue>
 #include <vector>
 
 #include "internal.cuh"
@@ -452,10 +454,12 @@ static int add_tiles(std::vector<OzProblem>& probs, int bn = OZ_BN) {
 // Half as many tiles fill the SMs less evenly, so narrow ones win up to one wave of them
 // and just above whole waves of wide ones.  Measured, K = 3584: 152 / 80 tiles 84 us narrow, 119 wide;
 // 171 / 90: 157, 118; 304 / 160: 164, 231; 480 / 240: 309, 239; 784 / 392: 461, 361 (K = 512: 20, 26; 34, 27;
-// 36, 47; 65, 49; 94, 70), which waves x the cycles of a K step below order as they came out.  A segment
+// 36, 47; 65, 49; 94, 70): a tile costs what the two constants of its width say, and the width whose tiles end
+// first wins (CISDT in 80 orbitals, unequal K: 442 narrow tiles 286 us, where whole waves alone took 272 wide
+// ones).  A segment
 // that reaches only the first half of a wide tile of its problem would move the chunk
 // boundaries of the second half: such lists stay narrow.
-constexpr int kT3Step256 = 850, kT3Step128 = 575;
+constexpr int kT3Step256 = 484, kT3Step128 = 333, kT3Tile256 = 7700, kT3Tile128 = 6500;  // ns
 int t3_tiles(std::vector<OzProblem>& probs, const std::vector<OzSeg>& segs, int& bn) {
   bool wide = true;
   for (const OzProblem& p : probs)
@@ -463,13 +467,35 @@ int t3_tiles(std::vector<OzProblem>& probs, const std::vector<OzSeg>& segs, int&
       const OzSeg& sg = segs[p.seg_begin + g];
       if (sg.K > 0 && sg.nrows_b < p.N && round_up(sg.nrows_b, OZ_BW_ROWS) % 256 != 0) wide = false;
     }
-  const int sms = tc_sm_count();
-  auto waves = [&](int t) { return (t + sms - 1) / sms; };
   const int narrow_tiles = add_tiles(probs, 128);
   bn = 128;
   if (!wide) return narrow_tiles;
+  // the end of the last tile when each goes to the SM that is free first, in launch order
+  auto makespan = [&](int cols, long long step, long long fixed) {
+    std::priority_queue<long long, std::vector<long long>, std::greater<long long>> sm;
+    for (int i = 0; i < tc_sm_count(); ++i) sm.push(0);
+    long long end = 0;
+    std::vector<long long> cost;
+    for (const OzProblem& p : probs) {
+      cost.assign(p.tiles_n, fixed);
+      for (int t = 0; t < p.tiles_n; ++t)
+        for (int g = 0; g < p.seg_count; ++g) {
+          const OzSeg& sg = segs[p.seg_begin + g];
+          if (t * cols < sg.nrows_b) cost[t] += sg.K / T3_BK * step;
+        }
+      for (int mt = 0; mt < round_up(p.M, OZ_BM) / OZ_BM; ++mt)
+        for (long long c : cost) {
+          const long long at = sm.top() + c;
+          sm.pop();
+          sm.push(at);
+          end = std::max(end, at);
+        }
+    }
+    return end;
+  };
+  const long long narrow = makespan(128, kT3Step128, kT3Tile128);
   const int wide_tiles = add_tiles(probs, 256);
-  if (waves(wide_tiles) * kT3Step256 < waves(narrow_tiles) * kT3Step128) {
+  if (makespan(256, kT3Step256, kT3Tile256) < narrow) {
     bn = 256;
     return wide_tiles;
   }

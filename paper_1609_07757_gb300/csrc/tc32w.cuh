@@ -17,8 +17,8 @@
 // of products.  So BN = 256: six MMAs of N = 256 for twice the products; a stage of two K
 // steps (TMA rows of 64 bytes, one wait for twelve MMAs); the stages of a turn of the ring unrolled, so
 // that a descriptor is a base plus a constant, of which only the low word is computed.  Full CI
-// n = 60, both spin parts in one launch: 834 -> 500 us, one sigma 1004 -> 671; a step of a
-// 256-column tile 900 cycles with its share of the drain, of a 128-column one 575.
+// n = 60, both spin parts in one launch: 834 -> 500 us, one sigma 1004 -> 671 (a step's and a tile's
+// time: t3_tiles).
 //
 // Warp 0 loads (TMA; A in a box of 128 rows x all terms, B in boxes of 128 rows of a term), warp 1 issues
 // the MMAs (its loop whole, one elected lane issuing), the others drain (BN / 64 per TMEM
@@ -283,11 +283,24 @@ __global__ void __launch_bounds__(T3wShape<BN>::THREADS, 1)
       const int rows = min(32, P.M - m0 - quarter * 32);
       float* dst = Tp + (long long)(m0 + quarter * 32) * P.ldt + n0 + cbase + lane;
       const bool c0 = n0 + cbase + lane < P.N, c1 = n0 + cbase + lane + 32 < P.N;
-#pragma unroll 4
-      for (int r = 0; r < rows; ++r, dst += P.ldt) {
-        const float x0 = buf[r * (T3W_EPI_COLS + 1) + lane], x1 = buf[r * (T3W_EPI_COLS + 1) + lane + 32];
-        if (c0) dst[0] = P.accumulate ? dst[0] + x0 : x0;
-        if (c1) dst[32] = P.accumulate ? dst[32] + x1 : x1;
+      // an accumulating block's old values eight rows at a time (a load before each store waited for 64 round
+      // trips one after the other: 28 tiles of 3 + 3 electrons in 18 orbitals 40 us, now 20)
+      for (int r0 = 0; r0 < rows; r0 += 8) {
+        float o0[8], o1[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const bool on = P.accumulate && r0 + j < rows;
+          o0[j] = on && c0 ? dst[(long long)(r0 + j) * P.ldt] : 0.0f;
+          o1[j] = on && c1 ? dst[(long long)(r0 + j) * P.ldt + 32] : 0.0f;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int r = r0 + j;
+          if (r >= rows) break;
+          const float x0 = buf[r * (T3W_EPI_COLS + 1) + lane], x1 = buf[r * (T3W_EPI_COLS + 1) + lane + 32];
+          if (c0) dst[(long long)r * P.ldt] = P.accumulate ? o0[j] + x0 : x0;
+          if (c1) dst[(long long)r * P.ldt + 32] = P.accumulate ? o1[j] + x1 : x1;
+        }
       }
     }
   }
