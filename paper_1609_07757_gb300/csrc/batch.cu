@@ -8,7 +8,10 @@
 // output addressing through a table of output bases (OzProblem::tb).  From the
 // second call with the same contexts, vectors, vector count and precision,
 // the whole sequence is replayed from one captured CUDA graph, so a batch of
-// any size costs one launch on the host.
+// any size costs one launch on the host.  The graph names the contexts' buffers,
+// work lists and scales as they were: when another call on a context has
+// changed one (sigma_layout), the graph is dropped, that batch runs directly
+// and the next one is captured again.
 #include <algorithm>
 #include <cstring>
 #include <memory>
@@ -87,13 +90,22 @@ struct BatchState {
   long long kernels = 0;
   bool failed = false;
   int calls = 0;
+  std::vector<unsigned long long> layout;  // of the contexts when the graph was captured
   BatchState() = default;
   BatchState(const BatchState&) = delete;
   BatchState& operator=(const BatchState&) = delete;
+  void drop_graph() {
+    if (x) {
+      cudaStreamSynchronize(bs);  // a replay may be running
+      cudaGraphExecDestroy(x);
+    }
+    if (g) cudaGraphDestroy(g);
+    x = nullptr;
+    g = nullptr;
+  }
   ~BatchState() {
     if (bs) cudaStreamSynchronize(bs);
-    if (x) cudaGraphExecDestroy(x);
-    if (g) cudaGraphDestroy(g);
+    drop_graph();
     if (ev) cudaEventDestroy(ev);
     if (bs) cudaStreamDestroy(bs);
   }
@@ -245,7 +257,17 @@ long long graph_kernel_nodes(cudaGraph_t g) {
   return c;
 }
 
+std::vector<unsigned long long> batch_layout(const SigmaBatch& sb) {
+  std::vector<unsigned long long> v;
+  for (const Context* c : sb.ctxs) v.push_back(sigma_layout(*c, sb.prec));
+  return v;
+}
+
 int batch_run(BatchState& B) {
+  if (B.x && batch_layout(B.sb) != B.layout) {
+    B.drop_graph();
+    B.calls = 0;
+  }
   if (B.x) {
     ISCSI_CUDA(cudaGraphLaunch(B.x, B.bs));
     g_launch_count += B.kernels;
@@ -264,6 +286,7 @@ int batch_run(BatchState& B) {
   if (ce == cudaSuccess && rc == kOk && ee == cudaSuccess && g && cudaGraphInstantiate(&B.x, g, 0) == cudaSuccess) {
     B.g = g;
     B.kernels = graph_kernel_nodes(g);
+    B.layout = batch_layout(B.sb);
     ISCSI_CUDA(cudaGraphLaunch(B.x, B.bs));
     g_launch_count += B.kernels;
     return kOk;

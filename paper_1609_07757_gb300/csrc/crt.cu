@@ -717,12 +717,18 @@ struct CrtState {
   std::vector<CrtFoldLaunch> folds;
   int ops_smem = 0, ops_blocks = 0;
   int nvec = -1, parts = 0;  // what job was built for (parts: 1 opposite spin, 2 same spin)
-  long long version = 0;
 };
 
 void crt_release(Context& ctx) {
+  if (ctx.crt) ++ctx.crt_version;
   delete ctx.crt;
   ctx.crt = nullptr;
+}
+
+void crt_invalidate(Context& ctx) {
+  if (!ctx.crt) return;
+  ctx.crt->nvec = -1;
+  ++ctx.crt_version;
 }
 
 constexpr int kFoldMaxSmem = 220 * 1024;
@@ -957,7 +963,7 @@ int crt_matrices_changed(Context& ctx) {
   ISCSI_TRY(take_norms(ctx, 2, rm, mmax));
   const double b = sigma_bound(ctx, S, S.parts, rm);
   if (!(b <= S.bound) || !(std::log2(std::max(mmax, 1e-300)) + S.sh < 52.0)) {
-    S.nvec = -1;
+    crt_invalidate(ctx);
     S.m_cut[0] = -1;
     return kOk;
   }
@@ -1283,7 +1289,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   ISCSI_TRY(S.job.upload(st));
   S.nvec = nvec;
   S.parts = parts;
-  ++S.version;
+  ++ctx.crt_version;
   return kOk;
 }
 
@@ -1369,7 +1375,7 @@ int crt_batch_launch(CrtBatch*& b, const std::vector<Context*>& ctxs, int* err, 
   if (ctxs.empty()) return kOk;
   if (!b) b = new CrtBatch();
   std::vector<std::pair<Context*, long long>> src;
-  for (Context* c : ctxs) src.push_back({c, c->crt->version});
+  for (Context* c : ctxs) src.push_back({c, c->crt_version});
   if (src != b->src) {
     b->job.probs.clear();
     for (Context* c : ctxs) b->job.probs.insert(b->job.probs.end(), c->crt->job.probs.begin(), c->crt->job.probs.end());

@@ -131,6 +131,7 @@ struct ProblemList {
   int mthin_cols = 0, mthin_rows = 0;  // columns in all, most rows of a problem
   int mthin_chunks = 1;
   long long mthin_part_stride = 0;
+  long long version = 0;  // bumped at every rebuild
 };
 constexpr int kThinN = 16;
 
@@ -261,6 +262,7 @@ struct Context {
   int pl_ss_tc = -1;  // same-spin routing the FP64 grouped-GEMM list was built for
   // FP64 contractions through residue numbers (crt.cu), built at first use
   CrtState* crt = nullptr;
+  long long crt_version = 0;  // bumped when its buffers, scale or work list change, are dropped, or may not be used as they are
   // FP32 form of the tensor-core contractions (three bf16 terms per element)
   OzJob t3_ab, t3_ss, t3_both;
   DevBuf t3_gs, t3_bs, t3_mas, t3_mbs, t3_cs;
@@ -343,6 +345,9 @@ int context_build(Context& ctx, int n, int na, int nb, int kmax, const double* h
 enum { kPhPre = 1, kPhAbGemm = 2, kPhMid = 4, kPhSsGemm = 8, kPhPost = 16, kPhAll = 31 };
 int sigma_run(Context& ctx, const double* c, double* sigma, int nvec, int precision, int phases = kPhAll);
 int sigma_workspace(Context& ctx, int nvec, int precision);
+// identifies the buffers, work lists, routing and scales that launches of sigma at this precision name: a captured
+// graph of them holds while it is unchanged
+unsigned long long sigma_layout(const Context& ctx, int precision);
 // algorithmic flops per sigma per vector of the opposite-spin GEMM (which = 0)
 // or of the same-spin GEMMs (which = 1): 2 x M x K x N summed over problems;
 // which = 2: bf16 MMA flops of the tensor-core opposite-spin contraction
@@ -396,6 +401,7 @@ int crt_operands(Context& ctx, const double* c, int nvec, int parts);
 int crt_gemm(Context& ctx);
 int crt_fold(Context& ctx, double* sigma);  // sigma (overwritten): the parts that went through residues
 int crt_matrices_changed(Context& ctx);
+void crt_invalidate(Context& ctx);  // a call ended early: build (and clear the exponents) anew at the next one
 void crt_release(Context& ctx);
 // bf16 MMA flops, work items and CTAs of the last built launch (0 without one)
 void crt_stats(const Context& ctx, double& flops, int& items, int& grid, int& moduli);

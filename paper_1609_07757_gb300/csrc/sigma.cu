@@ -311,6 +311,7 @@ struct TileCfg<float> {
 template <typename T>
 static int upload_problems(ProblemList<T>& pl, cudaStream_t st) {
   using C = TileCfg<T>;
+  ++pl.version;
   // split off the thin problems
   pl.thin.clear();
   pl.mthin.clear();
@@ -679,6 +680,38 @@ int sigma_workspace(Context& ctx, int nvec, int precision) {
     ctx.pl_nvec32 = 0;
   }
   return kOk;
+}
+
+unsigned long long sigma_layout(const Context& ctx, int precision) {
+  unsigned long long h = 1469598103934665603ull;  // FNV-1a over 64-bit words
+  auto add = [&](long long x) { h = (h ^ (unsigned long long)x) * 1099511628211ull; };
+  auto buf = [&](const DevBuf& b) { add((long long)reinterpret_cast<uintptr_t>(b.p)); };
+  const Options& o = options();
+  const Context::Route& R = ctx.route[precision == 32 ? 1 : 0];
+  add(R.ab_tc);
+  add(R.ss_min);
+  add(precision == 32 ? o.fp32_tc : o.fp64_tc);
+  add(o.samespin_tc);
+  buf(ctx.ct);
+  buf(ctx.tt);
+  buf(ctx.oz_err);
+  if (precision == 32) {
+    for (const DevBuf* b : {&ctx.c32, &ctx.s32, &ctx.G32, &ctx.M32[0], &ctx.M32[1], &ctx.t3_gs, &ctx.t3_bs, &ctx.t3_mas,
+                            &ctx.t3_mbs, &ctx.t3_cs})
+      buf(*b);
+    for (const OzJob* j : {&ctx.t3_ab, &ctx.t3_ss, &ctx.t3_both}) add(j->version);
+    add(ctx.pl_ab32.version);
+    add(ctx.pl_ss32.version);
+  } else {
+    for (const DevBuf* b : {&ctx.G64, &ctx.M64[0], &ctx.M64[1], &ctx.oz_gs, &ctx.oz_gexp, &ctx.oz_bs, &ctx.oz_bexp,
+                            &ctx.oz_mas, &ctx.oz_maexp, &ctx.oz_mbs, &ctx.oz_mbexp, &ctx.oz_cs, &ctx.oz_csexp})
+      buf(*b);
+    for (const OzJob* j : {&ctx.oz_ab, &ctx.oz_ss, &ctx.oz_both}) add(j->version);
+    add(ctx.pl_ab64.version);
+    add(ctx.pl_ss64.version);
+    add(ctx.crt_version);
+  }
+  return h;
 }
 
 // M = M_base + f M_v, elementwise

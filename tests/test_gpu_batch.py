@@ -143,3 +143,70 @@ def test_batch_davidson_matches_dense_and_single(precision):
         L.iscsi_set_option("precision", precision)
         r = s - torch.tensor(e[i], device="cuda")[:, None] * vecs[i]
         assert torch.linalg.norm(r, dim=1).max().item() < 1e-6
+
+
+def _fma(h, c, nvec):
+    """sigma on the FP64 FMA kernels, which share only the tables with the tensor-core products."""
+    L.iscsi_ctx_use(h)
+    L.iscsi_set_option("fp64_tc", 0)
+    s = torch.empty_like(c)
+    L.iscsi_sigma(c, s, nvec)
+    torch.cuda.synchronize()
+    L.iscsi_set_option("fp64_tc", 1)
+    return s
+
+
+def _close(outs, refs, rel=1e-12):
+    for o, r in zip(outs, refs):
+        for a, b in zip(o, r):  # vector by vector: each has its own scale
+            assert torch.linalg.norm(a - b).item() <= rel * torch.linalg.norm(b).item()
+            assert (a - b).abs().max().item() <= rel * b.abs().max().item()
+
+
+# another call on a member between two replays: a larger block (buffers and work lists move), a propagation under a
+# field that lifts the string matrices past the scale they were cut for, a single larger vector (exponents laid out
+# for another block)
+@pytest.mark.parametrize("other,precision,nvec", [("block", 64, 1), ("block", 32, 1), ("field", 64, 1),
+                                                  ("single", 64, 2), ("options", 64, 1)])
+def test_batch_replay_after_other_calls(other, precision, nvec):
+    L.iscsi_set_option("autotune", 0)
+    try:
+        hs, cs = [], []
+        for i, n in enumerate((12, 16)):
+            h1, eri = make_integrals(n, 1700 + i, ell=3.0, nchol=10)
+            L.iscsi_init(n, 2, 2, 4, h1, eri, 1e-14)
+            hs.append(L.iscsi_ctx_current())
+            nd = L.iscsi_ndet()
+            cs.append(torch.tensor(np.stack([unit_vector(nd, 60 + 7 * i + v) * 10.0 ** -v for v in range(nvec)]),
+                                   dtype=torch.float64, device="cuda"))
+        pos = np.arange(12) - 5.5
+        L.iscsi_init(12, 2, 2, 4, np.diag(pos / 12) + 0.3 * (np.eye(12, k=1) + np.eye(12, k=-1)), None, 1e-14)
+        coupling = L.iscsi_ctx_current()
+        refs = [_fma(h, c, nvec) for h, c in zip(hs, cs)]
+        outs = [torch.empty_like(c) for c in cs]
+        rel = 1e-12 if precision == 64 else 2e-5
+        L.iscsi_set_option("precision", precision)
+        for _ in range(3):  # direct, captured, replayed
+            L.iscsi_batch_sigma(hs, cs, outs, nvec)
+        L.iscsi_ctx_use(hs[0])
+        nd = L.iscsi_ndet()
+        if other == "block":
+            c = torch.randn(5, nd, dtype=torch.float64, device="cuda")
+            L.iscsi_sigma(c, torch.empty_like(c), 5)
+        elif other == "field":
+            c = cs[0][0].clone()
+            L.iscsi_propagate(c, 1, 1e-4, np.array([1e3]), coupling, 4, imaginary=True)
+        elif other == "single":
+            c = cs[0][:1] * 1e9
+            L.iscsi_sigma(c, torch.empty_like(c), 1)
+        else:
+            L.iscsi_set_option("fp64_tc", 0)
+        for _ in range(3):
+            for o in outs:
+                o.fill_(np.nan)
+            L.iscsi_batch_sigma(hs, cs, outs, nvec)
+            torch.cuda.synchronize()
+            _close(outs, refs, rel)
+    finally:
+        L.iscsi_set_option("fp64_tc", 1)
+        L.iscsi_set_option("autotune", 1)
