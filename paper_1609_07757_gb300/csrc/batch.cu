@@ -326,6 +326,8 @@ int batch_sigma(const std::vector<Context*>& ctxs, const std::vector<const doubl
   set_stream(B.bs);
   int rc = batch_run(B);
   set_stream(user);
+  if (rc != kOk)
+    for (Context* c : ctxs) crt_invalidate(*c);  // some contexts' steps may have ended before their folds
   ++B.calls;
   ISCSI_CUDA(cudaEventRecord(B.ev, B.bs));
   ISCSI_CUDA(cudaStreamWaitEvent(user, B.ev, 0));

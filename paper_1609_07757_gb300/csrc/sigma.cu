@@ -920,7 +920,7 @@ int crt_parts(Context& ctx, int nvec) {
   return parts;
 }
 
-int sigma_run(Context& ctx, const double* c, double* sigma, int nvec, int precision, int phases) {
+static int sigma_steps(Context& ctx, const double* c, double* sigma, int nvec, int precision, int phases) {
   cudaStream_t st = stream();
   if (phases == kPhAll) ISCSI_TRY(sigma_autotune(ctx, c, sigma, nvec, precision));
   if (phases & kPhPre) ISCSI_TRY(sigma_workspace(ctx, nvec, precision));
@@ -949,6 +949,12 @@ int sigma_run(Context& ctx, const double* c, double* sigma, int nvec, int precis
   }
   ISCSI_CUDA(cudaGetLastError());
   return kOk;
+}
+
+int sigma_run(Context& ctx, const double* c, double* sigma, int nvec, int precision, int phases) {
+  const int rc = sigma_steps(ctx, c, sigma, nvec, precision, phases);
+  if (rc != kOk) crt_invalidate(ctx);
+  return rc;
 }
 
 // ---------------------------------------------------------------------------

@@ -210,3 +210,38 @@ def test_batch_replay_after_other_calls(other, precision, nvec):
     finally:
         L.iscsi_set_option("fp64_tc", 1)
         L.iscsi_set_option("autotune", 1)
+
+
+def test_batch_that_fails_leaves_no_exponents():
+    """A batch that runs out of memory at its second context has taken the first one's exponents already: they must
+    not reach that context's next sigma (of a vector nine decades smaller)."""
+    L.iscsi_set_option("autotune", 0)
+    hog = None
+    try:
+        h1, eri = make_integrals(12, 1800, ell=3.0, nchol=10)
+        L.iscsi_init(12, 2, 2, 4, h1, eri, 1e-14)
+        small = L.iscsi_ctx_current()
+        nd = L.iscsi_ndet()
+        c = torch.tensor(unit_vector(nd, 3)[None], dtype=torch.float64, device="cuda")
+        ref = _fma(small, c, 1)
+        s = torch.empty_like(c)
+        L.iscsi_sigma(c, s, 1)
+        h1, eri = make_integrals(44, 1801, ell=3.0, nchol=10)
+        L.iscsi_init(44, 2, 2, 4, h1, eri, 1e-14)
+        large = L.iscsi_ctx_current()
+        cl = torch.randn(1, L.iscsi_ndet(), dtype=torch.float64, device="cuda")
+        sl = torch.empty_like(cl)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free = torch.cuda.mem_get_info()[0]
+        hog = torch.empty(free - (24 << 20), dtype=torch.uint8, device="cuda")  # its lifted vector takes 30 MB
+        with pytest.raises(L.IscsiError):
+            L.iscsi_batch_sigma([small, large], [c * 1e9, cl], [s, sl], 1)
+        L.iscsi_ctx_use(small)
+        L.iscsi_sigma(c, s, 1)
+        torch.cuda.synchronize()
+        _close([s], [ref])
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+        L.iscsi_set_option("autotune", 1)
