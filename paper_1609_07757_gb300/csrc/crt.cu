@@ -205,9 +205,18 @@ __global__ void __launch_bounds__(256) k_crt_cut(const double* __restrict__ X, i
   crt_store8(x, M, o, (long long)rows_pad * nkb * CRT_BK);
 }
 
-// exponent field of the largest |c| of each vector; acc starts at zero
-// (k_crt_fold clears it again)
-__global__ void __launch_bounds__(256) k_crt_cmax(const double* __restrict__ c, long long ndet, int* __restrict__ acc) {
+// Infinities and NaN of a vector: their number, and the determinants of the first kCrtBad of them
+constexpr int kCrtBad = 64;
+struct CrtBadList {
+  int* count;        // this call's, cleared by k_crt_fold
+  int* count_now;    // k_crt_operands' copy for k_crt_fold
+  long long* det;    // [vector][kCrtBad]
+};
+
+// exponent field of the largest finite |c| of each vector, and its elements that are not finite;
+// acc and the counts start at zero (k_crt_fold clears them again)
+__global__ void __launch_bounds__(256) k_crt_cmax(const double* __restrict__ c, long long ndet, int* __restrict__ acc,
+                                                  CrtBadList bad) {
   const double* v = c + (long long)blockIdx.y * ndet;
   const long long stride = (long long)gridDim.x * 256;
   int m = 0;
@@ -217,6 +226,18 @@ __global__ void __launch_bounds__(256) k_crt_cmax(const double* __restrict__ c, 
     m = max(m, max(max(oz_exp_field(a), oz_exp_field(b)), max(oz_exp_field(d), oz_exp_field(e))));
   }
   for (; i < ndet; i += stride) m = max(m, oz_exp_field(__ldg(v + i)));
+  if (m == 0x7FF) {
+    m = 0;
+    for (i = blockIdx.x * 256ll + threadIdx.x; i < ndet; i += stride) {
+      const int f = oz_exp_field(__ldg(v + i));
+      if (f < 0x7FF) {
+        m = max(m, f);
+      } else {
+        const int k = atomicAdd(bad.count + blockIdx.y, 1);
+        if (k < kCrtBad) bad.det[(long long)blockIdx.y * kCrtBad + k] = i;
+      }
+    }
+  }
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0 && m) atomicMax(acc + blockIdx.y, m);
 }
@@ -237,6 +258,7 @@ struct CrtOperands {
   const long long* off;
   long long ndet;
   int *cmax, *cexp;          // exponent fields: largest of this call, and the copy for k_crt_fold
+  CrtBadList bad;
   __nv_bfloat16* lift;
   // same spin
   int na, nb, ctx_x, ctx_y;  // strings; 64 x 64 tiles along beta and alpha (0: no same-spin part)
@@ -273,7 +295,10 @@ __global__ void __launch_bounds__(256) k_crt_operands(const __grid_constant__ Cr
   extern __shared__ __align__(16) unsigned char crt_dyn[];
   const int nlift = O.blk_start[O.ngroups];
   if (blockIdx.x == 0)
-    for (int v = threadIdx.x; v < O.nvec; v += 256) O.cexp[v] = O.cmax[v];
+    for (int v = threadIdx.x; v < O.nvec; v += 256) {
+      O.cexp[v] = O.cmax[v];
+      O.bad.count_now[v] = O.bad.count[v];
+    }
   if ((int)blockIdx.x < nlift) {
     int gi = 0;
     while ((int)blockIdx.x >= O.blk_start[gi + 1]) ++gi;
@@ -368,7 +393,7 @@ struct CrtFoldGroup {
   int ncol, ntile, tn;
 };
 struct CrtFold {
-  int na, nb, n, nholeB, nvec, nm;
+  int na, nb, n, nholeB, nvec, nm, na_strings;
   int parts;                 // 1: opposite spin, 2: same spin
   const int16_t* res;
   CrtFoldGroup g[2 * kMaxElec];
@@ -388,6 +413,7 @@ struct CrtFold {
   const int* nballow;
   long long ndet;
   int *cmax, *cexp;
+  CrtBadList bad;
   int ebias;                 // -(bits of the coefficients) - sh
   const int* ypos;           // per Y: run << 24 | position in a staged row (before the run's shift)
   int ypad[kMaxElec + 2];    // first position of each run in a staged row (multiples of 8)
@@ -405,6 +431,28 @@ constexpr int kFoldThreads = 1024;
 // first element of orbital r's row in a staged hole
 __device__ __forceinline__ int fold_row(const CrtFold& F, int r) {
   return r < F.rsplit ? r * F.stride : F.base1 + (r - F.rsplit) * F.stride1;
+}
+
+// whether a determinant of the list lies within two excitations of (A, B): where H reaches it (the orbitals of a
+// string are those of its dec entries)
+__device__ __forceinline__ bool crt_reached(const CrtFold& F, const long long* det, int count, int A, int B) {
+  if (count > kCrtBad) return true;
+  for (int k = 0; k < count; ++k) {
+    int a = 0, hi = F.na_strings;
+    while (hi - a > 1) {
+      const int mid = (a + hi) >> 1;
+      if (F.off[mid] <= det[k]) a = mid;
+      else hi = mid;
+    }
+    const int b = (int)(det[k] - F.off[a]);
+    int moved = F.na + F.nb;
+    for (int i = 0; i < F.na; ++i)
+      for (int j = 0; j < F.na; ++j) moved -= ((F.decA[A * F.na + i] ^ F.decA[a * F.na + j]) & 0x1FE) == 0;
+    for (int i = 0; i < F.nb; ++i)
+      for (int j = 0; j < F.nb; ++j) moved -= ((F.decB[B * F.nb + i] ^ F.decB[b * F.nb + j]) & 0x1FE) == 0;
+    if (moved <= 2) return true;
+  }
+  return false;
 }
 
 // One block per alpha string (and vector, and share of its beta strings): for
@@ -428,7 +476,7 @@ __global__ void __launch_bounds__(kFoldThreads) k_crt_fold(const __grid_constant
   const int lim = F.nballow[F.alevel[A]];
   const int B0 = blockIdx.y * (blockDim.x * kFoldPer) + threadIdx.x;
   if ((int)(blockIdx.y * (blockDim.x * kFoldPer)) >= lim) return;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) F.cmax[v] = 0;  // for the next call
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) F.cmax[v] = F.bad.count[v] = 0;  // for the next call
   const bool ab = (F.parts & 1) != 0, ss = (F.parts & 2) != 0;
   int16_t* const stage = reinterpret_cast<int16_t*>(crt_dyn);
   uint2* const unit = reinterpret_cast<uint2*>(crt_dyn + (size_t)F.nbuf * F.stage_bytes);
@@ -577,14 +625,18 @@ __global__ void __launch_bounds__(kFoldThreads) k_crt_fold(const __grid_constant
     }
   }
   const int f = F.cexp[v];
-  // a vector with an infinity or NaN: every nonzero sum overflows
-  const int e = (f > 0 ? f - 1022 : 0) + (f == 0x7FF ? 4096 : 0) + F.ebias;
+  const int e = (f > 0 ? f - 1022 : 0) + F.ebias;
   double* out = sigma + v * F.ndet + F.off[A];
 #pragma unroll
   for (int u = 0; u < kFoldPer; ++u) {
     const int B = B0 + u * (int)blockDim.x;
     if (B < lim) out[B] = crt_value(lo[u], hi[u], W.mman, W.mexp, e);
   }
+  const int nbad = F.bad.count_now[v];
+  if (nbad == 0) return;
+#pragma unroll 1
+  for (int B = B0; B < lim && B < B0 + kFoldPer * (int)blockDim.x; B += blockDim.x)
+    if (crt_reached(F, F.bad.det + v * kCrtBad, nbad, A, B)) out[B] = __longlong_as_double(0x7FF8000000000000ll);
 }
 
 // ---------------------------------------------------------------------------
@@ -709,7 +761,7 @@ struct CrtState {
   DevBuf norms;
   DevBuf g_res, b_res;                  // G, lifted vector
   DevBuf ma_res, mb_res, ca_res, ct_res;  // string matrices, C, C^T
-  DevBuf cfield;                        // exponent fields of the vectors: this call's, k_crt_fold's copy
+  DevBuf cfield;                        // of the vectors: lists of non-finite elements, exponent fields and counts (this call's, copies)
   DevBuf out;                           // residues of the products
   CrtOperands ops;
   CrtFold fold;
@@ -997,14 +1049,17 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   CrtFold& F = S.fold;
   std::memset(&O, 0, sizeof(O));
   std::memset(&F, 0, sizeof(F));
-  if (S.cfield.bytes < 2 * sizeof(int) * nvec) {
-    ISCSI_TRY(S.cfield.grow(2 * sizeof(int) * nvec));
-  }
+  const size_t per_vec = 4 * sizeof(int) + kCrtBad * sizeof(long long);
+  if (S.cfield.bytes < per_vec * nvec) ISCSI_TRY(S.cfield.grow(per_vec * nvec));
   ISCSI_CUDA(cudaMemsetAsync(S.cfield.p, 0, S.cfield.bytes, st));
   O.nvec = F.nvec = nvec;
   O.n = F.n = n;
-  O.cmax = F.cmax = S.cfield.as<int>();
-  O.cexp = F.cexp = S.cfield.as<int>() + nvec;
+  O.bad.det = S.cfield.as<long long>();
+  O.cmax = F.cmax = reinterpret_cast<int*>(O.bad.det + (size_t)nvec * kCrtBad);
+  O.cexp = F.cexp = O.cmax + nvec;
+  O.bad.count = O.cmax + 2 * (size_t)nvec;
+  O.bad.count_now = O.cmax + 3 * (size_t)nvec;
+  F.bad = O.bad;
   O.nholeA = SA.nhole;
   O.nholeB = F.nholeB = SB.nhole;
   O.off = F.off = ctx.off.as<long long>();
@@ -1015,6 +1070,9 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   F.nm = nm;
   F.na = ctx.na;
   F.nb = ctx.nb;
+  F.na_strings = NA;
+  F.decA = SA.dec.as<int>();
+  F.decB = SB.dec.as<int>();
   F.kmax = ctx.kmax;
   F.ni = F.nbuf = 1;
   F.ebias = -kCrtCBits - S.sh;
@@ -1145,8 +1203,6 @@ static int crt_build(Context& ctx, int nvec, int parts) {
       add_out(H.p);
       S.job.probs.push_back(H);
     }
-    F.decA = SA.dec.as<int>();
-    F.decB = SB.dec.as<int>();
     F.rruns = S.flat ? 1 : 2;
     F.rsplit = S.flat ? n : SB.nocc;
     F.yruns = (int)S.ystart.size() - 1;
@@ -1329,7 +1385,7 @@ int crt_operands(Context& ctx, const double* c, int nvec, int parts) {
     ISCSI_TRY(rc);
   }
   const int vb = (int)std::min<long long>(2 * tc_sm_count(), (ctx.ndet + 1023) / 1024);
-  k_crt_cmax<<<dim3(vb, nvec), 256, 0, st>>>(c, ctx.ndet, S.ops.cmax); ISCSI_COUNT_LAUNCH();
+  k_crt_cmax<<<dim3(vb, nvec), 256, 0, st>>>(c, ctx.ndet, S.ops.cmax, S.ops.bad); ISCSI_COUNT_LAUNCH();
   k_crt_operands<<<S.ops_blocks, 256, S.ops_smem, st>>>(S.ops, S.mods, c); ISCSI_COUNT_LAUNCH();
   ISCSI_CUDA(cudaGetLastError());
   return kOk;

@@ -21,11 +21,11 @@
 namespace iscsi {
 
 // v 2^(bits - e) rounded to an integer, |v| < 2^e, bits <= 53 (in integer
-// arithmetic; zeros and subnormals give 0)
+// arithmetic; zeros, subnormals and what is not finite give 0)
 __device__ __forceinline__ long long crt_fixed(double v, int e, int bits) {
   const long long b = __double_as_longlong(v);
   const int E = (int)((b >> 52) & 0x7FF);
-  if (E == 0) return 0;
+  if ((unsigned)(E - 1) >= 0x7FEu) return 0;
   const long long m = (b & 0xFFFFFFFFFFFFFll) | (1ll << 52);
   const int sh = 1075 - E + e - bits;  // v = m 2^(E - 1075); >= 0 when |v| < 2^e
   long long N = 0;

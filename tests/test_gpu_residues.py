@@ -155,3 +155,47 @@ def test_residues_many_vectors(n, kmax, parts, batch):
         s = out.cpu().numpy()
     for v in range(nvec):
         check(s[v], ref[v])
+
+
+def excitations(na, nb, kmax):
+    """(number of differing alpha + beta orbitals of determinants i, j) as a function of i: a row over all j."""
+    occ, lev = [], []
+    for spin, ne in enumerate((na, nb)):
+        o, l = L.iscsi_get_strings(spin, ne)
+        m = np.zeros((len(l), 256), dtype=np.int64)
+        m[np.arange(len(l))[:, None], np.asarray(o)] = 1
+        occ.append(m)
+        lev.append(np.asarray(l))
+    A, B = np.nonzero(lev[0][:, None] + lev[1][None, :] <= kmax)  # determinants in order
+
+    def row(i):
+        same = (occ[0][A[i]] @ occ[0].T)[A] + (occ[1][B[i]] @ occ[1].T)[B]
+        return occ[0][0].sum() + occ[1][0].sum() - same
+
+    return row
+
+
+# infinities and NaN: sigma is NaN exactly where H reaches them (within two excitations) and as without them
+# elsewhere; more than the list holds: everywhere
+@pytest.mark.parametrize("n,na,nb,kmax", [(18, 2, 2, 4), (24, 2, 2, 3), (9, 4, 4, 8), (12, 3, 3, 4), (20, 1, 1, 2),
+                                          (11, 2, 5, 7)])
+@pytest.mark.parametrize("count", [1, 3, 70])
+def test_residues_nonfinite(n, na, nb, kmax, count):
+    h1, eri = make_integrals(n, 7500 + n, ell=4.0, nchol=12)
+    L.iscsi_init(n, na, nb, kmax, h1, eri, 1e-14)
+    nd = L.iscsi_ndet()
+    row = excitations(na, nb, kmax)
+    rng = np.random.default_rng(n)
+    at = rng.choice(nd, size=count, replace=False)
+    bad = unit_vector(nd, 4)
+    bad[at] = rng.choice([np.nan, np.inf, -np.inf], size=count)
+    clean = np.where(np.isfinite(bad), bad, 0.0)
+    # the second vector is finite, and the call after this one sees no trace of it
+    s = sigma(np.stack([bad, clean]), 2)
+    assert L.iscsi_stats()["residues"]["items"] > 0
+    ref = sigma(clean[None], 1)[0]
+    reached = np.any([row(i) <= 2 for i in at], axis=0) if count <= 64 else np.ones(nd, bool)
+    assert np.isnan(s[0][reached]).all()
+    for got in (s[0][~reached], s[1][~reached]):
+        assert (np.abs(got - ref[~reached]) <= REL64 * np.abs(ref).max()).all()
+    check(s[1], ref)
