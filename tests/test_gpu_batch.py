@@ -231,17 +231,21 @@ def test_batch_that_fails_leaves_no_exponents():
         large = L.iscsi_ctx_current()
         cl = torch.randn(1, L.iscsi_ndet(), dtype=torch.float64, device="cuda")
         sl = torch.empty_like(cl)
+        big = c * 1e9
+        _close([c], [c])  # loads the kernels that the comparison below takes
         torch.cuda.synchronize()
         torch.cuda.empty_cache()
         free = torch.cuda.mem_get_info()[0]
         hog = torch.empty(free - (24 << 20), dtype=torch.uint8, device="cuda")  # its lifted vector takes 30 MB
         with pytest.raises(L.IscsiError):
-            L.iscsi_batch_sigma([small, large], [c * 1e9, cl], [s, sl], 1)
+            L.iscsi_batch_sigma([small, large], [big, cl], [s, sl], 1)
+        del hog
+        torch.cuda.empty_cache()
         L.iscsi_ctx_use(small)
         L.iscsi_sigma(c, s, 1)
         torch.cuda.synchronize()
         _close([s], [ref])
     finally:
-        del hog
+        hog = None
         torch.cuda.empty_cache()
         L.iscsi_set_option("autotune", 1)
