@@ -14,7 +14,16 @@
 // costs one reconstruction instead of one per T element (4 of them for 2 + 2
 // electrons, 16 for 4 + 4).  |sigma| is bounded by the units' row 1-norms, taken
 // at set-up, times 2^bc; the moduli are the fewest whose product holds that
-// bound with the largest unit at kCrtUnitBits bits.
+// bound with the largest coefficient at kCrtCBits bits and the largest unit at kCrtUnitBits.
+//
+// kCrtCBits: every coefficient is rounded to 2^-58 of the vector's largest one, so a sigma
+// element that only small coefficients reach is known to 2^-58 max |c| sum_J |H_IJ| and no
+// better.  The slices have an exponent per column (49 bits).  Largest error of an element
+// over its sum |G| |c| (2 + 2 electrons in 10 orbitals, coefficients falling by 10^-D with the
+// excitation level; 50 bits, 12 moduli / 58 bits, 13 moduli / slices): D = 0 4e-15 / 4e-15 /
+// 1.5e-14, 4 4e-13 / 3e-14 / 8e-13, 6 7e-12 / 1e-13 / 3e-12, 8 7e-10 / 5e-12 / 1e-11, 12 5e-8 /
+// 1e-10 / 2e-11; falling along the determinants or at random the 58 bits stay below the
+// slices to D = 12.
 //
 // Order: pairs (p, r) by level, then p, then r, and hole pairs by class, then X,
 // then Y, so that a determinant row's T elements -- rows (p, *), columns (X, *) for
@@ -41,8 +50,10 @@
 
 namespace iscsi {
 
-constexpr int kCrtUnitBits = 49;  // bits of the largest unit (the error-free slices' width)
-constexpr int kCrtCBits = 50;     // bits of the largest coefficient
+constexpr double kCrtUnitBits = 49.9;  // least bits of the largest unit (the error-free slices: 49)
+constexpr int kCrtUnitBitsMax = 52;    // bits that are left over go to the unit up to here, then to the coefficients
+constexpr int kCrtCBits = 58;          // least bits of the largest coefficient
+constexpr int kCrtIntBits = 62;        // integers stay below 2^62 (crt_limbs2)
 
 // ---------------------------------------------------------------------------
 // constants
@@ -77,6 +88,7 @@ CrtMods crt_make_mods(int nm) {
     c.c1[i] = sym(1ll << 13);
     c.c2[i] = sym(1ll << 26);
     c.c3[i] = sym(1ll << 39);
+    c.c4[i] = sym(1ll << 52);
     c.inv[i] = twice(1.0f / (float)m);
     c.neg[i] = twice(-(float)m);
   }
@@ -248,7 +260,7 @@ struct CrtLiftGroup {
   long long base, mod_stride;  // its block of the residue buffer (elements)
 };
 struct CrtOperands {
-  int nvec, ngroups, n, nholeA, nholeB;
+  int nvec, ngroups, n, nholeA, nholeB, cbits;
   CrtLiftGroup g[2 * kMaxElec];
   int blk_start[2 * kMaxElec + 1];  // first block of each group's columns; then the C tiles
   const int *pair, *hp_inv;  // K order -> (q << 16) | s; column order -> X * nholeB + Y (null: the same)
@@ -348,7 +360,7 @@ __global__ void __launch_bounds__(256) k_crt_operands(const __grid_constant__ Cr
       CrtLimbs2 x[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        x[j] = crt_limbs2(crt_fixed(val[2 * j], ex, kCrtCBits), crt_fixed(val[2 * j + 1], ex, kCrtCBits));
+        x[j] = crt_limbs2(crt_fixed(val[2 * j], ex, O.cbits), crt_fixed(val[2 * j + 1], ex, O.cbits));
       crt_store8(x, M, row + (long long)(kc >> 3) * G.bt * CRT_BK + (kc & 7) * 8, G.mod_stride);
     }
     return;
@@ -375,7 +387,7 @@ __global__ void __launch_bounds__(256) k_crt_operands(const __grid_constant__ Cr
     const int R = (tr ? B0 : A0) + r;
     if ((tr ? O.ct : O.ca) == nullptr || R >= (tr ? O.nb : O.na)) continue;
     CrtLimbs2 x[4];
-    auto value = [&](int j) { return crt_fixed(tr ? tile[kc * 8 + j][r] : tile[r][kc * 8 + j], ex, kCrtCBits); };
+    auto value = [&](int j) { return crt_fixed(tr ? tile[kc * 8 + j][r] : tile[r][kc * 8 + j], ex, O.cbits); };
 #pragma unroll
     for (int j = 0; j < 4; ++j) x[j] = crt_limbs2(value(2 * j), value(2 * j + 1));
     const int bt = tr ? O.bt : CRT_BM, rb = R / bt, kb = (tr ? A0 : B0) / CRT_BK;
@@ -753,7 +765,7 @@ struct CrtState {
   DevBuf pair, map, rowrun, colrun, ypos;
   // scales: units are integers of 2^-sh
   CrtMods mods;
-  int sh = 0;
+  int sh = 0, cbits = 0;                // and a vector's coefficients of 2^(e - cbits)
   double bound = 0.0;                   // the bound of |sigma| / max |c| that sh was chosen for
   int g_cut[2] = {-1, 0}, m_cut[2] = {-1, 0};  // moduli and sh of the residues in g_res, ma_res / mb_res
   double rg = 0.0, gmax = 0.0;          // G's row 1-norm and largest element (-1: not taken)
@@ -960,19 +972,21 @@ static double sigma_bound(const Context& ctx, const CrtState& S, int parts, doub
   return 1.000001 * (((parts & 1) ? (double)ctx.na * ctx.nb * S.rg : 0.0) + ((parts & 2) ? rm : 0.0));
 }
 
-// moduli and sh for a bound of |sigma| / max|c|, the largest unit maxel and the
+// moduli, sh and the coefficients' bits for a bound of |sigma| / max|c|, the largest unit maxel and the
 // unit whose bits count
-static void choose_scale(double bound, double maxel, double ref, int& nm, int& sh) {
+static void choose_scale(double bound, double maxel, double ref, int& nm, int& sh, int& cbits) {
   if (bound <= 0.0) bound = 1.0;
   if (maxel <= 0.0) maxel = 1.0;
   if (ref <= 0.0) ref = maxel;
+  const int cap = kCrtIntBits - 1 - (int)std::floor(std::log2(maxel));
   for (nm = 10; nm <= kCrtMaxMods; ++nm) {
     // 2^(sh + bc) bound < M / 2, a hundredth of a bit apart (the roundings of the integers)
-    sh = (int)std::floor(crt_log2_product(nm) - 1.01 - kCrtCBits - std::log2(bound));
-    const int cap = 51 - (int)std::floor(std::log2(maxel));  // integers below 2^52
-    const bool full = sh >= cap;  // more moduli would add nothing
-    sh = std::min(sh, cap);
-    if (nm == kCrtMaxMods || full || sh + std::log2(ref) >= kCrtUnitBits) return;
+    const double room = crt_log2_product(nm) - 1.01 - std::log2(bound);
+    sh = std::min(cap, (int)std::floor(room - kCrtCBits));
+    if (nm < kCrtMaxMods && sh < cap && room - kCrtCBits + std::log2(ref) < kCrtUnitBits) continue;
+    sh = std::min(sh, (int)std::ceil(kCrtUnitBitsMax - std::log2(ref)));
+    cbits = std::min(kCrtIntBits, (int)std::floor(room - sh));
+    return;
   }
 }
 
@@ -1014,7 +1028,7 @@ int crt_matrices_changed(Context& ctx) {
   double rm = 0.0, mmax = 0.0;
   ISCSI_TRY(take_norms(ctx, 2, rm, mmax));
   const double b = sigma_bound(ctx, S, S.parts, rm);
-  if (!(b <= S.bound) || !(std::log2(std::max(mmax, 1e-300)) + S.sh < 52.0)) {
+  if (!(b <= S.bound) || !(std::log2(std::max(mmax, 1e-300)) + S.sh < kCrtIntBits - 1.0)) {
     crt_invalidate(ctx);
     S.m_cut[0] = -1;
     return kOk;
@@ -1028,7 +1042,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   cudaStream_t st = stream();
   const SpinSpace &SA = ctx.sp[0], &SB = ctx.sp[1];
   const int NA = SA.count, NB = SB.count, n = ctx.n;
-  // scale: twice the bound of today's string matrices, so that a per-step one-body term keeps it
+  // scale: 1.25 times the bound of today's string matrices, so that a small per-step one-body term keeps it
   {
     double rm = 0.0, mmax = 0.0;
     ISCSI_TRY(take_norms(ctx, ((parts & 1) && !S.g_norm ? 1 : 0) | (parts & 2), rm, mmax));
@@ -1039,7 +1053,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
       return kErrNoMem;  // the caller takes the slices
     }
     int nm = 0;
-    choose_scale(b, maxel, (parts & 1) ? S.gmax : mmax, nm, S.sh);
+    choose_scale(b, maxel, (parts & 1) ? S.gmax : mmax, nm, S.sh, S.cbits);
     S.bound = b;
     S.mods = crt_make_mods(nm);
   }
@@ -1075,7 +1089,8 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   F.decB = SB.dec.as<int>();
   F.kmax = ctx.kmax;
   F.ni = F.nbuf = 1;
-  F.ebias = -kCrtCBits - S.sh;
+  F.ebias = -S.cbits - S.sh;
+  O.cbits = S.cbits;
   size_t out_elems = 0;
   std::vector<size_t> out_off;
   auto add_out = [&](const CrtProblem& P) {

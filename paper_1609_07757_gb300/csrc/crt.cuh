@@ -20,56 +20,59 @@
 
 namespace iscsi {
 
-// v 2^(bits - e) rounded to an integer, |v| < 2^e, bits <= 53 (in integer
+// v 2^(bits - e) rounded to an integer, |v| < 2^e, bits <= 62 (in integer
 // arithmetic; zeros, subnormals and what is not finite give 0)
 __device__ __forceinline__ long long crt_fixed(double v, int e, int bits) {
   const long long b = __double_as_longlong(v);
   const int E = (int)((b >> 52) & 0x7FF);
   if ((unsigned)(E - 1) >= 0x7FEu) return 0;
   const long long m = (b & 0xFFFFFFFFFFFFFll) | (1ll << 52);
-  const int sh = 1075 - E + e - bits;  // v = m 2^(E - 1075); >= 0 when |v| < 2^e
+  const int sh = 1075 - E + e - bits;  // v = m 2^(E - 1075); >= 53 - bits when |v| < 2^e
   long long N = 0;
-  if (sh <= 0) N = m;  // only sh = 0 occurs
+  if (sh <= 0) N = m << (-sh & 15);
   else if (sh < 55) N = (m + (1ll << (sh - 1))) >> sh;
   return b < 0 ? -N : N;
 }
 
-// Two integers |N| <= 2^52 as N = l0 + l1 2^13 + l2 2^26 + l3 2^39 (0 <= l0, l1,
-// l2 < 2^13), the limbs as packed FP32: a limb in the low mantissa bits of 2^23
-// (l3, signed: added to 1.5 2^23), less that constant.
+// Two integers |N| <= 2^62 as N = l0 + l1 2^13 + l2 2^26 + l3 2^39 + l4 2^52 (0 <= l0 .. l3 < 2^13,
+// |l4| <= 2^10), the limbs as packed FP32: a limb in the low mantissa bits of 2^23 (l4, signed: added to
+// 1.5 2^23), less that constant.
 struct CrtLimbs2 {
-  unsigned long long l0, l1, l2, l3;
+  unsigned long long l0, l1, l2, l3, l4;
 };
 __device__ __forceinline__ CrtLimbs2 crt_limbs2(long long a, long long b) {
   auto mant = [](uint32_t x) { return (x & 0x1FFFu) | 0x4B000000u; };
   auto pair = [](uint32_t lo, uint32_t hi) { return ((unsigned long long)hi << 32) | lo; };
   const unsigned long long k0 = pair(0xCB000000u, 0xCB000000u);  // -2^23, twice
+  const int ah = (int)(a >> 32), bh = (int)(b >> 32);
   CrtLimbs2 r;
   r.l0 = tc::add2(pair(mant((uint32_t)a), mant((uint32_t)b)), k0);
   r.l1 = tc::add2(pair(mant((uint32_t)a >> 13), mant((uint32_t)b >> 13)), k0);
   r.l2 = tc::add2(pair(mant((uint32_t)(a >> 26)), mant((uint32_t)(b >> 26))), k0);
-  r.l3 = tc::add2(pair(0x4B400000u + (uint32_t)((int)(a >> 32) >> 7), 0x4B400000u + (uint32_t)((int)(b >> 32) >> 7)),
+  r.l3 = tc::add2(pair(mant((uint32_t)ah >> 7), mant((uint32_t)bh >> 7)), k0);
+  r.l4 = tc::add2(pair(0x4B400000u + (uint32_t)(ah >> 20), 0x4B400000u + (uint32_t)(bh >> 20)),
                   pair(0xCB400000u, 0xCB400000u));
   return r;
 }
 
 // Residues of eight consecutive K values for every modulus, one 16-byte store
-// each.  t = l0 + l1 c1 + l2 c2 + l3 c3 is congruent to N, an exact FP32 integer
-// (|t| < 2^23); its quotient by m is rounded by adding 1.5 2^23 with an error
-// below 2^-11, under the 1 / (2 m) > 2^-10.1 that separates t / m from a tie, so
+// each.  t = l0 + l1 c1 + .. + l4 c4 is congruent to N, an exact FP32 integer (|t| below
+// 2^22.7); its quotient by m is rounded by adding 1.5 2^23 with an error below 2^-11.5
+// (over the sixteen moduli), under the 1 / (2 m) > 2^-10.1 that separates t / m from a tie, so
 // |t - q m| <= 256 and the upper halves of the floats are the bf16 residues.
-// Packed FP32: 3.5 instructions per residue, where integer arithmetic took ~13
+// Packed FP32: 4 instructions per residue, where integer arithmetic took ~13
 // (4 + 4 electrons in 16 orbitals, operand kernel: 750 us).
 __device__ __forceinline__ void crt_store8(const CrtLimbs2 (&x)[4], const CrtMods& M, __nv_bfloat16* out,
                                            long long mod_stride) {
   const unsigned long long mg = tc::f32x2(12582912.0f, 12582912.0f), ng = tc::f32x2(-12582912.0f, -12582912.0f);
 #pragma unroll 2
   for (int i = 0; i < M.nm; ++i) {
-    const unsigned long long c1 = M.c1[i], c2 = M.c2[i], c3 = M.c3[i], inv = M.inv[i], neg = M.neg[i];
+    const unsigned long long c1 = M.c1[i], c2 = M.c2[i], c3 = M.c3[i], c4 = M.c4[i], inv = M.inv[i], neg = M.neg[i];
     uint32_t pk[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const unsigned long long t = tc::fma2(x[j].l3, c3, tc::fma2(x[j].l2, c2, tc::fma2(x[j].l1, c1, x[j].l0)));
+      const unsigned long long t =
+          tc::fma2(x[j].l4, c4, tc::fma2(x[j].l3, c3, tc::fma2(x[j].l2, c2, tc::fma2(x[j].l1, c1, x[j].l0))));
       const unsigned long long q = tc::add2(tc::fma2(t, inv, mg), ng);
       const unsigned long long r = tc::fma2(q, neg, t);
       pk[j] = __byte_perm((uint32_t)r, (uint32_t)(r >> 32), 0x7632);

@@ -199,3 +199,34 @@ def test_residues_nonfinite(n, na, nb, kmax, count):
     for got in (s[0][~reached], s[1][~reached]):
         assert (np.abs(got - ref[~reached]) <= REL64 * np.abs(ref).max()).all()
     check(s[1], ref)
+
+
+# coefficients that fall over 8 and 12 decades with the excitation level, and along the determinants
+@pytest.mark.parametrize("n,na,nb,kmax", [(10, 2, 2, 4), (12, 2, 2, 3), (7, 3, 3, 6), (14, 2, 1, 3)])
+@pytest.mark.parametrize("how,decades", [("level", 8), ("level", 12), ("index", 12)])
+def test_residues_graded_elements(n, na, nb, kmax, how, decades):
+    """Element by element.  A coefficient is rounded to 2^-58 of the largest one (half a unit of 2^(e - 58) with
+    2^e <= 2 max|c|), a unit of H to 2^-50.9 of the largest opposite-spin one; so sigma_I is off by at most
+    2^-58 max|c| sum_J |H_IJ| + 2^-50.9 g n_u sum_J |c_J| over the J that H reaches, with n_u the units that meet in
+    an element of H (at most na nb + C(na, 2) + C(nb, 2) + na + nb), plus the reference's own rounding,
+    2^-48 sum_J |H_IJ| |c_J| (columns of H from FP64 sums of up to 100 terms)."""
+    h1, eri = make_integrals(n, 7600 + n, ell=3.0, nchol=20)
+    L.iscsi_init(n, na, nb, kmax, h1, eri, 0.0)
+    nd = L.iscsi_ndet()
+    row = excitations(na, nb, kmax)
+    rng = np.random.default_rng(7)
+    fall = row(0) / (na + nb) if how == "level" else np.arange(nd) / nd
+    c = rng.normal(size=nd) * 10.0 ** (-decades * fall)
+    c /= np.linalg.norm(c)
+    s = sigma(c[None], 1)[0]
+    assert L.iscsi_stats()["residues"]["items"] > 0
+    L.iscsi_set_option("fp64_tc", 0)
+    H = np.concatenate([sigma(e, len(e)) for e in np.array_split(np.eye(nd), nd // 64 + 1)])  # symmetric
+    L.iscsi_set_option("fp64_tc", 1)
+    reach = np.stack([row(i) <= 2 for i in range(nd)])
+    absH, absc = np.abs(H), np.abs(c)
+    ref = (H.astype(np.longdouble) * c).sum(axis=1)
+    units = na * nb + na * (na - 1) // 2 + nb * (nb - 1) // 2 + na + nb
+    bar = (2.0 ** -58 * absc.max() * absH.sum(axis=1) + 2.0 ** -50.9 * np.abs(eri).max() * units * (reach @ absc)
+           + 2.0 ** -48 * (absH @ absc))
+    assert (np.abs(s - ref) <= bar).all()
