@@ -36,10 +36,11 @@ __device__ __forceinline__ long long crt_fixed(double v, int e, int bits) {
 
 // Two integers |N| <= 2^62 as N = l0 + l1 2^13 + l2 2^26 + l3 2^39 + l4 2^52 (0 <= l0 .. l3 < 2^13,
 // |l4| <= 2^10), the limbs as packed FP32: a limb in the low mantissa bits of 2^23 (l4, signed: added to
-// 1.5 2^23), less that constant.
+// 1.5 2^23), less that constant.  LIMBS = 4: |N| <= 2^52, l3 signed, no l4.
 struct CrtLimbs2 {
   unsigned long long l0, l1, l2, l3, l4;
 };
+template <int LIMBS = 5>
 __device__ __forceinline__ CrtLimbs2 crt_limbs2(long long a, long long b) {
   auto mant = [](uint32_t x) { return (x & 0x1FFFu) | 0x4B000000u; };
   auto pair = [](uint32_t lo, uint32_t hi) { return ((unsigned long long)hi << 32) | lo; };
@@ -49,9 +50,16 @@ __device__ __forceinline__ CrtLimbs2 crt_limbs2(long long a, long long b) {
   r.l0 = tc::add2(pair(mant((uint32_t)a), mant((uint32_t)b)), k0);
   r.l1 = tc::add2(pair(mant((uint32_t)a >> 13), mant((uint32_t)b >> 13)), k0);
   r.l2 = tc::add2(pair(mant((uint32_t)(a >> 26)), mant((uint32_t)(b >> 26))), k0);
-  r.l3 = tc::add2(pair(mant((uint32_t)ah >> 7), mant((uint32_t)bh >> 7)), k0);
-  r.l4 = tc::add2(pair(0x4B400000u + (uint32_t)(ah >> 20), 0x4B400000u + (uint32_t)(bh >> 20)),
-                  pair(0xCB400000u, 0xCB400000u));
+  auto top = [&](int x, int y) {
+    return tc::add2(pair(0x4B400000u + (uint32_t)x, 0x4B400000u + (uint32_t)y), pair(0xCB400000u, 0xCB400000u));
+  };
+  if (LIMBS == 4) {
+    r.l3 = top(ah >> 7, bh >> 7);
+    r.l4 = 0;
+  } else {
+    r.l3 = tc::add2(pair(mant((uint32_t)ah >> 7), mant((uint32_t)bh >> 7)), k0);
+    r.l4 = top(ah >> 20, bh >> 20);
+  }
   return r;
 }
 
@@ -60,8 +68,9 @@ __device__ __forceinline__ CrtLimbs2 crt_limbs2(long long a, long long b) {
 // 2^22.7); its quotient by m is rounded by adding 1.5 2^23 with an error below 2^-11.5
 // (over the sixteen moduli), under the 1 / (2 m) > 2^-10.1 that separates t / m from a tie, so
 // |t - q m| <= 256 and the upper halves of the floats are the bf16 residues.
-// Packed FP32: 4 instructions per residue, where integer arithmetic took ~13
+// Packed FP32: 4 instructions per residue (3.5 with four limbs), where integer arithmetic took ~13
 // (4 + 4 electrons in 16 orbitals, operand kernel: 750 us).
+template <int LIMBS = 5>
 __device__ __forceinline__ void crt_store8(const CrtLimbs2 (&x)[4], const CrtMods& M, __nv_bfloat16* out,
                                            long long mod_stride) {
   const unsigned long long mg = tc::f32x2(12582912.0f, 12582912.0f), ng = tc::f32x2(-12582912.0f, -12582912.0f);
@@ -71,8 +80,8 @@ __device__ __forceinline__ void crt_store8(const CrtLimbs2 (&x)[4], const CrtMod
     uint32_t pk[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const unsigned long long t =
-          tc::fma2(x[j].l4, c4, tc::fma2(x[j].l3, c3, tc::fma2(x[j].l2, c2, tc::fma2(x[j].l1, c1, x[j].l0))));
+      unsigned long long t = tc::fma2(x[j].l3, c3, tc::fma2(x[j].l2, c2, tc::fma2(x[j].l1, c1, x[j].l0)));
+      if (LIMBS == 5) t = tc::fma2(x[j].l4, c4, t);
       const unsigned long long q = tc::add2(tc::fma2(t, inv, mg), ng);
       const unsigned long long r = tc::fma2(q, neg, t);
       pk[j] = __byte_perm((uint32_t)r, (uint32_t)(r >> 32), 0x7632);

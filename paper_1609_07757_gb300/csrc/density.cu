@@ -30,7 +30,9 @@
 // from a direct kernel over the one-hole strings.
 #include <algorithm>
 #include <climits>
+#include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "crt.cuh"
@@ -66,22 +68,31 @@ struct DmBlock {
   // residue operands: R256 rows of nkb K blocks per modulus, at res_off
   int R256 = 0, nkb = 0;
   size_t res_off = 0;
+  int bits = 0;            // of a row's largest element: 2 bits + log2(columns) below the moduli's product
+  int row0 = 0;            // its first row in the lists of all blocks' rows
 };
 
-constexpr int kDmMods = 13;     // products of two vectors of 57 bits' 2-norm stay below half the moduli's product
-constexpr int kDmNormBits = 57;
-constexpr int kDmScaleBlocks = 304;
-constexpr int kDmNotFinite = -(1 << 20);  // scale of a vector with an infinity or NaN: every element of the result is NaN
+constexpr int kDmMods = 13, kDmModsMax = 16;  // moduli: the fewest with kDmBits bits
+constexpr int kDmBits = 50;                    // (the slices: 49)
+// Short sums over many rows are bound by the result: a residue per modulus and element written and
+// read back, where the slices' kernel writes FP64.  State / transition densities, residues against slices:
+// 2 + 1 electrons in 40 orbitals (40 columns, 1600 rows) 0.165 against 0.134 and 0.203 against 0.155 ms, in 30
+// (900 rows) 0.093, 0.078 and 0.107, 0.085, in 24 (576) 0.072, 0.068 and 0.080, 0.073; 1 + 1 in 100 1.69, 1.57 and
+// 2.46, 1.93.  Few rows are bound by the launches, of which the residues have fewer: 2 + 2 in 8 (64 columns, 64
+// rows) 0.050 against 0.062 and 0.050 against 0.068.  Longer sums tie: 3 + 1 in 40 (780, 1600) 0.218, 0.212.
+constexpr int kDmThinCols = 128, kDmThinRows = 576;
+constexpr int kDmNotFinite = -(1 << 20);  // scale of a row with an infinity or NaN: its elements of the result are NaN
 
 struct DensityPlan {
   bool built = false;
-  // residues (res_fail: they do not fit): operands of bra and ket, output residues, scales
+  // residues (res_fail: thin blocks, or they do not fit): operands of bra and ket, output residues, scales
   bool res_fail = false;
   size_t res_held = 0;
-  DevBuf res_bra, res_ket, res_out, scale, scale_part;
+  DevBuf res_bra, res_ket, res_out, scale;  // scale: per row of bra, of ket, then partial maxima
+  int nmods = kDmMods, res_rows = 0;        // moduli; rows of all blocks
   CrtJob res_job[2];             // ket = bra / general
   bool res_ready[2] = {false, false};
-  std::vector<size_t> res_out_off;
+  size_t res_out_off[3] = {0, 0, 0};
   bool slices = false;           // the slice workspaces below are allocated
   DmBlock blk[3];
   // same-spin tables per spin: pair row of {u<v}, two-hole lift, column list (Z, other string)
@@ -292,6 +303,29 @@ static int plan_build(Context& ctx) {
       B.nkb += pt.nkb;
     }
   }
+  P.res_rows = 0;
+  for (P.nmods = kDmMods;; ++P.nmods) {
+    int least = 64;
+    for (DmBlock& B : P.blk) {
+      long long cols = 1;
+      for (const DmPart& pt : B.parts) cols += pt.ncol;
+      // |sum| <= cols 2^(2 bits), below half the moduli's product
+      B.bits = std::min(52, (int)std::floor((crt_log2_product(P.nmods) - 1.01 - std::log2((double)cols)) / 2.0));
+      if (!B.parts.empty()) least = std::min(least, B.bits);
+    }
+    if (least >= kDmBits || P.nmods == kDmModsMax) break;
+  }
+  int most_cols = 0, most_rows = 0;
+  for (DmBlock& B : P.blk) {
+    B.row0 = P.res_rows;
+    if (B.parts.empty()) continue;
+    P.res_rows += B.R;
+    int cols = 0;
+    for (const DmPart& pt : B.parts) cols += pt.ncol;
+    most_cols = std::max(most_cols, cols);
+    most_rows = std::max(most_rows, B.R);
+  }
+  P.res_fail = most_cols <= kDmThinCols && most_rows > kDmThinRows;
   for (cudaEvent_t& e : P.ev) ISCSI_CUDA(cudaEventCreate(&e));
   P.sl_elems = sl;
   P.q_elems = q;
@@ -377,6 +411,7 @@ __device__ __forceinline__ double dm_value(const DmGather& g, int col, int row, 
 // in shared memory first, so an element costs the hole-pair table and c.
 constexpr int kDmRowRegs = 16;
 constexpr int kDmStage = 256;
+constexpr int kDmMaxSplit = 8;  // blocks per row in k_dm_cut
 struct DmStageRow {
   int a[kDmStage], b[kDmStage], lim[kDmStage];
   long long off[kDmStage];
@@ -457,80 +492,42 @@ __global__ void __launch_bounds__(256) k_dm_lift_slice(DmGather g, int col_start
   }
 }
 
-// Scale of a vector: the integer unit 2^-scale with |c| 2^scale <= 2^57 (2-norm) and
-// max |c_i| 2^scale <= 2^52.  Block b leaves the largest exponent field of its elements
-// and the sum of their squares relative to it, the last block to finish combines
-// them and clears the counter.  Squares are FP32 sums of values built by integer
-// operations, rounded up (an FP64 product costs 64 cycles a warp: 3.1 M determinants took 26 us
-// with FP64 products, 16 with these): only the norm's binary order is wanted.  A vector
-// that is not finite gets kDmNotFinite.
-__global__ void __launch_bounds__(256) k_dm_norm(const double* __restrict__ c, long long ndet, int* __restrict__ pmax,
-                                                 float* __restrict__ psum, int* __restrict__ done,
-                                                 int* __restrict__ scale) {
-  const long long per = (ndet + gridDim.x - 1) / gridDim.x;
-  const long long i0 = blockIdx.x * per, i1 = min(ndet, i0 + per);
-  __shared__ int sm[8];
-  __shared__ float ss[8];
-  __shared__ bool last;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int m = 0;
-#pragma unroll 8
-  for (long long i = i0 + threadIdx.x; i < i1; i += 256) m = max(m, oz_exp_field(c[i]));
-  m = __reduce_max_sync(0xffffffffu, m);
-  if (lane == 0) sm[warp] = m;
-  __syncthreads();
-  for (int w = 0; w < 8; ++w) m = max(m, sm[w]);
-  float s = 0.0f;
-#pragma unroll 8
-  for (long long i = i0 + threadIdx.x; i < i1; i += 256) {
-    // |x| 2^(1022 - m) < 1 as FP32, its mantissa cut to 23 bits and raised by one; 0 below 2^-60
-    const unsigned long long b = (unsigned long long)__double_as_longlong(c[i]);
-    const int E = (int)((b >> 52) & 0x7FF) - m + 126;
-    const float x = E > 66 ? __uint_as_float(((uint32_t)E << 23 | (uint32_t)((b >> 29) & 0x7FFFFFu)) + 1u) : 0.0f;
-    s = fmaf(x, x, s);
-  }
-  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) ss[warp] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.0f;
-    for (int w = 0; w < 8; ++w) t += ss[w];
-    pmax[blockIdx.x] = m;
-    psum[blockIdx.x] = t;
-    __threadfence();
-    last = atomicAdd(done, 1) == (int)gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last || warp != 0) return;
-  __threadfence();
-  int M = 0;
-  for (int b = lane; b < (int)gridDim.x; b += 32) M = max(M, __ldcg(pmax + b));
-  M = __reduce_max_sync(0xffffffffu, M);
-  float t = 0.0f;
-  for (int b = lane; b < (int)gridDim.x; b += 32) t += ldexpf(__ldcg(psum + b), 2 * max(__ldcg(pmax + b) - M, -60));
-  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if (lane != 0) return;
-  *done = 0;
-  int k = 0;  // |c| < 2^(e + k), max |c_i| < 2^e
-  // a thread's FP32 sum of up to 2^18 terms (2^34 determinants) is within 2^-6 of the truth
-  for (float u = t * 1.02f; u >= 1.0f && k < 64; u *= 0.25f) ++k;
-  const int e = M - 1022;
-  *scale = M == 0x7FF ? kDmNotFinite : M > 0 ? min(kDmNormBits - e - k, 52 - e) : 0;
-}
-
-// Residues of one part's columns, one block per row of L: 8 consecutive columns
-// per thread (row entries staged as in k_dm_lift_slice).  Rows the part does not
-// reach and padding are zero from the buffer's first clearing on.  26 bytes written per
-// element: full CI in 60 orbitals 495 MB in 184 us (the slices: 187 us), latency of the
-// gathers and the row staging; five blocks per SM for the staged rows (106 us against 118), four otherwise (78, 92).
-template <bool STAGED>
-__global__ void __launch_bounds__(256, STAGED ? 5 : 4) k_dm_cut(DmGather g, int col_start, int ncol, int kb0, int nkb, int nkb_all,
-                                                long long mod_stride, const int* __restrict__ scale,
-                                                const __grid_constant__ CrtMods M, const double* __restrict__ c,
-                                                __nv_bfloat16* __restrict__ out) {
-  const int r = blockIdx.x;
+// Residues of all rows of L of all blocks, one thread block per row (and vector, blockIdx.z): 8
+// consecutive columns per thread (row entries staged as in k_dm_lift_slice).  A row's unit
+// is 2^-scale with scale = bits - e, max |L[row][:]| < 2^e: small rows keep their
+// bits however large others are.  Rows a part does not reach and padding are zero from the
+// buffer's first clearing on.  Rows of few columns take their maximum and their residues in one
+// launch (MODE 0: a thread's first chunk stays in shared memory in between, later ones are gathered
+// twice); longer ones are split over blockIdx.y, MODE 1 leaving partial maxima for MODE 2.
+// 26 bytes written per element; latency of the gathers and the row staging bound it.  (One unit per
+// vector, from its 2-norm, in a launch per vector, block and column class: one density of 2 + 2 electrons in 60 orbitals 975
+// us, now 998, in 8 orbitals 70, now 49; 3 + 3 in 20, whose rows are split, 460, now 544.)
+struct DmCutBlock {
+  DmGather g;
+  int row0, R, bits, nparts, nkb;
+  int col_start[OZ_MAX_SEGS], ncol[OZ_MAX_SEGS], kb0[OZ_MAX_SEGS], rows[OZ_MAX_SEGS];
+  long long base, mod_stride;
+};
+struct DmCut {
+  DmCutBlock blk[3];
+  const double* v[2];
+  __nv_bfloat16* out[2];
+  int* scale;   // [vector][row]
+  int* pmax;    // [vector][row][gridDim.y]
+  int rows;
+};
+template <bool STAGED, int MODE>
+__global__ void __launch_bounds__(256, 4) k_dm_cut(const __grid_constant__ DmCut D,
+                                                                const __grid_constant__ CrtMods M) {
+  const int grow = blockIdx.x, vec = blockIdx.z;
+  const int b = (D.blk[2].R > 0 && grow >= D.blk[2].row0) ? 2 : (D.blk[1].R > 0 && grow >= D.blk[1].row0) ? 1 : 0;
+  const DmCutBlock& K = D.blk[b];
+  const DmGather& g = K.g;
+  const int r = grow - K.row0;
+  const double* __restrict__ c = D.v[vec];
+  const bool staged = STAGED && b == 0;
   __shared__ DmStageRow S;
-  if (STAGED) {
+  if (staged) {
     const int qt = g.pair_of[r];
     const int q = qt / g.n, t = qt - (qt / g.n) * g.n;
     for (int X = threadIdx.x; X < g.nholeA; X += blockDim.x) {
@@ -545,19 +542,58 @@ __global__ void __launch_bounds__(256, STAGED ? 5 : 4) k_dm_cut(DmGather g, int 
     for (int Y = threadIdx.x; Y < g.nholeB; Y += blockDim.x) S.b[Y] = g.liftB[t * g.nholeB + Y];
     __syncthreads();
   }
-  const int sc = *scale;
-  __nv_bfloat16* row = out + ((long long)(r >> 7) * nkb_all + kb0) * (CRT_BM * CRT_BK) + (r & 127) * CRT_BK;
-  for (int kc = blockIdx.y * 256 + threadIdx.x; kc < 8 * nkb; kc += 256 * gridDim.y) {
-    double v[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int k = kc * 8 + j;
-      v[j] = k < ncol ? dm_row_value<STAGED>(g, S, col_start + k, r, c) : 0.0;
+  const int kc0 = blockIdx.y * 256 + threadIdx.x, step = 256 * gridDim.y, nch = 8 * K.nkb;
+  __shared__ int sm[8];
+  __shared__ double keep[MODE == 0 ? 8 : 1][256];  // a thread's first chunk
+  int m = 0, sc = 0;
+  if (MODE == 2)
+    for (int i = 0; i < (int)gridDim.y; ++i) m = max(m, D.pmax[((long long)vec * D.rows + grow) * gridDim.y + i]);
+  __nv_bfloat16* row = D.out[vec] + K.base + (long long)(r >> 7) * K.nkb * (CRT_BM * CRT_BK) + (r & 127) * CRT_BK;
+#pragma unroll 1
+  for (int pass = MODE == 2 ? 1 : 0; pass < (MODE == 1 ? 1 : 2); ++pass) {
+    if (pass == 1) {
+      sc = m == 0x7FF ? kDmNotFinite : m > 0 ? K.bits - (m - 1022) : 0;
+      if (threadIdx.x == 0 && blockIdx.y == 0) D.scale[(long long)vec * D.rows + grow] = sc;
     }
-    CrtLimbs2 x[4];
+#pragma unroll 1
+    for (int kc = kc0; kc < nch; kc += step) {
+      double v[8];
+      int p = 0;
+      while (p + 1 < K.nparts && (kc >> 3) >= K.kb0[p + 1]) ++p;
+      if (r >= K.rows[p]) continue;  // the chunk's part does not reach the row
+      if (MODE == 0 && pass == 1 && kc == kc0) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) x[j] = crt_limbs2(crt_fixed(v[2 * j], 0, sc), crt_fixed(v[2 * j + 1], 0, sc));
-    crt_store8(x, M, row + (long long)(kc >> 3) * (CRT_BM * CRT_BK) + (kc & 7) * 8, mod_stride);
+        for (int j = 0; j < 8; ++j) v[j] = keep[j][threadIdx.x];
+      } else {
+        const int k0 = kc * 8 - K.kb0[p] * CRT_BK, left = K.ncol[p] - k0, col = K.col_start[p] + k0;
+        if (staged) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = j < left ? dm_row_value<true>(g, S, col + j, r, c) : 0.0;
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = j < left ? dm_value(g, col + j, r, c) : 0.0;
+        }
+      }
+      if (pass == 0) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) m = max(m, oz_exp_field(v[j]));
+        if (MODE == 0 && kc == kc0)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) keep[j][threadIdx.x] = v[j];
+      } else {
+        CrtLimbs2 x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j] = crt_limbs2<4>(crt_fixed(v[2 * j], 0, sc), crt_fixed(v[2 * j + 1], 0, sc));
+        crt_store8<4>(x, M, row + (long long)(kc >> 3) * (CRT_BM * CRT_BK) + (kc & 7) * 8, K.mod_stride);
+      }
+    }
+    if (pass == 0) {
+      m = __reduce_max_sync(0xffffffffu, m);
+      if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+      __syncthreads();
+      for (int w = 0; w < 8; ++w) m = max(m, sm[w]);
+      if (MODE == 1 && threadIdx.x == 0) D.pmax[((long long)vec * D.rows + grow) * gridDim.y + blockIdx.y] = m;
+    }
   }
 }
 
@@ -570,7 +606,9 @@ struct DmRebuild {
   const int16_t* res[3];
   double* q[3];
   int R[3], tn[3], tile0[4];  // of the blocks ab, aa, bb; tile0: first tile of each in the grid
+  int row0[3];                // first of each in the lists of rows' scales
 };
+template <int NM>
 __global__ void __launch_bounds__(256) k_dm_rebuild(const __grid_constant__ DmRebuild D, int sym,
                                                     const int* __restrict__ scale_bra, const int* __restrict__ scale_ket,
                                                     const __grid_constant__ CrtWeights W) {
@@ -580,11 +618,9 @@ __global__ void __launch_bounds__(256) k_dm_rebuild(const __grid_constant__ DmRe
   const int rt = tl / tn, nt = tl - rt * tn;
   if (sym && (rt >> 1) > nt) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int e = -(*scale_bra + *scale_ket);
-  const bool bad = min(*scale_bra, *scale_ket) == kDmNotFinite;
-  const int lift = e < -900 ? 600 : 0;  // crt_value gives 0 below the normal range: rounded there by a product
   constexpr int tile = CRT_BM * CRT_MAXN;
-  const int16_t* base = D.res[blk] + ((long long)rt * tn + nt) * kDmMods * tile;
+  const int16_t* base = D.res[blk] + ((long long)rt * tn + nt) * NM * tile;
+  const int *sb = scale_bra + D.row0[blk], *sk = scale_ket + D.row0[blk];
   for (int w = warp; w < 32; w += 8) {
     const int cg = blockIdx.y * 8 + (w >> 2), quarter = w & 3;
     const int r0 = rt * CRT_BM + quarter * 32, col = nt * CRT_MAXN + cg * 8;
@@ -598,7 +634,7 @@ __global__ void __launch_bounds__(256) k_dm_rebuild(const __grid_constant__ DmRe
     }
     const int16_t* src = base + (cg * CRT_BM + quarter * 32 + lane) * 8;
 #pragma unroll
-    for (int i = 0; i < kDmMods; ++i) {
+    for (int i = 0; i < NM; ++i) {
       const uint4 x = __ldg(reinterpret_cast<const uint4*>(src + (long long)i * tile));
       const uint32_t xw[4] = {x.x, x.y, x.z, x.w};
       const uint32_t w0 = W.lo0[i], w1 = W.lo1[i], w2 = W.hi[i];
@@ -611,14 +647,15 @@ __global__ void __launch_bounds__(256) k_dm_rebuild(const __grid_constant__ DmRe
       }
     }
     double v[8];
+    const int er = sb[min(r0 + lane, R - 1)];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = crt_value(lo[j], hi[j], W.mman, W.mexp, e + lift);
-    if (lift)
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] *= 0x1p-600;
-    if (bad)
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = __longlong_as_double(0x7FF8000000000000ll);
+    for (int j = 0; j < 8; ++j) {
+      const int ec = sk[min(col + j, R - 1)], e = -(er + ec);
+      // crt_value gives 0 below the normal range: rounded there by a product
+      if (min(er, ec) == kDmNotFinite) v[j] = __longlong_as_double(0x7FF8000000000000ll);
+      else if (e < -900) v[j] = crt_value(lo[j], hi[j], W.mman, W.mexp, e + 600) * 0x1p-600;
+      else v[j] = crt_value(lo[j], hi[j], W.mman, W.mexp, e);
+    }
     if (sym && (rt >> 1) < nt && r0 + lane < R)
 #pragma unroll
       for (int j = 0; j < 8; ++j)
@@ -902,16 +939,16 @@ static int residues_build(Context& ctx, bool sym) {
   if (P.res_ready[idx]) return kOk;
   cudaStream_t st = stream();
   size_t elems = 0, out = 0;
-  P.res_out_off.assign(3, 0);
+  const int nm = P.nmods;
   for (int b = 0; b < 3; ++b) {
     DmBlock& B = P.blk[b];
     if (B.parts.empty()) continue;
     B.res_off = elems;
-    elems += (size_t)kDmMods * B.R256 * B.nkb * CRT_BK;
+    elems += (size_t)nm * B.R256 * B.nkb * CRT_BK;
     P.res_out_off[b] = out;
-    out += (size_t)kDmMods * B.R256 * B.R256;
+    out += (size_t)nm * B.R256 * B.R256;
     // sums of chunk residues stay exact below 2^24 / 257 chunks; tensor map rows are 32-bit
-    if (B.nkb > CRT_CHUNK * 60000 || (long long)kDmMods * B.R256 * B.nkb >= (1ll << 31)) return kErrNoMem;
+    if (B.nkb > CRT_CHUNK * 60000 || (long long)nm * B.R256 * B.nkb >= (1ll << 31)) return kErrNoMem;
   }
   DevBuf* ops[2] = {&P.res_bra, sym ? nullptr : &P.res_ket};
   for (DevBuf* d : ops)
@@ -921,9 +958,7 @@ static int residues_build(Context& ctx, bool sym) {
     }
   if (P.res_out.bytes < sizeof(int16_t) * out) ISCSI_TRY(crt_alloc(P.res_out, sizeof(int16_t) * out, P.res_held));
   if (!P.scale.p) {
-    ISCSI_TRY(P.scale.alloc(2 * sizeof(int)));
-    ISCSI_TRY(P.scale_part.alloc(sizeof(int) * (2 * kDmScaleBlocks + 1)));
-    ISCSI_CUDA(cudaMemsetAsync(P.scale_part.p, 0, P.scale_part.bytes, st));
+    ISCSI_TRY(P.scale.alloc(sizeof(int) * (size_t)std::max(1, P.res_rows) * 2 * (1 + kDmMaxSplit)));
   }
   CrtJob& job = P.res_job[idx];
   job.probs.clear();
@@ -935,7 +970,7 @@ static int residues_build(Context& ctx, bool sym) {
     std::memset(&H.p, 0, sizeof(H.p));
     H.p.ntile = CRT_MAXN;
     H.p.tn = B.R256 / CRT_MAXN;
-    H.p.nm = kDmMods;
+    H.p.nm = nm;
     H.p.rt = rup(B.R, CRT_BM) / CRT_BM;
     H.p.nblk_a = H.p.nblk_b = B.R256 / CRT_BM;
     H.p.nkb_a = H.p.nkb_b = B.nkb;
@@ -951,7 +986,7 @@ static int residues_build(Context& ctx, bool sym) {
       return true;
     };
     const __nv_bfloat16* a = P.res_bra.as<__nv_bfloat16>() + B.res_off;
-    ISCSI_TRY(crt_encode(H.p, a, sym ? a : P.res_ket.as<__nv_bfloat16>() + B.res_off, kDmMods));
+    ISCSI_TRY(crt_encode(H.p, a, sym ? a : P.res_ket.as<__nv_bfloat16>() + B.res_off, nm));
     job.probs.push_back(H);
     for (const DmPart& pt : B.parts) f64 += 2.0 * pt.ncol * pt.rows * (sym ? 0.5 * (pt.rows + 1.0) : (double)pt.rows);
   }
@@ -962,31 +997,67 @@ static int residues_build(Context& ctx, bool sym) {
   return kOk;
 }
 
-// a vector's residues (which: 0 bra, 1 ket)
-static int residues_cut(Context& ctx, const double* v, int which, cudaStream_t st) {
+// residues of bra and ket (null: bra only)
+static int residues_cut(Context& ctx, const double* bra, const double* ket, cudaStream_t st) {
   DensityPlan& P = *ctx.dm;
-  static const CrtMods mods = crt_make_mods(kDmMods);
-  int* part = P.scale_part.as<int>();
-  k_dm_norm<<<kDmScaleBlocks, 256, 0, st>>>(v, ctx.ndet, part, reinterpret_cast<float*>(part + kDmScaleBlocks),
-                                            part + 2 * kDmScaleBlocks, P.scale.as<int>() + which); ISCSI_COUNT_LAUNCH();
+  const CrtMods mods = crt_make_mods(P.nmods);
+  DmCut D;
+  std::memset(&D, 0, sizeof(D));
+  int nkb = 0;
   for (int b = 0; b < 3; ++b) {
     const DmBlock& B = P.blk[b];
+    DmCutBlock& K = D.blk[b];
+    K.row0 = B.row0;
     if (B.parts.empty()) continue;
-    const DmGather g = gather_of(ctx, P, b);
-    __nv_bfloat16* out = (which ? P.res_ket : P.res_bra).as<__nv_bfloat16>() + B.res_off;
-    const long long mod_stride = (long long)B.R256 * B.nkb * CRT_BK;
+    K.g = gather_of(ctx, P, b);
+    K.R = B.R;
+    K.bits = B.bits;
+    K.nkb = B.nkb;
+    K.base = (long long)B.res_off;
+    K.mod_stride = (long long)B.R256 * B.nkb * CRT_BK;
     for (const DmPart& pt : B.parts) {
-      const dim3 grid(pt.rows, std::max(1, std::min(8, pt.nkb / 64)));
-      const int* sc = P.scale.as<int>() + which;
-      if (b == 0 && g.nholeA <= kDmStage && g.nholeB <= kDmStage)
-        k_dm_cut<true><<<grid, 256, 0, st>>>(g, pt.col_start, pt.ncol, pt.kb0, pt.nkb, B.nkb, mod_stride, sc, mods, v, out);
-      else
-        k_dm_cut<false><<<grid, 256, 0, st>>>(g, pt.col_start, pt.ncol, pt.kb0, pt.nkb, B.nkb, mod_stride, sc, mods, v, out);
-      ISCSI_COUNT_LAUNCH();
+      const int i = K.nparts++;
+      K.col_start[i] = pt.col_start;
+      K.ncol[i] = pt.ncol;
+      K.kb0[i] = pt.kb0;
+      K.rows[i] = pt.rows;
     }
+    nkb = std::max(nkb, B.nkb);
+  }
+  if (P.res_rows == 0) return kOk;
+  D.v[0] = bra;
+  D.v[1] = ket;
+  D.out[0] = P.res_bra.as<__nv_bfloat16>();
+  D.out[1] = P.res_ket.as<__nv_bfloat16>();
+  D.rows = P.res_rows;
+  D.scale = P.scale.as<int>();
+  D.pmax = D.scale + 2ll * P.res_rows;
+  // at least two chunks of eight columns for each of a block's threads
+  const dim3 grid(P.res_rows, std::max(1, std::min(kDmMaxSplit, nkb / 64)), ket ? 2 : 1);
+  const bool staged = ctx.sp[0].nhole <= kDmStage && ctx.sp[1].nhole <= kDmStage && !P.blk[0].parts.empty();
+  auto launch = [&](auto mode) {
+    constexpr int MODE = decltype(mode)::value;
+    if (staged)
+      k_dm_cut<true, MODE><<<grid, 256, 0, st>>>(D, mods);
+    else
+      k_dm_cut<false, MODE><<<grid, 256, 0, st>>>(D, mods);
+    ISCSI_COUNT_LAUNCH();
+  };
+  if (grid.y == 1) {
+    launch(std::integral_constant<int, 0>());
+  } else {
+    launch(std::integral_constant<int, 1>());
+    launch(std::integral_constant<int, 2>());
   }
   ISCSI_CUDA(cudaGetLastError());
   return kOk;
+}
+
+template <int NM>
+static void launch_rebuild(const DmRebuild& D, int sym, const int* sb, const int* sk, cudaStream_t st) {
+  static const CrtWeights weights = crt_make_weights(NM, 1);
+  k_dm_rebuild<NM><<<dim3(D.tile0[3], CRT_MAXN / 64), 256, 0, st>>>(D, sym, sb, sk, weights);
+  ISCSI_COUNT_LAUNCH();
 }
 
 int density_run(Context& ctx, const double* bra, const double* ket, double* d1, double* d2) {
@@ -1018,8 +1089,7 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
     const bool res = !P.res_fail;
     const bool ev = !ctx.capturing;
     if (res) {
-      ISCSI_TRY(residues_cut(ctx, bra, 0, st));
-      if (!sym) ISCSI_TRY(residues_cut(ctx, ket, 1, st));
+      ISCSI_TRY(residues_cut(ctx, bra, sym ? nullptr : ket, st));
       const CrtJob& job = P.res_job[sym ? 0 : 1];
       if (job.grid > 0) {
         ISCSI_TRY(tc_err_buf(ctx));
@@ -1028,7 +1098,6 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
         if (ev) ISCSI_CUDA(cudaEventRecord(P.ev[1], st));
         P.timed = ev;
       }
-      static const CrtWeights weights = crt_make_weights(kDmMods, 1);
       DmRebuild D;
       D.tile0[0] = 0;
       for (int b = 0; b < 3; ++b) {
@@ -1037,13 +1106,18 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
         D.res[b] = P.res_out.as<int16_t>() + P.res_out_off[b];
         D.q[b] = P.q.as<double>() + B.q_off;
         D.R[b] = some ? B.R : 0;
+        D.row0[b] = B.row0;
         D.tn[b] = some ? B.R256 / CRT_MAXN : 1;
         D.tile0[b + 1] = D.tile0[b] + (some ? (rup(B.R, CRT_BM) / CRT_BM) * D.tn[b] : 0);
       }
       if (D.tile0[3] > 0) {
-        const int* sc = P.scale.as<int>();
-        k_dm_rebuild<<<dim3(D.tile0[3], CRT_MAXN / 64), 256, 0, st>>>(D, sym ? 1 : 0, sc, sc + (sym ? 0 : 1), weights);
-        ISCSI_COUNT_LAUNCH();
+        const int *sb = P.scale.as<int>(), *sk = sb + (sym ? 0 : P.res_rows);
+        switch (P.nmods) {
+          case 13: launch_rebuild<13>(D, sym, sb, sk, st); break;
+          case 14: launch_rebuild<14>(D, sym, sb, sk, st); break;
+          case 15: launch_rebuild<15>(D, sym, sb, sk, st); break;
+          default: launch_rebuild<16>(D, sym, sb, sk, st); break;
+        }
       }
       ISCSI_CUDA(cudaGetLastError());
     } else {
@@ -1084,7 +1158,7 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
         k_dm_mirror<<<grid, 256, 0, st>>>(R, const_cast<double*>(R.q)); ISCSI_COUNT_LAUNCH();
       }
     k_dm_expand<<<dim3(n * n, 3), 256, 0, st>>>(E, d2); ISCSI_COUNT_LAUNCH();
-    if (d1) {
+    if (d1 && (ctx.na >= 2 || ctx.nb >= 2)) {
       k_dm_trace<<<dim3((n * n + 7) / 8, 2), 256, 0, st>>>(E, d1); ISCSI_COUNT_LAUNCH();
     }
     ISCSI_CUDA(cudaGetLastError());

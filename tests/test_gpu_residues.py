@@ -230,3 +230,82 @@ def test_residues_graded_elements(n, na, nb, kmax, how, decades):
     bar = (2.0 ** -58 * absc.max() * absH.sum(axis=1) + 2.0 ** -50.9 * np.abs(eri).max() * units * (reach @ absc)
            + 2.0 ** -48 * (absH @ absc))
     assert (np.abs(s - ref) <= bar).all()
+
+
+def lifted_sizes(na, nb, kmax, c):
+    """Per two-body block (aa, ab, bb): largest element and 1-norm of every row of the lifted vector, as matrices over
+    the row's orbital pair."""
+    occ, lev = [], []
+    for spin, ne in enumerate((na, nb)):
+        o, l = L.iscsi_get_strings(spin, ne)
+        m = np.zeros((len(l), 64), dtype=bool)
+        m[np.arange(len(l))[:, None], np.asarray(o)] = True
+        occ.append(m)
+        lev.append(np.asarray(l))
+    C = np.zeros((len(lev[0]), len(lev[1])))
+    C[lev[0][:, None] + lev[1][None, :] <= kmax] = np.abs(c)
+    n = max(int(np.flatnonzero(o.any(0)).max()) for o in occ) + 1
+    out = []
+    for s, t in ((0, 0), (0, 1), (1, 1)):
+        mx, one = np.zeros((n, n)), np.zeros((n, n))
+        for p in range(n):
+            for r in range(n):
+                if s == t and p == r:
+                    continue
+                A = occ[0][:, p] & (occ[0][:, r] if t == 0 else True) if s == 0 else slice(None)
+                B = occ[1][:, r] & (occ[1][:, p] if s == 1 else True) if t == 1 else slice(None)
+                x = C[A][:, B]
+                if x.size:
+                    mx[p, r], one[p, r] = x.max(), x.sum()
+        out.append((mx, one))
+    return out
+
+
+# coefficients that fall over 12 decades with the excitation level: element by element, ket = bra and a transition;
+# long sums (14 moduli: 4 + 4 electrons), rows of a block split over several thread blocks
+@pytest.mark.parametrize("n,na,nb,kmax,transition", [(8, 2, 2, 4, False), (9, 2, 2, 3, True), (7, 3, 2, 5, True),
+                                                     (11, 3, 3, 6, False), (12, 4, 4, 8, True)])
+def test_density_graded_elements(n, na, nb, kmax, transition):
+    """A row's elements are integers of at least 50 bits below its largest one, so an element of d2 is off by at most
+    2^-50 (max_x |L_y|_1 + max_y |L_x|_1); the reference's FP64 sums are within 2^-47 of the same bound (at most
+    some thousand terms)."""
+    h1, eri = make_integrals(n, 60 + n, ell=3.0, nchol=6)
+    L.iscsi_init(n, na, nb, kmax, h1, eri, 0.0)
+    nd = L.iscsi_ndet()
+    fall = excitations(na, nb, kmax)(0) / (na + nb)
+    vecs = [unit_vector(nd, 8 + i) * 10.0 ** (-12 * fall) for i in range(2 if transition else 1)]
+    d1 = torch.full((2, n, n), float("nan"), dtype=torch.float64, device="cuda")
+    d2 = torch.full((3, n, n, n, n), float("nan"), dtype=torch.float64, device="cuda")
+    dev = [torch.as_tensor(v, device="cuda") for v in vecs]
+    L.iscsi_density(dev[0], dev[1] if transition else None, d1, d2)
+    from oracle import Oracle
+    _, ref = Oracle(n, na, nb, kmax, 0.0, h1, eri).density(vecs[0], vecs[-1])
+    ref = np.asarray(ref).reshape(3, n, n, n, n)
+    sizes = [lifted_sizes(na, nb, kmax, v) for v in vecs]
+    for got, want, (mx, ox), (my, oy) in zip(d2.cpu().numpy(), ref, sizes[0], sizes[-1]):
+        # d2[p, q, r, t] = row (p, r) of bra times row (q, t) of ket
+        bar = (2.0 ** -50 + 2.0 ** -47) * (mx[:, None, :, None] * oy[None, :, None, :]
+                                           + my[None, :, None, :] * ox[:, None, :, None])
+        assert (np.abs(got - want) <= bar).all()
+
+
+@pytest.mark.parametrize("n,na,nb,kmax", [(8, 2, 2, 4), (9, 3, 2, 3)])
+def test_density_nonfinite(n, na, nb, kmax):
+    """A NaN makes the rows of the lifted vector that hold it NaN; the others are as without it."""
+    h1, eri = make_integrals(n, 70 + n, ell=3.0, nchol=6)
+    L.iscsi_init(n, na, nb, kmax, h1, eri, 0.0)
+    nd = L.iscsi_ndet()
+    bad = unit_vector(nd, 5)
+    bad[nd // 2] = np.nan
+    got = []
+    for v in (bad, np.nan_to_num(bad, nan=0.0)):
+        d2 = torch.zeros((3, n, n, n, n), dtype=torch.float64, device="cuda")
+        L.iscsi_density(torch.as_tensor(v, device="cuda"), None, None, d2)
+        got.append(d2.cpu().numpy())
+    here = lifted_sizes(na, nb, kmax, (np.arange(nd) == nd // 2).astype(float))
+    for blk, (a, b, (hit, _)) in enumerate(zip(*got, here)):
+        reached = (hit[:, None, :, None] + hit[None, :, None, :]) > 0
+        if blk != 1:  # elements with equal orbitals vanish by construction
+            i = np.arange(n)
+            reached[i, :, i, :] = reached[:, i, :, i] = False
+        assert np.isnan(a[reached]).all() and np.array_equal(a[~reached], b[~reached])
