@@ -902,10 +902,25 @@ bool crt_ab_active(Context& ctx, int nvec) {
   return good >= 0.9 * heavy && S.groups[0].rows >= kCrtMinRows;
 }
 
+// Strings of the space: alpha strings with an allowed beta string, and the longest allowed beta
+// prefix (both are sorted by level).  A truncated space of many electrons reaches few of all strings (4 + 4
+// electrons in 30 orbitals, doubles: 2055 of 27405), and the string matrices are cut for these alone.
+static int alpha_strings(const Context& ctx) {
+  int l = 0;
+  while (l <= ctx.sp[0].maxlevel && ctx.nb_allowed_lvl[l] > 0) ++l;
+  return ctx.sp[0].level_start[l];
+}
+static int beta_strings(const Context& ctx) {
+  long long most = 0;
+  for (int l = 0; l <= ctx.sp[0].maxlevel; ++l)
+    if (ctx.sp[0].level_start[l + 1] > ctx.sp[0].level_start[l]) most = std::max(most, ctx.nb_allowed_lvl[l]);
+  return (int)most;
+}
+
 // the same-spin products, all levels at once, when the strings fill a tile or so
 bool crt_ss_active(Context& ctx, int nvec) {
   CrtState& S = crt_state(ctx);
-  return !S.off && nvec <= kCrtMaxVecs && ctx.sp[0].count >= kCrtMinRows && ctx.sp[1].count >= kCrtMinRows;
+  return !S.off && nvec <= kCrtMaxVecs && alpha_strings(ctx) >= kCrtMinRows && beta_strings(ctx) >= kCrtMinRows;
 }
 
 int crt_encode(CrtProblem& P, const void* a, const void* b, int nm) {
@@ -943,14 +958,14 @@ static int take_norms(Context& ctx, int what, double& rm, double& mmax) {
     k_crt_norms<<<ctx.npairs, 256, 0, st>>>(ctx.G64.as<double>(), ctx.npairs, ctx.npairs, 0, d); ISCSI_COUNT_LAUNCH();
   }
   if ((what & 2) && ctx.na > 0 && ctx.M64[0].p) {
-    const int NA = ctx.sp[0].count;
-    k_crt_norms<<<NA, 256, 0, st>>>(ctx.M64[0].as<double>(), NA, NA, 0, d + 2); ISCSI_COUNT_LAUNCH();
+    const int NA = alpha_strings(ctx);
+    k_crt_norms<<<NA, 256, 0, st>>>(ctx.M64[0].as<double>(), NA, ctx.sp[0].count, 0, d + 2); ISCSI_COUNT_LAUNCH();
   }
   if ((what & 2) && ctx.nb > 0) {
     int trans = 0;
     const double* Mb = beta_matrix(ctx, trans);
-    const int NB = ctx.sp[1].count;
-    k_crt_norms<<<NB, 256, 0, st>>>(Mb, NB, NB, trans, d + 4); ISCSI_COUNT_LAUNCH();
+    const int NB = beta_strings(ctx);
+    k_crt_norms<<<NB, 256, 0, st>>>(Mb, NB, ctx.sp[1].count, trans, d + 4); ISCSI_COUNT_LAUNCH();
   }
   ISCSI_CUDA(cudaGetLastError());
   double h[6];
@@ -994,14 +1009,14 @@ static void choose_scale(double bound, double maxel, double ref, int& nm, int& s
 static int crt_cut_m(Context& ctx) {
   CrtState& S = *ctx.crt;
   cudaStream_t st = stream();
-  const int NA = ctx.sp[0].count, NB = ctx.sp[1].count;
+  const int NA = alpha_strings(ctx), NB = beta_strings(ctx);
   const int ntile = tile_cols(NB), bt = ntile / 2, tn = (NB + ntile - 1) / ntile;
   const int ka = up(NA, CRT_BK) / CRT_BK, kb = up(NB, CRT_BK) / CRT_BK;
   if (ctx.na > 0 && ctx.M64[0].p) {
     const int rp = up(NA, 2 * CRT_BM);
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)S.mods.nm * rp * ka * CRT_BK;
     if (S.ma_res.bytes < bytes) ISCSI_TRY(crt_alloc(S.ma_res, bytes, S.held));
-    ISCSI_TRY(cut_matrix(ctx.M64[0].as<double>(), NA, NA, NA, 0, nullptr, S.sh, CRT_BM, rp, ka, S.mods,
+    ISCSI_TRY(cut_matrix(ctx.M64[0].as<double>(), NA, NA, ctx.sp[0].count, 0, nullptr, S.sh, CRT_BM, rp, ka, S.mods,
                          S.ma_res.as<__nv_bfloat16>(), st));
   }
   if (ctx.nb > 0) {
@@ -1010,7 +1025,8 @@ static int crt_cut_m(Context& ctx) {
     const int rp = tn * ntile;
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)S.mods.nm * rp * kb * CRT_BK;
     if (S.mb_res.bytes < bytes) ISCSI_TRY(crt_alloc(S.mb_res, bytes, S.held));
-    ISCSI_TRY(cut_matrix(Mb, NB, NB, NB, trans, nullptr, S.sh, bt, rp, kb, S.mods, S.mb_res.as<__nv_bfloat16>(), st));
+    ISCSI_TRY(cut_matrix(Mb, NB, NB, ctx.sp[1].count, trans, nullptr, S.sh, bt, rp, kb, S.mods,
+                         S.mb_res.as<__nv_bfloat16>(), st));
   }
   S.m_cut[0] = S.mods.nm;
   S.m_cut[1] = S.sh;
@@ -1041,7 +1057,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   CrtState& S = *ctx.crt;
   cudaStream_t st = stream();
   const SpinSpace &SA = ctx.sp[0], &SB = ctx.sp[1];
-  const int NA = SA.count, NB = SB.count, n = ctx.n;
+  const int NA = alpha_strings(ctx), NB = beta_strings(ctx), n = ctx.n;
   // scale: 1.25 times the bound of today's string matrices, so that a small per-step one-body term keeps it
   {
     double rm = 0.0, mmax = 0.0;
@@ -1084,7 +1100,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   F.nm = nm;
   F.na = ctx.na;
   F.nb = ctx.nb;
-  F.na_strings = NA;
+  F.na_strings = SA.count;
   F.decA = SA.dec.as<int>();
   F.decB = SB.dec.as<int>();
   F.kmax = ctx.kmax;
