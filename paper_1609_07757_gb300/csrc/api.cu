@@ -583,14 +583,15 @@ iscsi_status iscsi_stats(char* json, int len) {
       out += v;
     }
     // the residue products of the last FP64 sigma step (zeros: none): bf16 MMA flops issued, work
-    // items, CTAs, moduli
+    // items, CTAs, moduli; whether slices of the string matrices are held
     {
       double flops = 0.0;
       int items = 0, grid = 0, moduli = 0;
       crt_stats(*ctx, flops, items, grid, moduli);
       std::snprintf(v, sizeof(v),
-                    ", \"residues\": {\"bf16_flops\": %.17g, \"items\": %d, \"grid\": %d, \"moduli\": %d}", flops, items,
-                    grid, moduli);
+                    ", \"residues\": {\"bf16_flops\": %.17g, \"items\": %d, \"grid\": %d, \"moduli\": %d}, "
+                    "\"samespin_slices\": %d",
+                    flops, items, grid, moduli, ctx->oz_m_ready ? 1 : 0);
       out += v;
     }
     // GAS restriction: subspaces (0: none) and kept determinants

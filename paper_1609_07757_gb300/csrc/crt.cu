@@ -917,6 +917,13 @@ static int beta_strings(const Context& ctx) {
   return (int)most;
 }
 
+void crt_strings(const Context& ctx, int& sa, int& sb) {
+  sa = alpha_strings(ctx);
+  sb = beta_strings(ctx);
+}
+
+bool crt_full(Context& ctx) { return crt_state(ctx).flat; }
+
 // the same-spin products, all levels at once, when the strings fill a tile or so
 bool crt_ss_active(Context& ctx, int nvec) {
   CrtState& S = crt_state(ctx);

@@ -383,6 +383,7 @@ int tc_err_buf(Context& ctx);  // the context's error word (allocated and cleare
 int tc_wait_selftest(Context& ctx, long long polls);
 int tc_wait_status(int* err, const char* what);
 int samespin_matrices_changed(Context& ctx);  // re-cut the same-spin operand slices in place
+void samespin_drop_slices(Context& ctx);       // frees the FP64 slices of the same-spin products (built anew when needed)
 // M <- M_base + f M_v (cpl: the context of v); f = 0 restores (sigma.cu)
 int onebody_shift(Context& ctx, const Context& cpl, double f);
 // jobs assembled elsewhere: append a segment (K from column 0 of both arrays),
@@ -396,6 +397,8 @@ int oz_job_launch(Context& ctx, const OzJob& job, cudaStream_t st);
 // spin, 2 same spin (all levels); crt_parts: what the current routing sends there
 bool crt_ab_active(Context& ctx, int nvec);
 bool crt_ss_active(Context& ctx, int nvec);
+bool crt_full(Context& ctx);                              // one class that reaches every row (full CI)
+void crt_strings(const Context& ctx, int& sa, int& sb);  // strings that determinants of the space have
 int crt_parts(Context& ctx, int nvec);
 int crt_operands(Context& ctx, const double* c, int nvec, int parts);
 int crt_gemm(Context& ctx);

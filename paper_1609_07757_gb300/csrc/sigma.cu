@@ -905,19 +905,41 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
 // 0.78 16.3 / 8.2, 0.55 50.7 / 38.7; the square of a one-body operator (full CI, 60 orbitals, 0.004)
 // 1.02 / 1.26.  The line through these meets 1 between 0.3 and 0.45.
 constexpr double kCrtMinKept = 0.45;
-constexpr int kCrtSsAlone = 2048;
+// Where the residues win over the slices otherwise, from 950 spaces and block sizes of 1 to 12 vectors (1 + 1 to 7 + 1
+// electrons, every truncation).  One sigma in ms: residues in both parts, in the same-spin part alone, slices.
+//  * Opposite spin.  The fold adds na nb residues per modulus and determinant where k_fold adds na nb doubles, and in a
+//    truncated space its blocks are short: 4 + 4 in 15 orbitals, quadruples 0.78, 0.54, 0.61; 5 + 5 in 12 1.07, 0.51, 0.58;
+//    3 + 3 in 22, doubles, 12 vectors 0.56, 0.42, 0.86; 3 + 2 in 24, quadruples 0.20, 0.22, 0.29.  Full spaces (long rows,
+//    one run of columns) win up to na nb = 16: 4 + 4 in 14 0.89, 0.98, 1.19; 5 + 4 in 11 0.36, 0.29, 0.44.  One or two
+//    alpha electrons have few holes: 1 + 4 in 18, triples 0.10, 0.15, 0.17.  A few thousand elements are bound by launches: 5 + 2
+//    in 14, doubles 0.068, 0.090, 0.136.
+//  * Same spin.  All blocks in one launch, and a launch or two per vector and block less: 3 + 3 in 9, quintuples, 12
+//    vectors 0.18, 0.15, 1.02.  But the whole string matrices are read, 26 bytes an element, where the slices read 14
+//    of the blocks that are there, which counts in sparse truncations of many strings (doubles: 2 + 2 in 70, 2415
+//    strings, this part alone 0.312, slices 0.302, in 100 0.726, 0.665; 3 + 3 in 36, triples, 7140 strings 1.20, 1.11) and
+//    with many strings of one spin beside few of the other (6 + 1 in 18, 18564 and 18: 1.44, 1.45, 1.01).
+constexpr int kCrtFoldFull = 16, kCrtFoldSmall = 12;
+constexpr long long kCrtSmall = 8000;
+constexpr int kCrtStrings = 2048, kCrtThinStrings = 64, kCrtThinOther = 6000;
+constexpr double kCrtDense = 0.02;
 
 int crt_parts(Context& ctx, int nvec) {
   if (ctx.units_opposite_total > 0 && (double)ctx.units_opposite < kCrtMinKept * (double)ctx.units_opposite_total) return 0;
-  int parts = 0;
-  if (ctx.have_ab && ab_on_tc(ctx, 64) && crt_ab_active(ctx, nvec)) parts |= 1;
-  // the same-spin part follows the opposite-spin part; alone (a thin column class keeps that one on the
-  // slices) it pays while the string matrices are small: CISD, slices / residues, 50 orbitals (1225 strings)
-  // 0.219 / 0.189 ms, 70 (2415) 0.307 / 0.308, 100 (4950) 0.66 / 0.69, 150 2.02 / 2.35
-  if (ctx.route[0].ss_min <= kThinN && samespin_tc_active(ctx) && crt_ss_active(ctx, nvec) &&
-      ((parts & 1) || !ctx.have_ab || std::max(ctx.sp[0].count, ctx.sp[1].count) <= kCrtSsAlone))
-    parts |= 2;
-  return parts;
+  bool ab = ctx.have_ab && ab_on_tc(ctx, 64) && crt_ab_active(ctx, nvec);
+  if (ab) {
+    const int na = ctx.na, nb = ctx.nb, c = na * nb;
+    ab = crt_full(ctx) ? c <= kCrtFoldFull
+                       : nb <= 4 && (na <= 2 || (na == 3 && nb <= 2) ||
+                                     (c <= kCrtFoldSmall && ctx.ndet * nvec <= kCrtSmall));
+  }
+  // the string matrices elsewhere by an option or the autotuner, or too few strings for a tile: opposite spin alone
+  if (ctx.route[0].ss_min > kThinN || !samespin_tc_active(ctx) || !crt_ss_active(ctx, nvec)) return ab ? 1 : 0;
+  int sa = 0, sb = 0;
+  crt_strings(ctx, sa, sb);
+  const int more = std::max(sa, sb), less = std::min(sa, sb);
+  const bool ss = !ctx.have_ab || (!(less <= kCrtThinStrings && more > kCrtThinOther) &&
+                                   (more <= kCrtStrings || (double)ctx.ndet >= kCrtDense * sa * sb));
+  return ss ? (ab ? 3 : 2) : 0;
 }
 
 static int sigma_steps(Context& ctx, const double* c, double* sigma, int nvec, int precision, int phases) {
@@ -965,7 +987,8 @@ int sigma_run(Context& ctx, const double* c, double* sigma, int nvec, int precis
 // A model from the flop counts and the kernels' measured rates (tensor-core
 // FP64-accurate contraction ~1.1 PFLOP/s of bf16 products, FP32 form ~0.6,
 // FP64 FMA ~1.1 TFLOP/s, FP32 FMA ~24 TFLOP/s) keeps the candidates within 3x
-// of the best prediction; each of those is timed on the caller's vector (one
+// of the best prediction (thresholds that put the same blocks on the tensor cores are one candidate, the
+// lowest, which is the one that the residues may take); each of those is timed on the caller's vector (one
 // untimed sigma to build its lists, then the best of three timed with CUDA
 // events, since close candidates differ by a few percent) and the fastest is
 // kept.  Runs once per context, precision and vector count, before
@@ -1029,8 +1052,6 @@ int sigma_autotune(Context& ctx, const double* c, double* sigma, int nvec, int p
           double rows = block_rows(ctx, a), nba = (double)ctx.nb_allowed_lvl[a];
           same = (rows > q.ss && nba > q.ss) == (rows > ss && nba > ss);
         }
-        // the lowest threshold is the residue products (all blocks at once), the others slices
-        if (prec == 64 && crt_ss_active(ctx, nvec) && (q.ss == kThinN) != (ss == kThinN)) same = false;
         if (same) dup = true;
       }
       if (!dup) cands.push_back({ab, ss, route_model_ms(ctx, prec, ab, ss, nvec), -1.0});
@@ -1069,6 +1090,11 @@ int sigma_autotune(Context& ctx, const double* c, double* sigma, int nvec, int p
     if ((q.ms >= 0 ? q.ms : q.pred) < (best->ms >= 0 ? best->ms : best->pred)) best = &q;
   R.ab_tc = best->ab;
   R.ss_min = best->ss;
+  if (prec == 64 && keep.size() > 1) {  // what only the other candidates used
+    const int parts = crt_parts(ctx, nvec);
+    if (parts & 2) samespin_drop_slices(ctx);
+    if (parts == 0) crt_release(ctx);
+  }
   for (const Cand& q : cands) {
     R.trials.push_back(q.ab);
     R.trials.push_back(q.ss >= (1 << 30) ? -1 : q.ss);

@@ -1111,6 +1111,18 @@ int launch_tc_problems(const OzProblem* probs, int nprobs, const OzSeg* segs, co
   return launch_t3(tiles, bn, probs, nprobs, segs, maps, nullptr, reinterpret_cast<float* const*>(tbases), err, st);
 }
 
+void samespin_drop_slices(Context& ctx) {
+  if (!ctx.oz_m_ready) return;
+  for (DevBuf* b : {&ctx.oz_mas, &ctx.oz_maexp, &ctx.oz_malive, &ctx.oz_mbs, &ctx.oz_mbexp, &ctx.oz_mblive, &ctx.oz_macol,
+                    &ctx.oz_marow, &ctx.oz_cs, &ctx.oz_csexp})
+    b->release();
+  ctx.oz_malive_h.clear();
+  ctx.oz_mblive_h.clear();
+  ctx.oz_cs_elems = 0;
+  ctx.oz_m_ready = false;
+  ctx.oz_ss.nvec = -1;
+}
+
 // the same-spin string matrices changed in place: cut the slices prepared so far again
 int samespin_matrices_changed(Context& ctx) {
   if (ctx.oz_m_ready) ISCSI_TRY(tc_prepare_m(ctx, true));

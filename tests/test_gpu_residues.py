@@ -309,3 +309,37 @@ def test_density_nonfinite(n, na, nb, kmax):
             i = np.arange(n)
             reached[i, :, i, :] = reached[:, i, :, i] = False
         assert np.isnan(a[reached]).all() and np.array_equal(a[~reached], b[~reached])
+
+
+# spaces on either side of each line of the routing: the same sigma whichever part takes the residues (3 both, 2 same
+# spin, 1 opposite spin, 0 neither)
+@pytest.mark.parametrize("n,na,nb,kmax,nvec", [(11, 3, 3, 4, 1), (11, 3, 3, 4, 12), (13, 4, 4, 4, 1), (10, 5, 4, 9, 1),
+                                               (9, 4, 4, 8, 1), (12, 1, 4, 3, 4), (10, 5, 5, 3, 1), (14, 6, 1, 6, 2),
+                                               (9, 1, 1, 2, 1), (18, 5, 1, 4, 1), (30, 3, 1, 2, 1)])
+def test_residues_routing(n, na, nb, kmax, nvec):
+    h1, eri = make_integrals(n, 7700 + n, ell=3.0, nchol=12)
+    L.iscsi_init(n, na, nb, kmax, h1, eri, 1e-14)
+    C = np.stack([unit_vector(L.iscsi_ndet(), 30 + v) for v in range(nvec)])
+    s = sigma(C, nvec)
+    assert np.array_equal(s, sigma(C, nvec))
+    L.iscsi_set_option("fp64_tc", 0)
+    ref = sigma(C, nvec)
+    for v in range(nvec):
+        check(s[v], ref[v])
+
+
+def test_autotune_leaves_no_slices_beside_residues():
+    """The autotuner's other candidates cut the string matrices into slices; where the residues win, their memory is
+    given back, a field step cuts nothing but residues, and the slices come back when they are asked for."""
+    n = 40
+    h1, eri = make_integrals(n, 7800, ell=4.0, nchol=12)
+    L.iscsi_init(n, 2, 2, 4, h1, eri, 1e-14)
+    c = unit_vector(L.iscsi_ndet(), 6)[None]
+    L.iscsi_set_option("autotune", 1)
+    s = sigma(c, 1)
+    st = L.iscsi_stats()
+    L.iscsi_set_option("autotune", 0)
+    assert sum(t[3] >= 0 for t in st["route_fp64"]["trials"]) >= 2 and st["residues"]["items"] > 0
+    assert st["samespin_slices"] == 0
+    L.iscsi_set_option("fp64_tc", 0)
+    check(s, sigma(c, 1))
