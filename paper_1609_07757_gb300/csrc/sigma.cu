@@ -270,8 +270,8 @@ __global__ void __launch_bounds__(256)
 }
 
 // sigma's elements from the chunks' partial sums, in chunk order; a thread per column and row (grid.y).
-// Bound by the latency of the chunks' loads: eight in flight, rows side by side (a thread per column for all rows:
-// FP32 sigma of 4 + 3 electrons in 10 orbitals, 5 chunks, 139 us; now 121).
+// Bound by the latency of the chunks' loads: sixteen in flight (155 chunks, CISD in 100 orbitals: eight 32 us), rows side
+// by side (a thread per column for all rows: FP32 sigma of 4 + 3 electrons in 10 orbitals, 5 chunks, 139 us; now 121).
 template <typename T>
 __global__ void k_mthin_reduce(const Problem<T>* __restrict__ probs, int nprobs, const long long* __restrict__ part_off,
                                T* sbase, const T* __restrict__ cbase, int total_cols, int nchunks,
@@ -292,8 +292,16 @@ __global__ void k_mthin_reduce(const Problem<T>* __restrict__ probs, int nprobs,
            n + (long long)m * P.ldc;
   T acc = T(0);
   const T* src = part + part_off[lo] + (long long)m * P.N + n;
-#pragma unroll 8
-  for (int c = 0; c < nchunks; ++c) acc += src[c * part_stride];
+  int c = 0;
+  for (; c + 16 <= nchunks; c += 16, src += 16 * part_stride) {
+    T x[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) x[j] = __ldg(src + j * part_stride);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) acc += x[j];
+  }
+#pragma unroll 4
+  for (; c < nchunks; ++c, src += part_stride) acc += __ldg(src);
   *dst = P.accumulate ? *dst + acc : acc;
 }
 
