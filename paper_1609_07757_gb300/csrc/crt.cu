@@ -755,9 +755,12 @@ struct CrtFoldLaunch {
   int rows = 0, threads = 0, blocks = 0, smem = 0;
 };
 
+constexpr int kCrtMaxVecs = 65535;  // vectors are a grid dimension of k_crt_cmax and k_crt_fold
+
 struct CrtState {
-  bool off = false;  // its buffers did not fit (or its units are not finite): the context stays on the slices
-  size_t held = 0;   // bytes of residue buffers (crt_alloc)
+  bool off = false;  // its units are not finite: the context stays on the slices
+  int max_vecs = kCrtMaxVecs;  // larger blocks did not fit: they take the slices
+  CrtHeld held;      // residue buffers (crt_alloc)
   bool flat = false;  // every class reaches every row: no levels in the orders
   std::vector<CrtGroup> groups;
   std::vector<int> ystart;
@@ -886,12 +889,11 @@ static FoldShape fold_shape(const Context& ctx, const CrtState& S, int lev) {
 // to fit k_crt_fold's shared memory.
 constexpr int kCrtMinCols = 64;
 constexpr int kCrtMinRows = 16;
-constexpr int kCrtMaxVecs = 65535;  // vectors are a grid dimension of k_crt_cmax and k_crt_fold
 
 bool crt_ab_active(Context& ctx, int nvec) {
-  if (!ctx.have_ab || nvec > kCrtMaxVecs) return false;
+  if (!ctx.have_ab) return false;
   CrtState& S = crt_state(ctx);
-  if (S.off || S.groups.empty() || fold_shape(ctx, S, 0).ni == 0) return false;
+  if (S.off || nvec > S.max_vecs || S.groups.empty() || fold_shape(ctx, S, 0).ni == 0) return false;
   double heavy = 0.0, good = 0.0;
   for (const CrtGroup& g : S.groups) {
     const double w = (double)g.rows * g.rows;
@@ -927,7 +929,7 @@ bool crt_full(Context& ctx) { return crt_state(ctx).flat; }
 // the same-spin products, all levels at once, when the strings fill a tile or so
 bool crt_ss_active(Context& ctx, int nvec) {
   CrtState& S = crt_state(ctx);
-  return !S.off && nvec <= kCrtMaxVecs && alpha_strings(ctx) >= kCrtMinRows && beta_strings(ctx) >= kCrtMinRows;
+  return !S.off && nvec <= S.max_vecs && alpha_strings(ctx) >= kCrtMinRows && beta_strings(ctx) >= kCrtMinRows;
 }
 
 int crt_encode(CrtProblem& P, const void* a, const void* b, int nm) {
@@ -1387,23 +1389,38 @@ static int crt_build(Context& ctx, int nvec, int parts) {
   return kOk;
 }
 
-int crt_alloc(DevBuf& d, size_t bytes, size_t& held) {
-  held -= std::min(held, d.bytes);
+static size_t g_crt_held = 0;
+
+void CrtHeld::add(size_t n) {
+  bytes += n;
+  g_crt_held += n;
+}
+
+int crt_alloc(DevBuf& d, size_t bytes, CrtHeld& held) {
+  held.add(0 - std::min(held.bytes, d.bytes));
   d.release();
   size_t free_b = 0, total = 0;
   ISCSI_CUDA(cudaMemGetInfo(&free_b, &total));
-  if (held + bytes > (free_b + held) / 2) {
+  if (g_crt_held + bytes > (free_b + g_crt_held) / 2) {
     set_error("residues: less than half of the free memory would be left");
     return kErrNoMem;
   }
   ISCSI_TRY(d.alloc(bytes));
-  held += bytes;
+  held.add(bytes);
   return kOk;
 }
 
+bool crt_drop(Context& ctx) {
+  if (!ctx.crt || ctx.crt->held.bytes == 0) return false;
+  const int most = ctx.crt->max_vecs;
+  crt_release(ctx);
+  crt_state(ctx).max_vecs = most;
+  return true;
+}
+
 // Operands of this call's vectors (building buffers and work list when they
-// changed).  parts: 1 opposite spin, 2 same spin.  kErrNoMem leaves the
-// context without residues (the caller takes the slices instead).
+// changed).  parts: 1 opposite spin, 2 same spin.  kErrNoMem leaves blocks of this
+// many vectors and more without residues (the caller takes the slices instead).
 int crt_operands(Context& ctx, const double* c, int nvec, int parts) {
   CrtState& S = crt_state(ctx);
   cudaStream_t st = stream();
@@ -1415,9 +1432,12 @@ int crt_operands(Context& ctx, const double* c, int nvec, int parts) {
     S.nvec = -1;
     const int rc = crt_build(ctx, nvec, parts);
     if (rc == kErrNoMem) {
+      // blocks of fewer vectors may still fit
+      const bool off = S.off;
       cudaStreamSynchronize(st);
       crt_release(ctx);
-      crt_state(ctx).off = true;
+      crt_state(ctx).off = off;
+      crt_state(ctx).max_vecs = nvec - 1;
       cudaGetLastError();
     }
     ISCSI_TRY(rc);

@@ -35,10 +35,19 @@ struct CrtJob {
 CrtMods crt_make_mods(int nm);
 CrtWeights crt_make_weights(int nm, int terms, int terms_next = 0, int passes_next = 0);
 double crt_log2_product(int nm);
+// Bytes of residue buffers of one user, counted for the process as well.
+struct CrtHeld {
+  size_t bytes = 0;
+  CrtHeld() = default;
+  CrtHeld(const CrtHeld&) = delete;
+  CrtHeld& operator=(const CrtHeld&) = delete;
+  ~CrtHeld() { add(0 - bytes); }
+  void add(size_t n);  // (modulo 2^64: also takes back)
+};
 // A residue buffer: the residues take a few times the memory of the slices, and are taken only while
-// all of one user's (`held` bytes, kept here) stay below half of what the device has free, so that a
-// program's own vectors find the room they found with the slices.  kErrNoMem otherwise.
-int crt_alloc(DevBuf& d, size_t bytes, size_t& held);
+// all of the process's stay below half of what the device would have free without them, so that a
+// program's own vectors and other contexts find the room they found with the slices.  kErrNoMem otherwise.
+int crt_alloc(DevBuf& d, size_t bytes, CrtHeld& held);
 // tensor maps of a product's operands
 int crt_encode(CrtProblem& P, const void* a, const void* b, int nm);
 

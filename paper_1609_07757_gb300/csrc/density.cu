@@ -85,9 +85,10 @@ constexpr int kDmNotFinite = -(1 << 20);  // scale of a row with an infinity or 
 
 struct DensityPlan {
   bool built = false;
-  // residues (res_fail: thin blocks, or they do not fit): operands of bra and ket, output residues, scales
-  bool res_fail = false;
-  size_t res_held = 0;
+  // residues (not for thin blocks, nor where they do not fit: ket = bra / general): operands of bra and
+  // ket, output residues, scales
+  bool thin = false, no_room[2] = {false, false};
+  CrtHeld res_held;
   DevBuf res_bra, res_ket, res_out, scale;  // scale: per row of bra, of ket, then partial maxima
   int nmods = kDmMods, res_rows = 0;        // moduli; rows of all blocks
   CrtJob res_job[2];             // ket = bra / general
@@ -117,6 +118,15 @@ struct DensityPlan {
 void density_release(Context& ctx) {
   delete ctx.dm;
   ctx.dm = nullptr;
+}
+
+bool density_drop(Context& ctx) {
+  if (!ctx.dm || ctx.dm->res_held.bytes == 0) return false;
+  DensityPlan& P = *ctx.dm;
+  for (DevBuf* d : {&P.res_bra, &P.res_ket, &P.res_out}) d->release();
+  P.res_held.add(0 - P.res_held.bytes);
+  P.res_ready[0] = P.res_ready[1] = false;
+  return true;
 }
 
 static inline int rup(int x, int m) { return (x + m - 1) / m * m; }
@@ -325,7 +335,7 @@ static int plan_build(Context& ctx) {
     most_cols = std::max(most_cols, cols);
     most_rows = std::max(most_rows, B.R);
   }
-  P.res_fail = most_cols <= kDmThinCols && most_rows > kDmThinRows;
+  P.thin = most_cols <= kDmThinCols && most_rows > kDmThinRows;
   for (cudaEvent_t& e : P.ev) ISCSI_CUDA(cudaEventCreate(&e));
   P.sl_elems = sl;
   P.q_elems = q;
@@ -1076,17 +1086,19 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
     ISCSI_TRY(plan_build(ctx));
     Pp = ctx.dm;
     DensityPlan& P = *Pp;
-    if (!P.res_fail) {
+    bool res = !P.thin && !P.no_room[sym ? 0 : 1];
+    if (res) {
       const int rc = residues_build(ctx, sym);
       if (rc == kErrNoMem) {
-        P.res_fail = true;
-        for (DevBuf* d : {&P.res_bra, &P.res_ket, &P.res_out}) d->release();
         cudaGetLastError();
+        density_drop(ctx);
+        P.no_room[1] = true;  // a ket of its own takes more
+        P.no_room[0] = P.no_room[0] || sym;
+        res = false;
       } else {
         ISCSI_TRY(rc);
       }
     }
-    const bool res = !P.res_fail;
     const bool ev = !ctx.capturing;
     if (res) {
       ISCSI_TRY(residues_cut(ctx, bra, sym ? nullptr : ket, st));

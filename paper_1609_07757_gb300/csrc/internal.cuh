@@ -406,6 +406,7 @@ int crt_fold(Context& ctx, double* sigma);  // sigma (overwritten): the parts th
 int crt_matrices_changed(Context& ctx);
 void crt_invalidate(Context& ctx);  // a call ended early: build (and clear the exponents) anew at the next one
 void crt_release(Context& ctx);
+bool crt_drop(Context& ctx);  // frees the residues' memory (built anew when it fits again); false: none held
 // bf16 MMA flops, work items and CTAs of the last built launch (0 without one)
 void crt_stats(const Context& ctx, double& flops, int& items, int& grid, int& moduli);
 int crt_batch_launch(CrtBatch*& b, const std::vector<Context*>& ctxs, int* err, cudaStream_t st);
@@ -414,6 +415,7 @@ void crt_batch_release(CrtBatch*& b);
 // density.cu: one- and two-body density matrices (Eqs. d1, d2)
 int density_run(Context& ctx, const double* bra, const double* ket, double* d1, double* d2);
 void density_release(Context& ctx);
+bool density_drop(Context& ctx);  // frees the residues' memory; false: none held
 // flops of one launch of the density contraction (sym: ket = bra); which 0:
 // bf16 MMA flops, 1: 2 M N K of the computed regions; 0 before the first call
 double density_flops(const Context& ctx, int sym, int which);

@@ -343,3 +343,42 @@ def test_autotune_leaves_no_slices_beside_residues():
     assert st["samespin_slices"] == 0
     L.iscsi_set_option("fp64_tc", 0)
     check(s, sigma(c, 1))
+
+
+def leave_free(nbytes):
+    """Holds all of the device's memory but nbytes."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.empty(torch.cuda.mem_get_info()[0] - nbytes, dtype=torch.uint8, device="cuda")
+
+
+def test_residues_refused_for_a_large_block_only():
+    """A block whose residues do not fit (40 vectors: 5 GB of 3.4 free) takes the slices; smaller ones take residues,
+    before and after."""
+    n, nvec = 40, 40
+    h1, eri = make_integrals(n, 7950, ell=4.0, nchol=12)
+    L.iscsi_init(n, 2, 2, 4, h1, eri, 1e-14)
+    nd = L.iscsi_ndet()
+    C = np.stack([unit_vector(nd, 50 + v) for v in range(nvec)])
+    L.iscsi_set_option("fp64_tc", 0)
+    ref = sigma(C, nvec)
+    L.iscsi_finalize()
+    L.iscsi_set_option("fp64_tc", 1)
+    L.iscsi_init(n, 2, 2, 4, h1, eri, 1e-14)
+    dev = torch.as_tensor(C, device="cuda")
+    out = torch.empty_like(dev)
+    hog = leave_free(5 << 30)
+    try:
+        items = []
+        for k in (1, nvec, 1, nvec):
+            out.fill_(float("nan"))
+            L.iscsi_sigma(dev[:k], out[:k], k)
+            items.append(L.iscsi_stats()["residues"]["items"])
+            s = out.cpu().numpy()
+            for v in range(k):
+                check(s[v], ref[v])
+    finally:
+        hog = None
+        torch.cuda.empty_cache()
+    # (a block on the slices leaves the smaller one's residues where they are)
+    assert items[0] > 0 and items[1] == 0 and items[2] == items[0]
