@@ -31,6 +31,20 @@ static Context* current() {
   return it == g_ctx.end() ? nullptr : it->second.get();
 }
 
+// A call that ran out of device memory: the residues of every context give theirs back (they are a few times the
+// slices' memory), and it runs once more.  f: the call from its start, nothing of it in progress.
+template <typename F>
+static int with_room(F f) {
+  const int s = f();
+  if (s != kErrNoMem) return s;
+  bool freed = false;
+  for (auto& c : g_ctx) {
+    if (crt_drop(*c.second)) freed = true;
+    if (density_drop(*c.second)) freed = true;
+  }
+  return freed ? f() : s;
+}
+
 }  // namespace iscsi
 
 using namespace iscsi;
@@ -68,8 +82,11 @@ static iscsi_status init_context(int norb, int nalpha, int nbeta, int max_excita
     set_error("iscsi_init: string space too large for the dense same-spin string Hamiltonian");
     return ISCSI_E_ARG;
   }
-  auto ctx = std::make_unique<Context>();
-  int s = context_build(*ctx, norb, nalpha, nbeta, max_excitation, h1, eri, tau, ninner);
+  std::unique_ptr<Context> ctx;
+  int s = with_room([&] {
+    ctx = std::make_unique<Context>();
+    return context_build(*ctx, norb, nalpha, nbeta, max_excitation, h1, eri, tau, ninner);
+  });
   if (s == kOk && gas) {
     s = gas_set(*ctx, gas->nspace, gas->sizes, gas->cmin, gas->cmax);
     // the level truncation alone gives the GAS space: no projection needed
@@ -147,13 +164,15 @@ iscsi_status iscsi_sigma(const void* c, void* sigma, int nvec) {
     set_error("iscsi_sigma: NULL pointer or nvec < 1");
     return ISCSI_E_ARG;
   }
-  const double* cin = static_cast<const double*>(c);
-  if (ctx->gas_nspace) {  // sigma = P H P c: the projected input in a context buffer
-    ISCSI_TRY(ctx->gas_in.grow(sizeof(double) * (size_t)ctx->ndet * nvec));
-    ISCSI_TRY(gas_project(*ctx, cin, ctx->gas_in.as<double>(), nvec, stream()));
-    cin = ctx->gas_in.as<double>();
-  }
-  return sigma_run(*ctx, cin, static_cast<double*>(sigma), nvec, options().precision);
+  return with_room([&]() -> int {
+    const double* cin = static_cast<const double*>(c);
+    if (ctx->gas_nspace) {  // sigma = P H P c: the projected input in a context buffer
+      ISCSI_TRY(ctx->gas_in.grow(sizeof(double) * (size_t)ctx->ndet * nvec));
+      ISCSI_TRY(gas_project(*ctx, cin, ctx->gas_in.as<double>(), nvec, stream()));
+      cin = ctx->gas_in.as<double>();
+    }
+    return sigma_run(*ctx, cin, static_cast<double*>(sigma), nvec, options().precision);
+  });
 }
 
 iscsi_status iscsi_sigma_noalloc(const void* c, void* sigma) {
@@ -180,11 +199,13 @@ iscsi_status iscsi_sigma_host(const double* c, double* sigma, int nvec) {
   // staging buffers kept by the context (no allocation on repeated calls)
   DevBuf& dc = ctx->host_io[0];
   DevBuf& ds = ctx->host_io[1];
-  ISCSI_TRY(dc.grow(bytes));
-  ISCSI_TRY(ds.grow(bytes));
-  ISCSI_CUDA(cudaMemcpyAsync(dc.p, c, bytes, cudaMemcpyHostToDevice, st));
-  if (ctx->gas_nspace) ISCSI_TRY(gas_project(*ctx, dc.as<double>(), dc.as<double>(), nvec, st));
-  ISCSI_TRY(sigma_run(*ctx, dc.as<double>(), ds.as<double>(), nvec, options().precision));
+  ISCSI_TRY(with_room([&]() -> int {
+    ISCSI_TRY(dc.grow(bytes));
+    ISCSI_TRY(ds.grow(bytes));
+    ISCSI_CUDA(cudaMemcpyAsync(dc.p, c, bytes, cudaMemcpyHostToDevice, st));
+    if (ctx->gas_nspace) ISCSI_TRY(gas_project(*ctx, dc.as<double>(), dc.as<double>(), nvec, st));
+    return sigma_run(*ctx, dc.as<double>(), ds.as<double>(), nvec, options().precision);
+  }));
   ISCSI_CUDA(cudaMemcpyAsync(sigma, ds.p, bytes, cudaMemcpyDeviceToHost, st));
   ISCSI_CUDA(cudaStreamSynchronize(st));
   return tc_check(*ctx);
@@ -196,8 +217,10 @@ iscsi_status iscsi_density(const void* bra, const void* ket, void* d1, void* d2)
     set_error("iscsi_density: bra is NULL or both outputs are NULL");
     return ISCSI_E_ARG;
   }
-  return density_run(*ctx, static_cast<const double*>(bra), static_cast<const double*>(ket),
-                     static_cast<double*>(d1), static_cast<double*>(d2));
+  return with_room([&] {
+    return density_run(*ctx, static_cast<const double*>(bra), static_cast<const double*>(ket),
+                       static_cast<double*>(d1), static_cast<double*>(d2));
+  });
 }
 
 iscsi_status iscsi_density_host(const double* bra, const double* ket, double* d1, double* d2) {
@@ -215,16 +238,18 @@ iscsi_status iscsi_density_host(const double* bra, const double* ket, double* d1
   DevBuf& o1 = ctx->host_io[2];
   DevBuf& o2 = ctx->host_io[3];
   const bool has_ket = ket && ket != bra;
-  ISCSI_TRY(db.grow(vb));
-  ISCSI_CUDA(cudaMemcpyAsync(db.p, bra, vb, cudaMemcpyHostToDevice, st));
-  if (has_ket) {
-    ISCSI_TRY(dk.grow(vb));
-    ISCSI_CUDA(cudaMemcpyAsync(dk.p, ket, vb, cudaMemcpyHostToDevice, st));
-  }
-  if (d1) ISCSI_TRY(o1.grow(b1));
-  if (d2) ISCSI_TRY(o2.grow(b2));
-  ISCSI_TRY(density_run(*ctx, db.as<double>(), has_ket ? dk.as<double>() : nullptr, d1 ? o1.as<double>() : nullptr,
-                        d2 ? o2.as<double>() : nullptr));
+  ISCSI_TRY(with_room([&]() -> int {
+    ISCSI_TRY(db.grow(vb));
+    ISCSI_CUDA(cudaMemcpyAsync(db.p, bra, vb, cudaMemcpyHostToDevice, st));
+    if (has_ket) {
+      ISCSI_TRY(dk.grow(vb));
+      ISCSI_CUDA(cudaMemcpyAsync(dk.p, ket, vb, cudaMemcpyHostToDevice, st));
+    }
+    if (d1) ISCSI_TRY(o1.grow(b1));
+    if (d2) ISCSI_TRY(o2.grow(b2));
+    return density_run(*ctx, db.as<double>(), has_ket ? dk.as<double>() : nullptr, d1 ? o1.as<double>() : nullptr,
+                       d2 ? o2.as<double>() : nullptr);
+  }));
   if (d1) ISCSI_CUDA(cudaMemcpyAsync(d1, o1.p, b1, cudaMemcpyDeviceToHost, st));
   if (d2) ISCSI_CUDA(cudaMemcpyAsync(d2, o2.p, b2, cudaMemcpyDeviceToHost, st));
   ISCSI_CUDA(cudaStreamSynchronize(st));
@@ -271,7 +296,11 @@ iscsi_status iscsi_propagate(void* c, int nsteps, double dt, const double* field
   // a GAS restriction: the start vector is projected onto the kept determinants
   if (ctx->gas_nspace)
     ISCSI_TRY(gas_project(*ctx, static_cast<double*>(c), static_cast<double*>(c), imaginary ? 1 : 2, stream()));
-  return propagate_run(*ctx, cpl, static_cast<double*>(c), nsteps, dt, field, krylov, imaginary, diag);
+  int done = 0;  // (a vector that has moved is not propagated again)
+  return with_room([&]() -> int {
+    return done > 0 ? kErrNoMem
+                    : propagate_run(*ctx, cpl, static_cast<double*>(c), nsteps, dt, field, krylov, imaginary, diag, &done);
+  });
 }
 
 iscsi_status iscsi_set_gas(int nspace, const int* sizes, const int* cmin, const int* cmax, long long* ndet_gas) {
@@ -372,7 +401,7 @@ iscsi_status iscsi_davidson(int nroots, double tol, double* energies, void* vecs
     set_error("iscsi_davidson: the context's one-body part is not symmetric (not a Hamiltonian)");
     return ISCSI_E_ARG;
   }
-  int s = davidson_run(*ctx, nroots, tol, energies, static_cast<double*>(vecs));
+  int s = with_room([&] { return davidson_run(*ctx, nroots, tol, energies, static_cast<double*>(vecs)); });
   int w = tc_check(*ctx);
   return s != ISCSI_OK ? s : w;
 }
@@ -675,7 +704,7 @@ iscsi_status iscsi_batch_sigma(const int* handles, const void* const* cs, void* 
     c[i] = static_cast<const double*>(cs[i]);
     s[i] = static_cast<double*>(sigmas[i]);
   }
-  return batch_sigma(ctxs, c, s, nvec, options().precision == 32 ? 32 : 64);
+  return with_room([&] { return batch_sigma(ctxs, c, s, nvec, options().precision == 32 ? 32 : 64); });
 }
 
 iscsi_status iscsi_batch_check(void) { return batch_check(); }
@@ -706,7 +735,9 @@ iscsi_status iscsi_batch_davidson(const int* handles, int count, int nroots, dou
     }
     ctxs[i] = it->second.get();
   }
-  int s = davidson_batch_run(ctxs, nroots, tol, energies, reinterpret_cast<double* const*>(vecs), statuses);
+  int s = with_room([&] {
+    return davidson_batch_run(ctxs, nroots, tol, energies, reinterpret_cast<double* const*>(vecs), statuses);
+  });
   for (Context* c : ctxs) {
     int w = tc_check(*c);
     if (w != ISCSI_OK && s == ISCSI_OK) s = w;

@@ -431,7 +431,7 @@ size_t noalloc_scratch_bytes();
 // [ndet] (imaginary time); diag: host [2 * nsteps] or nullptr
 constexpr int kPrMaxKrylov = 64;
 int propagate_run(Context& ctx, Context* cpl, double* c, int nsteps, double dt, const double* field, int m,
-                  int imaginary, double* diag);
+                  int imaginary, double* diag, int* steps_done);
 
 // davidson.cu
 int davidson_run(Context& ctx, int nroots, double tol, double* energies, double* vecs);

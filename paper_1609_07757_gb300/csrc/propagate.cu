@@ -229,7 +229,7 @@ static void jacobi_eigh(std::vector<double>& A, int m, std::vector<double>& w, s
 static int pr_blocks(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 152 * 8)); }
 
 static int propagate_steps(Context& ctx, Context* cpl, double* c, int nsteps, double dt, const double* field, int m,
-                           int imaginary, double* diag) {
+                           int imaginary, double* diag, int* steps_done) {
   cudaStream_t st = stream();
   const int nc = imaginary ? 1 : 2;
   const long long N = ctx.ndet, qs = (long long)nc * N;
@@ -318,6 +318,7 @@ static int propagate_steps(Context& ctx, Context* cpl, double* c, int nsteps, do
       diag[2 * step + 1] = h.alpha[0];
     }
     ISCSI_CUDA(cudaMemcpyAsync(ctl, &up, sizeof(PrCtl), cudaMemcpyHostToDevice, st));
+    *steps_done = step + 1;
     k_pr_combine<<<gb, kPrThreads, 0, st>>>(Q, qs, mm, c, nc, N, ctl); ISCSI_COUNT_LAUNCH();
     ISCSI_CUDA(cudaGetLastError());
     ISCSI_CUDA(cudaStreamSynchronize(st));  // 'up' is read by the copy
@@ -326,8 +327,8 @@ static int propagate_steps(Context& ctx, Context* cpl, double* c, int nsteps, do
 }
 
 int propagate_run(Context& ctx, Context* cpl, double* c, int nsteps, double dt, const double* field, int m,
-                  int imaginary, double* diag) {
-  int s = propagate_steps(ctx, cpl, c, nsteps, dt, field, m, imaginary, diag);
+                  int imaginary, double* diag, int* steps_done) {
+  int s = propagate_steps(ctx, cpl, c, nsteps, dt, field, m, imaginary, diag, steps_done);
   // the context's string matrices lose the step's one-body term, also after an error
   int r = cpl ? onebody_shift(ctx, *cpl, 0.0) : kOk;
   return s != kOk ? s : r;

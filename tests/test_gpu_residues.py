@@ -352,6 +352,40 @@ def leave_free(nbytes):
     return torch.empty(torch.cuda.mem_get_info()[0] - nbytes, dtype=torch.uint8, device="cuda")
 
 
+def test_residues_make_room_for_another_context():
+    """A context whose workspaces do not fit beside another one's residues (1.5 GB) gets their memory."""
+    n = 60
+    ints = [make_integrals(n, 7900 + i, ell=4.0, nchol=12) for i in range(2)]
+    refs, hs = [], []
+    for h1, eri in ints:
+        L.iscsi_init(n, 2, 2, 4, h1, eri, 1e-14)
+        c = unit_vector(L.iscsi_ndet(), 3)[None]
+        L.iscsi_set_option("fp64_tc", 0)
+        refs.append(sigma(c, 1))
+        L.iscsi_set_option("fp64_tc", 1)
+        L.iscsi_finalize()
+    for h1, eri in ints:
+        L.iscsi_init(n, 2, 2, 4, h1, eri, 1e-14)
+        hs.append(L.iscsi_ctx_current())
+    dev = torch.as_tensor(c, device="cuda")
+    out = torch.empty_like(dev)
+    L.iscsi_ctx_use(hs[0])
+    L.iscsi_sigma(dev, out, 1)
+    assert L.iscsi_stats()["residues"]["items"] > 0
+    hog = leave_free(100 << 20)  # the second one's lifted vector and product take 208 MB
+    try:
+        got = []
+        for h in (hs[1], hs[0]):
+            L.iscsi_ctx_use(h)
+            L.iscsi_sigma(dev, out, 1)
+            got.append(out.cpu().numpy())
+    finally:
+        hog = None
+        torch.cuda.empty_cache()
+    check(got[0], refs[1])
+    check(got[1], refs[0])
+
+
 def test_residues_refused_for_a_large_block_only():
     """A block whose residues do not fit (40 vectors: 5 GB of 3.4 free) takes the slices; smaller ones take residues,
     before and after."""
