@@ -1345,6 +1345,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
       }
     }
   }
+  if (out_elems >> 35) return kErrNoMem;  // k_crt_fold addresses 16-byte units of it with 32 bits
   if (S.out.bytes < sizeof(int16_t) * out_elems) ISCSI_TRY(crt_alloc(S.out, sizeof(int16_t) * out_elems, S.held));
   for (size_t i = 0; i < S.job.probs.size(); ++i) S.job.probs[i].p.res = S.out.as<int16_t>() + out_off[i];
   F.res = S.out.as<int16_t>();

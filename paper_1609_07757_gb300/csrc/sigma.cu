@@ -130,13 +130,11 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
   }
 }
 
-// Thin problems (N <= 16 columns, e.g. the single allowed beta string of the
-// highest-level CISD block): one warp per output row, lanes split K, the
-// per-column partial sums are reduced with shuffles, of the columns there are only, in fours (an FP64
-// addition takes 64 cycles a warp; all 16 and a serial sum of the chunks in k_mthin_reduce:
-// CISD, 100 orbitals 0.710 ms, 200 orbitals 4.76, now 0.687 and 4.71).  The column count is
-// a template parameter so no FMA is spent on absent columns.  The K loops stay rolled: four to sixteen
-// loads in flight cost occupancy (200 orbitals: 4.87 to 5.02 ms).
+// Thin problems (N <= 16 columns, e.g. the single allowed beta string of the highest-level CISD block): one warp per
+// output row, lanes split K, the column count a template parameter.  The lanes' sums are added by
+// shuffles for the columns there are, four columns side by side: an FP64 addition takes 64 cycles a warp.  (CISD, 100
+// orbitals: 0.710 ms with all 16 columns added, 0.687 so; 200 orbitals 4.76, 4.71.)  The K loops stay rolled: four to
+// sixteen loads in flight cost occupancy (200 orbitals: 4.87 to 5.02 ms).
 template <typename T, int NB>
 __device__ __forceinline__ void thin_row_seg(T (&acc)[16], const T* __restrict__ Ap, const T* __restrict__ Bp,
                                              int K, long long ldb, int lane) {
@@ -908,11 +906,15 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
   return kOk;
 }
 
-// The slices skip screened blocks of the integrals, the residue products do not.  One sigma,
-// slices / residues, by the share of opposite-spin integrals kept (CISDT in a box): 0.98 3.17 / 1.39 ms,
-// 0.78 16.3 / 8.2, 0.55 50.7 / 38.7; the square of a one-body operator (full CI, 60 orbitals, 0.004)
-// 1.02 / 1.26.  The line through these meets 1 between 0.3 and 0.45.
-constexpr double kCrtMinKept = 0.45;
+// The slices skip screened blocks of the integrals, the residue products do not.  Time of the residues over
+// that of the slices, by the share of opposite-spin integrals kept (tau raised from 1e-14 to 0.01):
+//   full CI, 60 orbitals     1 0.48, 0.36 0.56, 0.14 0.70, 0.08 0.79, 0.04 0.90, 0.013 1.06
+//   80 orbitals              0.91 0.48, 0.30 0.59, 0.14 0.76, 0.07 0.92, 0.03 1.15
+//   100 orbitals             0.99 0.53, 0.34 0.63, 0.12 0.86, 0.05 1.13
+//   CISDT in a box, 100      0.98 0.46, 0.34 0.58, 0.12 0.79, 0.05 0.97, 0.02 1.07
+//   150 orbitals             0.78 0.56, 0.31 0.70, 0.16 0.86, 0.10 0.99, 0.05 1.19
+constexpr double kCrtMinKept = 0.1;
+
 // Where the residues win over the slices otherwise, from 950 spaces and block sizes of 1 to 12 vectors (1 + 1 to 7 + 1
 // electrons, every truncation).  One sigma in ms: residues in both parts, in the same-spin part alone, slices.
 //  * Opposite spin.  The fold adds na nb residues per modulus and determinant where k_fold adds na nb doubles, and in a
