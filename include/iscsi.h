@@ -149,6 +149,25 @@ ISCSI_API iscsi_status iscsi_init_gas(int norb, int nalpha, int nbeta, int nspac
  *   sigma  device, FP64, [nvec][ndet]; overwritten; must not overlap c.
  * Arithmetic follows the "precision" option (64: FP64 throughout; 32: FP32
  * products and accumulation, inputs rounded to FP32, result widened to FP64).
+ * FP64 products on the tensor cores (option "fp64_tc") run through residue
+ * numbers or through error-free slices, as the space and nvec suit.  Through
+ * residues a vector's coefficients are integers of at least 58 bits below its
+ * largest one, the integrals of at least 49, and a sigma element is formed
+ * exactly and rounded once:
+ *   |error of sigma_I| <= 2^-58 max|c| sum_J |H_IJ| + 2^-50 g sum_J n_IJ |c_J|
+ * with g the largest integral and n_IJ the integrals that meet in H_IJ; an
+ * element that only coefficients below 2^-58 max|c| reach is lost.  The slices
+ * keep 49 bits below the largest coefficient that a column (all determinants
+ * sharing na - 1 alpha and nb - 1 beta orbitals) holds.  Infinities and NaN in
+ * c: through residues sigma is NaN at the determinants within two excitations
+ * of one (everywhere beyond 64 of them in a vector), otherwise unaffected.
+ * Device memory: the workspaces stay with the context (16 bytes per element
+ * of the lifted vector, ndet times the pairs that a determinant leaves, and
+ * 14 per element for the slices); residues take 26 bytes per element of the
+ * integrals, string matrices, lifted vector and product, but at most half of
+ * the memory that the process would have free without them (a block of
+ * vectors beyond that takes the slices), and any call that runs out of memory
+ * takes them back first.
  * Asynchronous on the library stream; does not synchronise except the first
  * time a new nvec is used (work lists are uploaded once per nvec).  A bounded
  * device wait that runs out inside the tensor-core kernels is reported as
@@ -211,12 +230,15 @@ ISCSI_API iscsi_status iscsi_sigma_host(const double* c, double* sigma, int nvec
  *   d1   device, FP64 [2][n][n], or NULL;  d2: device, FP64 [3][n^4], or NULL
  *        (at least one of them); overwritten.
  * The two-body blocks are FP64-accurate products of lifted vectors on the
- * tensor cores (exact bf16 slices); the first call with d2 builds the string
- * tables and work lists and synchronises; later calls are asynchronous on the
- * library stream.  Workspace: about 14 bytes per element of the lifted
- * vectors (n^2 rows x the hole-pair count for the alpha-beta block) plus the
- * pair-indexed results (n^4 doubles); a ket different from bra adds its own
- * slices.  A bounded device wait that runs out is reported by the next
+ * tensor cores: residue numbers with a scale per orbital pair (50 bits and
+ * more below the pair's largest coefficient; an infinity or NaN makes the
+ * elements of its pairs NaN), or exact bf16 slices for thin blocks and where
+ * the residues do not fit (as in iscsi_sigma).  The first call with d2 builds
+ * the string tables and work lists and synchronises; later calls are
+ * asynchronous on the library stream.  Workspace: about 26 bytes (slices 14)
+ * per element of the lifted vectors (n^2 rows x the hole-pair count for the
+ * alpha-beta block) and of the pair-indexed results, plus the latter in FP64
+ * (n^4 doubles); a ket different from bra adds its own lifted vectors.  A bounded device wait that runs out is reported by the next
  * synchronising call.
  * Errors: ISCSI_E_NOINIT, ISCSI_E_ARG (bra NULL, both outputs NULL), ISCSI_E_NOMEM,
  * ISCSI_E_CUDA.
@@ -414,11 +436,13 @@ ISCSI_API iscsi_status iscsi_set_stream(void* stream);
  *                      preconditioner; 0: plain diagonal preconditioner
  *   "fp64_tc"          1 (default): with precision 64, the opposite-spin
  *                      contraction runs on the bf16 tensor cores with FP64
- *                      accuracy (operands cut into exact 7-bit slices, exact
- *                      integer accumulation of the leading levels; relative
- *                      error ~1e-14 of sum |g||c|); 0: native FP64 FMA
+ *                      accuracy (residue numbers, or exact 7-bit slices with
+ *                      exact integer accumulation of the leading levels;
+ *                      error ~1e-14 of the 2-norm, element by element as
+ *                      given at iscsi_sigma); 0: native FP64 FMA
  *   "samespin_tc"      1 (default): the same for the same-spin level blocks
  *                      with more than 16 rows and 16 allowed beta strings
+ *                      (through residues all blocks at once)
  *   "fp32_tc"          1 (default): with precision 32, both contractions run
  *                      on the tensor cores with three bf16 terms per element
  *                      and FP32 accumulation; 0: FP32 FMA kernels
@@ -443,7 +467,9 @@ ISCSI_API iscsi_status iscsi_set_option(const char* key, double value);
  * surviving units and in-space determinant pairs), last sigma time, and of
  * the last iscsi_davidson: iterations, those of the FP32 phase, whether a
  * captured graph was replayed, time, and the largest residual norm per
- * iteration ("davidson_rmax", up to 400 values).
+ * iteration ("davidson_rmax", up to 400 values); of the FP64 sigma's residue
+ * products "residues" (bf16 flops, work items, CTAs, moduli; zeros: none), and
+ * whether slices of the string matrices are held ("samespin_slices").
  * Errors: ISCSI_E_NOINIT, ISCSI_E_ARG (also when len is too small; the
  * truncated text is still written).
  */
@@ -468,7 +494,9 @@ ISCSI_API void iscsi_finalize(void);
  * caller owns them).  The precision option applies to all.  The tensor-core
  * contractions of all contexts run as one launch each; from the second call
  * with the same handles, pointers, nvec and precision the whole batch is
- * replayed from one captured CUDA graph (option "use_graph").  The FP64
+ * replayed from one captured CUDA graph (option "use_graph"); another call on
+ * one of the contexts that moves its buffers, lists or scales (another nvec,
+ * a propagation under a strong field) has the batch captured again.  The FP64
  * contraction's schedule covers the whole launch and may cut a tile along K
  * at other points than a single-context call would (each part is rounded to
  * FP64 before the parts are added), so sigma_i agrees with iscsi_sigma on

@@ -8,8 +8,8 @@
 // accurate matrix products this way: Ozaki, Uchino, Imamura, "Ozaki Scheme II",
 // arXiv:2504.08009).  With m_i <= 513 the symmetric residues are at most 256 in
 // magnitude, integers that bf16 holds exactly, so a residue matrix costs ONE
-// bf16 tensor-core product: 12 or 13 products for FP64 accuracy where the
-// error-free slices of ozaki.cuh need 28.  A chunk of 256 K sums products of
+// bf16 tensor-core product: 13 products for FP64 accuracy where the error-free
+// slices of ozaki.cuh need 28.  A chunk of 256 K sums products of
 // at most 2^16 to at most 2^24: exact in the FP32 accumulator whatever its
 // rounding.  Each chunk is reduced modulo m_i and the residues added up.
 #pragma once

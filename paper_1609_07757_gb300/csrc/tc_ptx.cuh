@@ -241,10 +241,9 @@ TC_DEVI unsigned long long add2(unsigned long long a, unsigned long long b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// Shared-memory matrix descriptor, K-major with the 128-byte swizzle (the
-// layout TMA writes for a box whose rows are 128 bytes under
-// CU_TENSOR_MAP_SWIZZLE_128B): 8-row groups 1024 bytes apart; the 16-deep K
-// steps inside the 128-byte row start 32 bytes apart.
+// Shared-memory matrix descriptors, K-major (the layout TMA writes for a box whose rows are 64 or
+// 128 bytes under CU_TENSOR_MAP_SWIZZLE_64B / _128B): 8-row groups 512 or 1024 bytes apart; the
+// 16-deep K steps inside a row start 32 bytes apart.
 TC_DEVI uint64_t smem_desc_sw64(uint32_t saddr) {
   uint64_t d = (uint64_t)((saddr & 0x3FFFF) >> 4);
   d |= (uint64_t)1 << 16;             // leading byte offset: unused for this layout
