@@ -1077,8 +1077,8 @@ def run_gas(name, steps=10, warmup=3, with_cpu=True, projected=True):
         ach = flops / (gemm_ms * 1e-3) / 1e12
         roof = {"bound": "tensor", "achieved": round(ach, 4), "peak": peak, "unit": "TFLOP/s",
                 "frac": round(ach / peak, 4),
-                "traffic": None if residues else
-                profile_traffic("k_oz_gemm%s_gas_%s" % ("_both" if both else "", name))[0],
+                "traffic": profile_traffic("k_crt_gemm_gas_%s" % name if residues else
+                                           "k_oz_gemm%s_gas_%s" % ("_both" if both else "", name))[0],
                 "kernel": "k_crt_gemm (tcgen05 CTA pairs, one bf16 product per modulus)" if residues else
                 "k_oz_gemm (tcgen05, FP64-accurate, %s)" % (
                     "opposite- and same-spin contractions in one launch" if both else "opposite-spin"),

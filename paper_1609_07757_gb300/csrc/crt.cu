@@ -53,7 +53,7 @@ namespace iscsi {
 constexpr double kCrtUnitBits = 49.9;  // least bits of the largest unit (the error-free slices: 49)
 constexpr int kCrtUnitBitsMax = 52;    // bits that are left over go to the unit up to here, then to the coefficients
 constexpr int kCrtCBits = 58;          // least bits of the largest coefficient
-constexpr int kCrtIntBits = 62;        // integers stay below 2^62 (crt_limbs2)
+constexpr int kCrtCBitsMax = 59, kCrtIntBits = 62;  // of coefficients (four limbs) and of units (five)
 
 // ---------------------------------------------------------------------------
 // constants
@@ -69,7 +69,7 @@ static int mod_inverse(int a, int m) {
   return (int)(t < 0 ? t + m : t);
 }
 
-CrtMods crt_make_mods(int nm) {
+CrtMods crt_make_mods(int nm, int limbs) {
   CrtMods c;
   std::memset(&c, 0, sizeof(c));
   c.nm = nm;
@@ -85,10 +85,7 @@ CrtMods crt_make_mods(int nm) {
       return twice((float)(2 * r > m ? r - m : r));
     };
     c.m[i] = m;
-    c.c1[i] = sym(1ll << 13);
-    c.c2[i] = sym(1ll << 26);
-    c.c3[i] = sym(1ll << 39);
-    c.c4[i] = sym(1ll << 52);
+    for (int k = 1; k < limbs; ++k) c.c[k - 1][i] = sym(1ll << ((limbs == 4 ? 15 : 13) * k));
     c.inv[i] = twice(1.0f / (float)m);
     c.neg[i] = twice(-(float)m);
   }
@@ -204,14 +201,14 @@ __global__ void __launch_bounds__(256) k_crt_cut(const double* __restrict__ X, i
   // neighbouring threads read neighbouring elements: chunks of a row, or rows of a transposed matrix
   const int r = trans ? (int)(t % rows_pad) : (int)(t / nch);
   const int kc = trans ? (int)(t / rows_pad) : (int)(t % nch);
-  CrtLimbs2 x[4];
+  CrtLimbs2<5> x[4];
   auto value = [&](int k) -> long long {
     if (r >= rows || k >= cols) return 0;
     const long long rr = map ? map[r] : r, kk = map ? map[k] : k;
     return crt_fixed(trans ? X[kk * ld + rr] : X[rr * ld + kk], 0, sh);
   };
 #pragma unroll
-  for (int j = 0; j < 4; ++j) x[j] = crt_limbs2(value(kc * 8 + 2 * j), value(kc * 8 + 2 * j + 1));
+  for (int j = 0; j < 4; ++j) x[j] = crt_limbs2<5>(value(kc * 8 + 2 * j), value(kc * 8 + 2 * j + 1));
   const int rb = r / bt;
   __nv_bfloat16* o = out + (((long long)rb * nkb + (kc >> 3)) * bt + (r - rb * bt)) * CRT_BK + (kc & 7) * 8;
   crt_store8(x, M, o, (long long)rows_pad * nkb * CRT_BK);
@@ -357,10 +354,10 @@ __global__ void __launch_bounds__(256) k_crt_operands(const __grid_constant__ Cr
       double val[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) val[j] = kc * 8 + j < G.krows ? crt_lift_value(L, qs[j], cv) : 0.0;
-      CrtLimbs2 x[4];
+      CrtLimbs2<4> x[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        x[j] = crt_limbs2(crt_fixed(val[2 * j], ex, O.cbits), crt_fixed(val[2 * j + 1], ex, O.cbits));
+        x[j] = crt_limbs2<4>(crt_fixed(val[2 * j], ex, O.cbits), crt_fixed(val[2 * j + 1], ex, O.cbits));
       crt_store8(x, M, row + (long long)(kc >> 3) * G.bt * CRT_BK + (kc & 7) * 8, G.mod_stride);
     }
     return;
@@ -386,10 +383,10 @@ __global__ void __launch_bounds__(256) k_crt_operands(const __grid_constant__ Cr
     const int r = (i & 511) >> 3, kc = i & 7;
     const int R = (tr ? B0 : A0) + r;
     if ((tr ? O.ct : O.ca) == nullptr || R >= (tr ? O.nb : O.na)) continue;
-    CrtLimbs2 x[4];
+    CrtLimbs2<4> x[4];
     auto value = [&](int j) { return crt_fixed(tr ? tile[kc * 8 + j][r] : tile[r][kc * 8 + j], ex, O.cbits); };
 #pragma unroll
-    for (int j = 0; j < 4; ++j) x[j] = crt_limbs2(value(2 * j), value(2 * j + 1));
+    for (int j = 0; j < 4; ++j) x[j] = crt_limbs2<4>(value(2 * j), value(2 * j + 1));
     const int bt = tr ? O.bt : CRT_BM, rb = R / bt, kb = (tr ? A0 : B0) / CRT_BK;
     __nv_bfloat16* o = (tr ? O.ct + z * O.ct_vec : O.ca + z * O.ca_vec) +
                        (((long long)rb * (tr ? O.nkb_ct : O.nkb_ca) + kb) * bt + (R - rb * bt)) * CRT_BK + kc * 8;
@@ -767,7 +764,7 @@ struct CrtState {
   std::vector<int> ypad;
   DevBuf pair, map, rowrun, colrun, ypos;
   // scales: units are integers of 2^-sh
-  CrtMods mods;
+  CrtMods mods, unit_mods;              // of the vectors, and of G and the string matrices
   int sh = 0, cbits = 0;                // and a vector's coefficients of 2^(e - cbits)
   double bound = 0.0;                   // the bound of |sigma| / max |c| that sh was chosen for
   int g_cut[2] = {-1, 0}, m_cut[2] = {-1, 0};  // moduli and sh of the residues in g_res, ma_res / mb_res
@@ -1009,7 +1006,7 @@ static void choose_scale(double bound, double maxel, double ref, int& nm, int& s
     sh = std::min(cap, (int)std::floor(room - kCrtCBits));
     if (nm < kCrtMaxMods && sh < cap && room - kCrtCBits + std::log2(ref) < kCrtUnitBits) continue;
     sh = std::min(sh, (int)std::ceil(kCrtUnitBitsMax - std::log2(ref)));
-    cbits = std::min(kCrtIntBits, (int)std::floor(room - sh));
+    cbits = std::min(kCrtCBitsMax, (int)std::floor(room - sh));
     return;
   }
 }
@@ -1025,7 +1022,7 @@ static int crt_cut_m(Context& ctx) {
     const int rp = up(NA, 2 * CRT_BM);
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)S.mods.nm * rp * ka * CRT_BK;
     if (S.ma_res.bytes < bytes) ISCSI_TRY(crt_alloc(S.ma_res, bytes, S.held));
-    ISCSI_TRY(cut_matrix(ctx.M64[0].as<double>(), NA, NA, ctx.sp[0].count, 0, nullptr, S.sh, CRT_BM, rp, ka, S.mods,
+    ISCSI_TRY(cut_matrix(ctx.M64[0].as<double>(), NA, NA, ctx.sp[0].count, 0, nullptr, S.sh, CRT_BM, rp, ka, S.unit_mods,
                          S.ma_res.as<__nv_bfloat16>(), st));
   }
   if (ctx.nb > 0) {
@@ -1034,7 +1031,7 @@ static int crt_cut_m(Context& ctx) {
     const int rp = tn * ntile;
     const size_t bytes = sizeof(__nv_bfloat16) * (size_t)S.mods.nm * rp * kb * CRT_BK;
     if (S.mb_res.bytes < bytes) ISCSI_TRY(crt_alloc(S.mb_res, bytes, S.held));
-    ISCSI_TRY(cut_matrix(Mb, NB, NB, ctx.sp[1].count, trans, nullptr, S.sh, bt, rp, kb, S.mods,
+    ISCSI_TRY(cut_matrix(Mb, NB, NB, ctx.sp[1].count, trans, nullptr, S.sh, bt, rp, kb, S.unit_mods,
                          S.mb_res.as<__nv_bfloat16>(), st));
   }
   S.m_cut[0] = S.mods.nm;
@@ -1081,6 +1078,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
     choose_scale(b, maxel, (parts & 1) ? S.gmax : mmax, nm, S.sh, S.cbits);
     S.bound = b;
     S.mods = crt_make_mods(nm);
+    S.unit_mods = crt_make_mods(nm, 5);
   }
   const int nm = S.mods.nm;
   S.job.probs.clear();
@@ -1182,7 +1180,7 @@ static int crt_build(Context& ctx, int nvec, int parts) {
       S.g_cut[0] = -1;
     }
     if (S.g_cut[0] != nm || S.g_cut[1] != S.sh) {
-      ISCSI_TRY(cut_matrix(ctx.G64.as<double>(), np, np, np, 0, S.map.as<int>(), S.sh, CRT_BM, rp, gk, S.mods,
+      ISCSI_TRY(cut_matrix(ctx.G64.as<double>(), np, np, np, 0, S.map.as<int>(), S.sh, CRT_BM, rp, gk, S.unit_mods,
                            S.g_res.as<__nv_bfloat16>(), st));
       S.g_cut[0] = nm;
       S.g_cut[1] = S.sh;

@@ -34,54 +34,57 @@ __device__ __forceinline__ long long crt_fixed(double v, int e, int bits) {
   return b < 0 ? -N : N;
 }
 
-// Two integers |N| <= 2^62 as N = l0 + l1 2^13 + l2 2^26 + l3 2^39 + l4 2^52 (0 <= l0 .. l3 < 2^13,
-// |l4| <= 2^10), the limbs as packed FP32: a limb in the low mantissa bits of 2^23 (l4, signed: added to
-// 1.5 2^23), less that constant.  LIMBS = 4: |N| <= 2^52, l3 signed, no l4.
+// Two integers in limbs as packed FP32: a limb in the low mantissa bits of 2^23, less a constant.
+// LIMBS = 4, |N| <= 2^59: N = l0 + l1 2^15 + l2 2^30 + l3 2^45 with -2^14 <= l0, l1, l2 < 2^14
+// (balanced: the fields of N + 2^14 (1 + 2^15 + 2^30), less 2^14) and |l3| <= 2^14.
+// LIMBS = 5, |N| <= 2^62: l0 + l1 2^13 + .. + l4 2^52, 0 <= l0 .. l3 < 2^13, |l4| <= 2^10.
+template <int LIMBS>
 struct CrtLimbs2 {
-  unsigned long long l0, l1, l2, l3, l4;
+  unsigned long long l[LIMBS];
 };
-template <int LIMBS = 5>
-__device__ __forceinline__ CrtLimbs2 crt_limbs2(long long a, long long b) {
-  auto mant = [](uint32_t x) { return (x & 0x1FFFu) | 0x4B000000u; };
-  auto pair = [](uint32_t lo, uint32_t hi) { return ((unsigned long long)hi << 32) | lo; };
-  const unsigned long long k0 = pair(0xCB000000u, 0xCB000000u);  // -2^23, twice
-  const int ah = (int)(a >> 32), bh = (int)(b >> 32);
-  CrtLimbs2 r;
-  r.l0 = tc::add2(pair(mant((uint32_t)a), mant((uint32_t)b)), k0);
-  r.l1 = tc::add2(pair(mant((uint32_t)a >> 13), mant((uint32_t)b >> 13)), k0);
-  r.l2 = tc::add2(pair(mant((uint32_t)(a >> 26)), mant((uint32_t)(b >> 26))), k0);
-  auto top = [&](int x, int y) {
-    return tc::add2(pair(0x4B400000u + (uint32_t)x, 0x4B400000u + (uint32_t)y), pair(0xCB400000u, 0xCB400000u));
-  };
+template <int LIMBS>
+__device__ __forceinline__ CrtLimbs2<LIMBS> crt_limbs2(long long a, long long b) {
+  static_assert(LIMBS == 4 || LIMBS == 5, "limbs of 15 or of 13 bits");
+  constexpr int W = LIMBS == 4 ? 15 : 13;
+  constexpr uint32_t kMask = (1u << W) - 1, kBias = LIMBS == 4 ? 1u << 14 : 0u;
   if (LIMBS == 4) {
-    r.l3 = top(ah >> 7, bh >> 7);
-    r.l4 = 0;
-  } else {
-    r.l3 = tc::add2(pair(mant((uint32_t)ah >> 7), mant((uint32_t)bh >> 7)), k0);
-    r.l4 = top(ah >> 20, bh >> 20);
+    constexpr long long kAll = (1ll << 14) + (1ll << 29) + (1ll << 44);
+    a += kAll;
+    b += kAll;
   }
+  auto mant = [](long long x) { return ((uint32_t)x & kMask) | 0x4B000000u; };
+  auto pair = [](uint32_t lo, uint32_t hi) { return ((unsigned long long)hi << 32) | lo; };
+  const unsigned long long k0 = pair(0xCB000000u + kBias, 0xCB000000u + kBias);  // -(2^23 + bias), twice
+  CrtLimbs2<LIMBS> r;
+#pragma unroll
+  for (int i = 0; i + 1 < LIMBS; ++i) r.l[i] = tc::add2(pair(mant(a >> (W * i)), mant(b >> (W * i))), k0);
+  // the last one signed: added to 1.5 2^23
+  r.l[LIMBS - 1] = tc::add2(pair(0x4B400000u + (uint32_t)(int)(a >> (W * (LIMBS - 1))),
+                                 0x4B400000u + (uint32_t)(int)(b >> (W * (LIMBS - 1)))),
+                            pair(0xCB400000u, 0xCB400000u));
   return r;
 }
 
 // Residues of eight consecutive K values for every modulus, one 16-byte store
-// each.  t = l0 + l1 c1 + .. + l4 c4 is congruent to N, an exact FP32 integer (|t| below
-// 2^22.7); its quotient by m is rounded by adding 1.5 2^23 with an error below 2^-11.5
-// (over the sixteen moduli), under the 1 / (2 m) > 2^-10.1 that separates t / m from a tie, so
-// |t - q m| <= 256 and the upper halves of the floats are the bf16 residues.
-// Packed FP32: 4 instructions per residue (3.5 with four limbs), where integer arithmetic took ~13
-// (4 + 4 electrons in 16 orbitals, operand kernel: 750 us).
-template <int LIMBS = 5>
-__device__ __forceinline__ void crt_store8(const CrtLimbs2 (&x)[4], const CrtMods& M, __nv_bfloat16* out,
+// each.  t = l0 + l1 c1 + .. is congruent to N, an exact FP32 integer (|t| below 2^23.4
+// with four limbs, 2^22.2 with five); its quotient by m is rounded by adding 1.5 2^23 with
+// an error below 0.8 of the 1 / (2 m) that separates t / m from a tie (over the sixteen
+// moduli), so |t - q m| <= 256 and the upper halves of the floats are the bf16 residues.
+// Packed FP32, 3.5 instructions per residue with four limbs, 4 with five, which bound it (five limbs: full
+// CI in 60 orbitals 188 us, 4 + 4 electrons in 16 787; four 161 and 667); integer arithmetic took ~13.
+template <int LIMBS>
+__device__ __forceinline__ void crt_store8(const CrtLimbs2<LIMBS> (&x)[4], const CrtMods& M, __nv_bfloat16* out,
                                            long long mod_stride) {
   const unsigned long long mg = tc::f32x2(12582912.0f, 12582912.0f), ng = tc::f32x2(-12582912.0f, -12582912.0f);
 #pragma unroll 2
   for (int i = 0; i < M.nm; ++i) {
-    const unsigned long long c1 = M.c1[i], c2 = M.c2[i], c3 = M.c3[i], c4 = M.c4[i], inv = M.inv[i], neg = M.neg[i];
+    const unsigned long long inv = M.inv[i], neg = M.neg[i];
     uint32_t pk[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      unsigned long long t = tc::fma2(x[j].l3, c3, tc::fma2(x[j].l2, c2, tc::fma2(x[j].l1, c1, x[j].l0)));
-      if (LIMBS == 5) t = tc::fma2(x[j].l4, c4, t);
+      unsigned long long t = x[j].l[0];
+#pragma unroll
+      for (int k = 1; k < LIMBS; ++k) t = tc::fma2(x[j].l[k], M.c[k - 1][i], t);
       const unsigned long long q = tc::add2(tc::fma2(t, inv, mg), ng);
       const unsigned long long r = tc::fma2(q, neg, t);
       pk[j] = __byte_perm((uint32_t)r, (uint32_t)(r >> 32), 0x7632);

@@ -30,9 +30,9 @@ struct CrtJob {
   int launch(int* err, cudaStream_t st) const;
 };
 
-// constants of the first nm moduli; weights of the reconstruction from sums of `terms`
+// constants of the first nm moduli for integers in four or five limbs; weights of the reconstruction from sums of `terms`
 // stored residues (later passes: terms_next each); log2 of the moduli's product
-CrtMods crt_make_mods(int nm);
+CrtMods crt_make_mods(int nm, int limbs = 4);
 CrtWeights crt_make_weights(int nm, int terms, int terms_next = 0, int passes_next = 0);
 double crt_log2_product(int nm);
 // Bytes of residue buffers of one user, counted for the process as well.

@@ -27,12 +27,12 @@ constexpr int CRT_THREADS = 64 + 32 * CRT_EPI_WARPS;
 constexpr int kCrtModuli[kCrtMaxMods] = {513, 512, 511, 509, 505, 503, 499, 493, 491, 487, 481, 479, 473, 467, 463, 461};
 
 // Constants of the first nm moduli, each FP32 value twice in a 64-bit word
-// (packed operations on two elements): 2^13, 2^26, 2^39 and 2^52 mod m (symmetric),
-// 1 / m and -m.
+// (packed operations on two elements): the limbs' weights mod m (symmetric: 2^15, 2^30 and
+// 2^45, or 2^13, 2^26, 2^39 and 2^52 for five limbs), 1 / m and -m.
 struct CrtMods {
   int nm;
   int m[kCrtMaxMods];
-  unsigned long long c1[kCrtMaxMods], c2[kCrtMaxMods], c3[kCrtMaxMods], c4[kCrtMaxMods], inv[kCrtMaxMods], neg[kCrtMaxMods];
+  unsigned long long c[4][kCrtMaxMods], inv[kCrtMaxMods], neg[kCrtMaxMods];
 };
 
 // Reconstruction S = F M, F = sum_i r_i (M/m_i)^-1 / m_i mod 1, as a 78-bit

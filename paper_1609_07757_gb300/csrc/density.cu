@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(256, 4) k_dm_cut(const __grid_constant__ DmCut
 #pragma unroll
           for (int j = 0; j < 8; ++j) keep[j][threadIdx.x] = v[j];
       } else {
-        CrtLimbs2 x[4];
+        CrtLimbs2<4> x[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) x[j] = crt_limbs2<4>(crt_fixed(v[2 * j], 0, sc), crt_fixed(v[2 * j + 1], 0, sc));
         crt_store8<4>(x, M, row + (long long)(kc >> 3) * (CRT_BM * CRT_BK) + (kc & 7) * 8, K.mod_stride);
