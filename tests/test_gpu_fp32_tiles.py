@@ -48,3 +48,22 @@ def test_fp32_form_against_fp64(n, na, nb, k, nvec):
     L.iscsi_set_option("precision", 64)
     for v in range(nvec):
         assert np.linalg.norm(out[32][v] - out[64][v]) <= REL32 * np.linalg.norm(out[64][v])
+
+
+@pytest.mark.parametrize("n,na,nb,k", [(24, 2, 2, 4), (22, 3, 2, 5), (44, 2, 2, 3)])
+def test_fp32_form_bits_do_not_depend_on_the_tiles(n, na, nb, k):
+    # one vector fills a wave of narrow tiles at most, a block of sixteen many: the launch takes another tile width and
+    # other tiles, and every vector comes out with the same bits
+    h1, eri = make_integrals(n, 90 + n, ell=4.0, nchol=8)
+    L.iscsi_init(n, na, nb, k, h1, eri, 1e-14)
+    c = torch.as_tensor(np.stack([unit_vector(L.iscsi_ndet(), 7 + v) for v in range(16)]), device="cuda")
+    L.iscsi_set_option("precision", 32)
+    try:
+        block = torch.empty_like(c)
+        L.iscsi_sigma(c, block, 16)
+        one = torch.empty_like(c[:1])
+        for v in (0, 5, 15):
+            L.iscsi_sigma(c[v:v + 1], one, 1)
+            assert torch.equal(one[0], block[v])
+    finally:
+        L.iscsi_set_option("precision", 64)

@@ -416,3 +416,22 @@ def test_residues_refused_for_a_large_block_only():
         torch.cuda.empty_cache()
     # (a block on the slices leaves the smaller one's residues where they are)
     assert items[0] > 0 and items[1] == 0 and items[2] == items[0]
+
+
+# thin blocks of many rows (on the slices), just below and above the lines
+@pytest.mark.parametrize("n,na,nb,k,transition", [(26, 2, 1, 3, False), (30, 2, 1, 3, True), (27, 1, 1, 2, True),
+                                                  (25, 1, 1, 2, False), (40, 2, 0, 2, False), (24, 1, 1, 2, True)])
+def test_density_thin_blocks(n, na, nb, k, transition):
+    h1, eri = make_integrals(n, 80 + n, ell=3.0, nchol=6)
+    L.iscsi_init(n, na, nb, k, h1, eri, 0.0)
+    nd = L.iscsi_ndet()
+    bra = unit_vector(nd, 5)
+    ket = unit_vector(nd, 6) if transition else bra
+    d1 = torch.full((2, n, n), float("nan"), dtype=torch.float64, device="cuda")
+    d2 = torch.full((3, n, n, n, n), float("nan"), dtype=torch.float64, device="cuda")
+    b = torch.as_tensor(bra, device="cuda")
+    L.iscsi_density(b, torch.as_tensor(ket, device="cuda") if transition else None, d1, d2)
+    from oracle import Oracle
+    r1, r2 = Oracle(n, na, nb, k, 0.0, h1, eri).density(bra, ket)
+    for got, ref in [(d1.cpu().numpy(), np.asarray(r1))] + list(zip(d2.cpu().numpy(), np.asarray(r2))):
+        assert np.abs(got - ref).max() <= 1e-12 * max(np.abs(ref).max(), 1e-300)
