@@ -12,7 +12,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from paper_1609_07757_gb300 import _lib as L
-from paper_1609_07757_gb300.synthetic import make_integrals, unit_vector
+from paper_1609_07757_gb300.synthetic import make_integrals, transition_operator, unit_vector
 
 pytestmark = pytest.mark.gpu
 
@@ -435,3 +435,25 @@ def test_density_thin_blocks(n, na, nb, k, transition):
     r1, r2 = Oracle(n, na, nb, k, 0.0, h1, eri).density(bra, ket)
     for got, ref in [(d1.cpu().numpy(), np.asarray(r1))] + list(zip(d2.cpu().numpy(), np.asarray(r2))):
         assert np.abs(got - ref).max() <= 1e-12 * max(np.abs(ref).max(), 1e-300)
+
+
+@pytest.mark.parametrize("kind", ["transition", "dense"])
+def test_autotune_times_slices_for_one_body_operators(kind):
+    """An operator without a two-body part: the slices skip the zero blocks of its string matrices, the residues do
+    not, so both are timed; what the loser held is given back."""
+    n = 60
+    h1 = transition_operator(n, n - 1, 0) if kind == "transition" else make_integrals(n, 8100, ell=4.0, nchol=12)[0]
+    L.iscsi_init(n, 2, 2, 4, h1, None, 0.0)
+    c = unit_vector(L.iscsi_ndet(), 6)[None]
+    L.iscsi_set_option("autotune", 1)
+    s = sigma(c, 1)
+    st = L.iscsi_stats()
+    L.iscsi_set_option("autotune", 0)
+    timed = {t[1]: t[3] for t in st["route_fp64"]["trials"] if t[0] == 1 and t[3] >= 0}
+    assert 16 in timed and 64 in timed
+    if timed[64] < min(t for k, t in timed.items() if k != 64):
+        assert st["residues"]["items"] == 0 and st["samespin_slices"] == 1
+    if timed[16] < min(t for k, t in timed.items() if k != 16):
+        assert st["residues"]["items"] > 0 and st["samespin_slices"] == 0
+    L.iscsi_set_option("fp64_tc", 0)
+    check(s, sigma(c, 1))
