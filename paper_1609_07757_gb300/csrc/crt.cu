@@ -863,7 +863,8 @@ static FoldShape fold_shape(const Context& ctx, const CrtState& S, int lev) {
   const long long units = 8ll * (f.hole / 8 + 8);
   const int together = ctx.na * ctx.nb <= 25 ? ctx.na : 1;  // (at most 26 residues per pass: sums below 2^64)
   // two blocks per SM (113 KB) before all holes in one pass: 4 + 4 electrons in 16 orbitals 182 KB in one
-  // pass 710 us, 91 KB in two passes 545; but one hole per pass is slower (CISDT, 100 orbitals: 302 against 279)
+  // pass 710 us, 91 KB in two passes 545 (12 moduli; 13: 559); but one hole per pass is slower (CISDT, 100
+  // orbitals: 302 against 279)
   const struct { int ni, nbuf; long long limit; } tries[] = {
       {together, 4, 56 * 1024}, {together, 3, 75 * 1024}, {together, 2, 113 * 1024},
       {(together + 1) / 2, 2, together > 2 ? 113 * 1024 : 0}, {together, 2, kFoldMaxSmem}, {1, 2, kFoldMaxSmem}};

@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(256, 4) k_dm_cut(const __grid_constant__ DmCut
 // Q (R x R) from the residues of L_bra L_ket^T: a warp 32 rows x 8 columns, its rows' runs turned
 // across lane octets; ket = bra: only the tiles on and above the diagonal exist, their mirror
 // images are written with them (32 rows of a column at once).  All moduli's loads in flight, one
-// launch for the three blocks (four in flight and a launch per block: 160 us at n = 60, now 88;
+// launch for the three blocks (four in flight and a launch per block: 160 us at n = 60, now 96;
 // the slices' kernel rebuilt in its epilogue and mirrored in 46).
 struct DmRebuild {
   const int16_t* res[3];
