@@ -915,41 +915,39 @@ static int sigma_impl(Context& ctx, const TC* c_in, T* s_out, const T* c, T* sig
 //   150 orbitals             0.78 0.56, 0.31 0.70, 0.16 0.86, 0.10 0.99, 0.05 1.19
 constexpr double kCrtMinKept = 0.1;
 
-// Where the residues win over the slices otherwise, from 950 spaces and block sizes of 1 to 12 vectors (1 + 1 to 7 + 1
-// electrons, every truncation).  One sigma in ms: residues in both parts, in the same-spin part alone, slices.
+// Otherwise the residues, which are more accurate (5 + 1 electrons in 18 orbitals: 1e-14 of the sigma's norm, slices
+// 1.3e-12), but where they gave up most of the slices' speed (1465 spaces and block sizes of 1 to 12 vectors: 1 + 1 to
+// 7 + 1 electrons, every truncation).  One sigma in ms: residues in both parts, in the same-spin part alone, slices.
 //  * Opposite spin.  The fold adds na nb residues per modulus and determinant where k_fold adds na nb doubles, and in a
-//    truncated space its blocks are short: 4 + 4 in 15 orbitals, quadruples 0.78, 0.54, 0.61; 5 + 5 in 12 1.07, 0.51, 0.58;
-//    3 + 3 in 22, doubles, 12 vectors 0.56, 0.42, 0.86; 3 + 2 in 24, quadruples 0.20, 0.22, 0.29.  Full spaces (long rows,
-//    one run of columns) win up to na nb = 16: 4 + 4 in 14 0.89, 0.98, 1.19; 5 + 4 in 11 0.36, 0.29, 0.44.  One or two
-//    alpha electrons have few holes: 1 + 4 in 18, triples 0.10, 0.15, 0.17.  A few thousand elements are bound by launches: 5 + 2
-//    in 14, doubles 0.068, 0.090, 0.136.
-//  * Same spin.  All blocks in one launch, and a launch or two per vector and block less: 3 + 3 in 9, quintuples, 12
-//    vectors 0.18, 0.15, 1.02.  But the whole string matrices are read, 26 bytes an element, where the slices read 14
-//    of the blocks that are there, which counts in sparse truncations of many strings (doubles: 2 + 2 in 70, 2415
-//    strings, this part alone 0.312, slices 0.302, in 100 0.726, 0.665; 3 + 3 in 36, triples, 7140 strings 1.20, 1.11) and
-//    with many strings of one spin beside few of the other (6 + 1 in 18, 18564 and 18: 1.44, 1.45, 1.01).
-constexpr int kCrtFoldFull = 16, kCrtFoldSmall = 12;
-constexpr long long kCrtSmall = 8000;
-constexpr int kCrtStrings = 2048, kCrtThinStrings = 64, kCrtThinOther = 6000;
+//    truncated space its runs are short.  Full spaces: 5 + 4 in 11 orbitals 0.35, 0.30, 0.46; 5 + 5 1.14, 0.75, 1 of the
+//    slices' time.  Truncated, of the slices' time: 5 + 2 in 16, quadruples 0.92, 0.81, 1; 5 + 3 in 13 0.92, 0.75, 1; 4 + 4 in
+//    15 to 18 1.2, 0.9, 1; 5 + 5 in 12 1.8, 0.9, 1.  Where the same-spin part has too few strings (a spin of fewer than 16)
+//    the slices' launches stay: 5 + 1 in 12, quadruples 0.107, slices 0.076, 12 vectors 0.297, 0.225; 1 + 5 in 17, triples
+//    0.219, 0.219, 12 vectors 0.616, 0.870.
+//  * Same spin alone.  The whole string matrices are read, 26 bytes an element, where the slices read 14 of the blocks
+//    that are there, which counts in sparse truncations of many strings (2 + 2 in 70, doubles, 2415 strings, 0.312, slices
+//    0.302; in 100 0.726, 0.665; 4 + 4 in 24, triples 1.08 of the slices' time).  With both parts it is the smaller loss: 3 + 3
+//    in 36, triples 1.13, 5 + 1 in 19 1.07, in 18 0.89, 1 + 3 in 40 0.33 of the slices' time.
+constexpr int kCrtFoldFull = 20, kCrtFoldCut = 15, kCrtFoldFew = 4;
+constexpr int kCrtStrings = 2048;
 constexpr double kCrtDense = 0.02;
 
 int crt_parts(Context& ctx, int nvec) {
   if (ctx.units_opposite_total > 0 && (double)ctx.units_opposite < kCrtMinKept * (double)ctx.units_opposite_total) return 0;
+  // the string matrices elsewhere by an option or the autotuner, or too few strings for a tile: opposite spin alone
+  const bool elsewhere = ctx.route[0].ss_min > kThinN;
+  const bool ss = !elsewhere && samespin_tc_active(ctx) && crt_ss_active(ctx, nvec);
   bool ab = ctx.have_ab && ab_on_tc(ctx, 64) && crt_ab_active(ctx, nvec);
   if (ab) {
-    const int na = ctx.na, nb = ctx.nb, c = na * nb;
+    const int c = ctx.na * ctx.nb;
     ab = crt_full(ctx) ? c <= kCrtFoldFull
-                       : nb <= 4 && (na <= 2 || (na == 3 && nb <= 2) ||
-                                     (c <= kCrtFoldSmall && ctx.ndet * nvec <= kCrtSmall));
+                       : ss || elsewhere ? c <= kCrtFoldCut : c <= kCrtFoldFew || (ctx.na <= 2 && nvec > 1);
   }
-  // the string matrices elsewhere by an option or the autotuner, or too few strings for a tile: opposite spin alone
-  if (ctx.route[0].ss_min > kThinN || !samespin_tc_active(ctx) || !crt_ss_active(ctx, nvec)) return ab ? 1 : 0;
+  if (ab || !ss) return (ab ? 1 : 0) | (ss ? 2 : 0);
   int sa = 0, sb = 0;
   crt_strings(ctx, sa, sb);
-  const int more = std::max(sa, sb), less = std::min(sa, sb);
-  const bool ss = !ctx.have_ab || (!(less <= kCrtThinStrings && more > kCrtThinOther) &&
-                                   (more <= kCrtStrings || (double)ctx.ndet >= kCrtDense * sa * sb));
-  return ss ? (ab ? 3 : 2) : 0;
+  const bool dense = std::max(sa, sb) <= kCrtStrings || (double)ctx.ndet >= kCrtDense * sa * sb;
+  return !ctx.have_ab || dense ? 2 : 0;
 }
 
 static int sigma_steps(Context& ctx, const double* c, double* sigma, int nvec, int precision, int phases) {

@@ -315,7 +315,9 @@ def test_density_nonfinite(n, na, nb, kmax):
 # spin, 1 opposite spin, 0 neither)
 @pytest.mark.parametrize("n,na,nb,kmax,nvec", [(11, 3, 3, 4, 1), (11, 3, 3, 4, 12), (13, 4, 4, 4, 1), (10, 5, 4, 9, 1),
                                                (9, 4, 4, 8, 1), (12, 1, 4, 3, 4), (10, 5, 5, 3, 1), (14, 6, 1, 6, 2),
-                                               (9, 1, 1, 2, 1), (18, 5, 1, 4, 1), (30, 3, 1, 2, 1)])
+                                               (9, 1, 1, 2, 1), (18, 5, 1, 4, 1), (30, 3, 1, 2, 1),
+                                               (13, 5, 1, 4, 1), (13, 1, 5, 4, 1), (13, 1, 5, 4, 2), (12, 5, 3, 4, 1),
+                                               (19, 5, 1, 3, 1), (23, 1, 4, 5, 1), (11, 5, 5, 10, 1)])
 def test_residues_routing(n, na, nb, kmax, nvec):
     h1, eri = make_integrals(n, 7700 + n, ell=3.0, nchol=12)
     L.iscsi_init(n, na, nb, kmax, h1, eri, 1e-14)
@@ -457,3 +459,20 @@ def test_autotune_times_slices_for_one_body_operators(kind):
         assert st["residues"]["items"] > 0 and st["samespin_slices"] == 0
     L.iscsi_set_option("fp64_tc", 0)
     check(s, sigma(c, 1))
+
+
+@pytest.mark.parametrize("n,na,nb,kmax,nvec", [(17, 5, 1, 6, 1), (18, 4, 1, 3, 1), (19, 5, 1, 4, 1), (23, 1, 4, 5, 1),
+                                               (35, 3, 1, 4, 1), (18, 4, 2, 4, 4), (14, 5, 2, 4, 1), (12, 4, 3, 4, 4)])
+def test_residues_for_many_strings_and_electrons(n, na, nb, kmax, nvec):
+    """Many strings of one spin or up to 15 pairs of electrons: both parts through residues, to their accuracy (the
+    rounding of coefficients and integrals, 2^-58 and 2^-50 of the largest, at random in sums of K <= 5e3 terms of
+    like size: below 1e-13 of the norm)."""
+    h1, eri = make_integrals(n, 8200 + n, ell=3.0, nchol=12)
+    L.iscsi_init(n, na, nb, kmax, h1, eri, 1e-14)
+    C = np.stack([unit_vector(L.iscsi_ndet(), 30 + v) for v in range(nvec)])
+    s = sigma(C, nvec)
+    assert L.iscsi_stats()["residues"]["items"] > 0
+    L.iscsi_set_option("fp64_tc", 0)
+    ref = sigma(C, nvec)
+    for v in range(nvec):
+        assert np.linalg.norm(s[v] - ref[v]) <= 1e-13 * np.linalg.norm(ref[v])
