@@ -232,8 +232,8 @@ ISCSI_API iscsi_status iscsi_sigma_host(const double* c, double* sigma, int nvec
  * The two-body blocks are FP64-accurate products of lifted vectors on the
  * tensor cores: residue numbers with a scale per orbital pair (50 bits and
  * more below the pair's largest coefficient; an infinity or NaN makes the
- * elements of its pairs NaN), or exact bf16 slices for thin blocks and where
- * the residues do not fit (as in iscsi_sigma).  The first call with d2 builds
+ * elements of its pairs NaN), or exact bf16 slices where the residues do not
+ * fit (as in iscsi_sigma).  The first call with d2 builds
  * the string tables and work lists and synchronises; later calls are
  * asynchronous on the library stream.  Workspace: about 26 bytes (slices 14)
  * per element of the lifted vectors (n^2 rows x the hole-pair count for the

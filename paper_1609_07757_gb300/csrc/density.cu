@@ -74,20 +74,13 @@ struct DmBlock {
 
 constexpr int kDmMods = 13, kDmModsMax = 16;  // moduli: the fewest with kDmBits bits
 constexpr int kDmBits = 50;                    // (the slices: 49)
-// Short sums over many rows are bound by the result: a residue per modulus and element written and
-// read back, where the slices' kernel writes FP64.  State / transition densities, residues against slices:
-// 2 + 1 electrons in 40 orbitals (40 columns, 1600 rows) 0.165 against 0.134 and 0.203 against 0.155 ms, in 30
-// (900 rows) 0.093, 0.078 and 0.107, 0.085, in 24 (576) 0.072, 0.068 and 0.080, 0.073; 1 + 1 in 100 1.69, 1.57 and
-// 2.46, 1.93.  Few rows are bound by the launches, of which the residues have fewer: 2 + 2 in 8 (64 columns, 64
-// rows) 0.050 against 0.062 and 0.050 against 0.068.  Longer sums tie: 3 + 1 in 40 (780, 1600) 0.218, 0.212.
-constexpr int kDmThinCols = 128, kDmThinRows = 576;
 constexpr int kDmNotFinite = -(1 << 20);  // scale of a row with an infinity or NaN: its elements of the result are NaN
 
 struct DensityPlan {
   bool built = false;
-  // residues (not for thin blocks, nor where they do not fit: ket = bra / general): operands of bra and
+  // residues (unless they do not fit: ket = bra / general): operands of bra and
   // ket, output residues, scales
-  bool thin = false, no_room[2] = {false, false};
+  bool no_room[2] = {false, false};
   CrtHeld res_held;
   DevBuf res_bra, res_ket, res_out, scale;  // scale: per row of bra, of ket, then partial maxima
   int nmods = kDmMods, res_rows = 0;        // moduli; rows of all blocks
@@ -325,17 +318,10 @@ static int plan_build(Context& ctx) {
     }
     if (least >= kDmBits || P.nmods == kDmModsMax) break;
   }
-  int most_cols = 0, most_rows = 0;
   for (DmBlock& B : P.blk) {
     B.row0 = P.res_rows;
-    if (B.parts.empty()) continue;
-    P.res_rows += B.R;
-    int cols = 0;
-    for (const DmPart& pt : B.parts) cols += pt.ncol;
-    most_cols = std::max(most_cols, cols);
-    most_rows = std::max(most_rows, B.R);
+    if (!B.parts.empty()) P.res_rows += B.R;
   }
-  P.thin = most_cols <= kDmThinCols && most_rows > kDmThinRows;
   for (cudaEvent_t& e : P.ev) ISCSI_CUDA(cudaEventCreate(&e));
   P.sl_elems = sl;
   P.q_elems = q;
@@ -1086,7 +1072,7 @@ int density_run(Context& ctx, const double* bra, const double* ket, double* d1, 
     ISCSI_TRY(plan_build(ctx));
     Pp = ctx.dm;
     DensityPlan& P = *Pp;
-    bool res = !P.thin && !P.no_room[sym ? 0 : 1];
+    bool res = !P.no_room[sym ? 0 : 1];
     if (res) {
       const int rc = residues_build(ctx, sym);
       if (rc == kErrNoMem) {

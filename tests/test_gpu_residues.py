@@ -420,7 +420,7 @@ def test_residues_refused_for_a_large_block_only():
     assert items[0] > 0 and items[1] == 0 and items[2] == items[0]
 
 
-# thin blocks of many rows (on the slices), just below and above the lines
+# short sums over many rows
 @pytest.mark.parametrize("n,na,nb,k,transition", [(26, 2, 1, 3, False), (30, 2, 1, 3, True), (27, 1, 1, 2, True),
                                                   (25, 1, 1, 2, False), (40, 2, 0, 2, False), (24, 1, 1, 2, True)])
 def test_density_thin_blocks(n, na, nb, k, transition):
